@@ -41,8 +41,10 @@ def listed():
         # a few maps solved in FP64 together, an odd number of them, at a serving shape
         dict(name="fp64_256x5", kind="batch", precision="fp64", nside=256, lmax=512, nrhs=5, tol=1e-4, max_iter=10000,
              nominal=60),
-        # constrained realisations: 15 draws and the Wiener filter of the data, host arrays in and out
-        dict(name="realisations_256x15", kind="realisations", nside=256, lmax=512, nreal=15, tol=1e-4, nominal=60),
+        # constrained realisations: 7 draws and the Wiener filter of the data, host arrays in and out. In FP64: the
+        # draws pass through a transform before the solves, and the FP32 steps of a mixed solve would turn a change in
+        # that transform's last bit into another rounding everywhere
+        dict(name="realisations_256x7", kind="realisations", nside=256, lmax=512, nreal=7, tol=1e-4, nominal=60),
         # three detectors with their own beams, noise and masks, joint filter
         dict(name="multi_256x3", kind="multi", nside=256, lmax=512, ndet=3, tol=1e-4, nominal=60),
         # temperature and polarisation, cooled joint filter at a serving shape
@@ -81,7 +83,7 @@ def draw(rng):
                     nrhs=rng.randint(2, 40 if ns < 256 else 12), tol=1e-4, max_iter=10000, nominal=60)
     if kind == "realisations":
         ns = 2 ** rng.randint(4, 8)
-        return dict(kind=kind, nside=ns, lmax=_odd_lmax(rng, ns), nreal=rng.randint(1, 15), tol=1e-4, nominal=60)
+        return dict(kind=kind, nside=ns, lmax=_odd_lmax(rng, ns), nreal=rng.randint(1, 7), tol=1e-4, nominal=60)
     if kind == "multi":
         ns = 2 ** rng.randint(3, 8)
         return dict(kind=kind, nside=ns, lmax=_odd_lmax(rng, ns), ndet=rng.randint(2, 5), tol=1e-4, nominal=60)
@@ -289,7 +291,7 @@ def prepare(case, seed):
         s.update(plan=wf.Plan(ns, lmax, q["cl"], _host(q["nv"]), _host(q["mask"]), opts), d=q["d"],
                  out=torch.zeros(case["nrhs"], nalm, dtype=C16, device=DEV))
     elif kind == "realisations":
-        opts = wf.options(precision=wf.WF_PREC_MIXED, tol=case["tol"], batch_slots=case["nreal"] + 1)
+        opts = wf.options(tol=case["tol"])
         s.update(plan=wf.Plan(ns, lmax, q["cl"], _host(q["nv"]), _host(q["mask"]), opts), d=_host(q["d"]), seed=q["seed"])
     elif kind == "multi":
         s.update(plan=wf.Multi(ns, lmax, q["cl"], list(_host(q["nv"])), list(_host(q["mask"])), list(q["beams"]),
