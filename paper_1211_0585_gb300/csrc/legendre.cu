@@ -25,6 +25,7 @@
 //   analysis and the synthesis.
 #include <cuda_runtime.h>
 
+#include "start_values.cuh"
 #include "wf_internal.h"
 
 namespace wfk {
@@ -53,29 +54,31 @@ __device__ __forceinline__ double warp_transpose_sum(double (&v)[32]) {
 }
 
 // Start values: one thread per (m, k). Scaled recurrence with an explicit
-// binary exponent so that sin^m(theta) cannot underflow.
-__global__ void start_values_kernel(const double *xk, const double2 *rec, int lmax, int RP, int *ls_out,
-                                    double2 *sv_out) {
+// binary exponent so that sin^m(theta) cannot underflow. Bound by the FP64
+// pipe: the factors sqrt((2i + 1) / 2i) of lambda_mm are the same for every
+// column, so the CTA forms them once (a division and a square root each), and
+// exponents are compared as integers; with both in every thread's own loop the
+// kernel took 199 us at Nside 64 / lmax 128.
+__global__ void __launch_bounds__(256) start_values_kernel(const double *xk, const double2 *rec, int lmax, int RP,
+                                                           int *ls_out, double2 *sv_out) {
+  extern __shared__ double croot[];   // [m + 1] sqrt((2i + 1) / 2i)
   const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (id >= (long long)(lmax + 1) * RP) return;
+  const long long nid = (long long)(lmax + 1) * RP;
+  lambda_mm_factors(croot, (int)(min(id - threadIdx.x + blockDim.x, nid) - 1) / RP);
+  if (id >= nid) return;
   const int m = (int)(id / RP), k = (int)(id % RP);
   const double x = xk[k];
   const double st = sqrt((1.0 - x) * (1.0 + x));
   int ls = kNoStart;
   double v0 = 0.0, v1 = 0.0;
   if (m == 0 || st > 0.0) {
-    // lambda_mm = (-1)^m sqrt((2m+1)/(4 pi) prod_{i<=m} (2i-1)/(2i)) sin^m(theta), as v * 2^e
-    double v = 0.28209479177387814347;  // 1 / sqrt(4 pi)
     int e = 0;
-    for (int i = 1; i <= m; ++i) {
-      v *= -sqrt((2.0 * i + 1.0) / (2.0 * i)) * st;
-      if (fabs(v) < 0x1p-400) { v *= 0x1p400; e -= 400; }
-    }
+    const double v = lambda_mm_scaled(croot, m, st, e);
     // walk up in l until the true value reaches 2^kStartExp
     double p2 = v;                               // lambda_l (scaled)
     double p1 = x * sqrt(2.0 * m + 3.0) * v;     // lambda_{l+1} (scaled)
     for (int l = m; l <= lmax; ++l) {
-      if (p2 != 0.0 && ilogb(p2) + e >= kStartExp) {
+      if (p2 != 0.0 && exponent_of(p2) + e >= kStartExp) {
         ls = l;
         v0 = ldexp(p2, e);
         v1 = (l + 1 <= lmax) ? ldexp(p1, e) : 0.0;
@@ -86,7 +89,7 @@ __global__ void start_values_kernel(const double *xk, const double2 *rec, int lm
         const double nx = ab.x * x * p1 - ab.y * p2;
         p2 = p1;
         p1 = nx;
-        if (fabs(p2) > 0x1p400 || fabs(p1) > 0x1p400) { p1 *= 0x1p-400; p2 *= 0x1p-400; e += 400; }
+        if (exponent_of(p2) >= 400 || exponent_of(p1) >= 400) { p1 *= 0x1p-400; p2 *= 0x1p-400; e += 400; }
       } else {
         p2 = p1;
         p1 = 0.0;
@@ -184,16 +187,20 @@ __global__ void __launch_bounds__(kThreads) legendre_kernel(const LegArgs A) {
           E[i] = O[i] = make_double2(0.0, 0.0);
         }
       }
+      // ring pairs of this warp in the pass: groups of 32 at k0 + 32 warp + i kThreads. A group past
+      // RP holds zeros and is left out, and a warp of none only joins the barriers
+      const int left = RP - k0 - 32 * warp;
+      const int na = left > kThreads ? 2 : left > 0 ? 1 : 0;
+      const int nw = min((RP - k0 + 31) >> 5, kThreads / 32);   // warps with ring pairs
       for (int l0 = m; l0 <= L; l0 += kLB) {
         double acc[32];
 #pragma unroll
         for (int j = 0; j < 32; ++j) acc[j] = 0.0;
+        auto group = [&](int i) {
 #pragma unroll
-        for (int j = 0; j < kLB; ++j) {
-          const int l = l0 + j;
-          const double2 ab = rc[l - m];
-#pragma unroll
-          for (int i = 0; i < kKPT; ++i) {
+          for (int j = 0; j < kLB; ++j) {
+            const int l = l0 + j;
+            const double2 ab = rc[l - m];
             double lv = fma(ab.x * x[i], p1[i], -ab.y * p2[i]);
             lv = (l == ls[i]) ? v0[i] : lv;
             lv = (l == ls[i] + 1) ? v1[i] : lv;
@@ -203,14 +210,14 @@ __global__ void __launch_bounds__(kThreads) legendre_kernel(const LegArgs A) {
             acc[2 * j] = fma(lv, X.x, acc[2 * j]);
             acc[2 * j + 1] = fma(lv, X.y, acc[2 * j + 1]);
           }
-        }
-        const double v = warp_transpose_sum(acc);
-        red[warp][lane] = v;
+        };
+        if (na > 0) group(0);
+        if (na > 1) group(1);
+        if (na > 0) red[warp][lane] = warp_transpose_sum(acc);
         __syncthreads();
         if (threadIdx.x < 32) {
           double s = 0.0;
-#pragma unroll
-          for (int w = 0; w < kThreads / 32; ++w) s += red[w][threadIdx.x];
+          for (int w = 0; w < nw; ++w) s += red[w][threadIdx.x];
           double *t = reinterpret_cast<double *>(&tl[l0 - m + (threadIdx.x >> 1)]);
           t[threadIdx.x & 1] += s;
         }
@@ -341,7 +348,7 @@ void launch_start_values(const double *x, const double2 *rec, int lmax, int RP, 
                          cudaStream_t s) {
   const long long n = (long long)(lmax + 1) * RP;
   const int blocks = (int)((n + 255) / 256);
-  start_values_kernel<<<blocks, 256, 0, s>>>(x, rec, lmax, RP, ls, sv);
+  start_values_kernel<<<blocks, 256, (size_t)(lmax + 1) * sizeof(double), s>>>(x, rec, lmax, RP, ls, sv);
 }
 
 }  // namespace wfk

@@ -41,6 +41,7 @@
 #include <cuda_runtime.h>
 
 #include "df.cuh"
+#include "start_values.cuh"
 #include "wf_internal.h"
 
 namespace wfk {
@@ -102,25 +103,24 @@ __device__ __forceinline__ void analysis_block(int l0, int m, const float2 *sA, 
 
 // Start values for the double-float recurrence: first l with |lambda| >= 2^-60,
 // and mu at that l and the next (mu = lambda / g), one thread per (m, k).
-__global__ void start_values_df_kernel(const double *xk, const double2 *rec, const double *g, int lmax, int RP,
-                                       int *ls_out, float4 *sv_out) {
+__global__ void __launch_bounds__(256) start_values_df_kernel(const double *xk, const double2 *rec, const double *g,
+                                                              int lmax, int RP, int *ls_out, float4 *sv_out) {
+  extern __shared__ double croot[];   // [m + 1] sqrt((2i + 1) / 2i)
   const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (id >= (long long)(lmax + 1) * RP) return;
+  const long long nid = (long long)(lmax + 1) * RP;
+  lambda_mm_factors(croot, (int)(min(id - threadIdx.x + blockDim.x, nid) - 1) / RP);
+  if (id >= nid) return;
   const int m = (int)(id / RP), k = (int)(id % RP);
   const double x = xk[k];
   const double st = sqrt((1.0 - x) * (1.0 + x));
   int ls = kNoStartD;
   double v0 = 0.0, v1 = 0.0;
   if (m == 0 || st > 0.0) {
-    double v = 0.28209479177387814347;  // 1 / sqrt(4 pi)
     int e = 0;
-    for (int i = 1; i <= m; ++i) {
-      v *= -sqrt((2.0 * i + 1.0) / (2.0 * i)) * st;
-      if (fabs(v) < 0x1p-400) { v *= 0x1p400; e -= 400; }
-    }
+    const double v = lambda_mm_scaled(croot, m, st, e);
     double p2 = v, p1 = x * sqrt(2.0 * m + 3.0) * v;
     for (int l = m; l <= lmax; ++l) {
-      if (p2 != 0.0 && ilogb(p2) + e >= -60) {
+      if (p2 != 0.0 && exponent_of(p2) + e >= -60) {
         ls = l;
         v0 = ldexp(p2, e);
         v1 = (l + 1 <= lmax) ? ldexp(p1, e) : 0.0;
@@ -131,7 +131,7 @@ __global__ void start_values_df_kernel(const double *xk, const double2 *rec, con
         const double nx = ab.x * x * p1 - ab.y * p2;
         p2 = p1;
         p1 = nx;
-        if (fabs(p2) > 0x1p400 || fabs(p1) > 0x1p400) { p1 *= 0x1p-400; p2 *= 0x1p-400; e += 400; }
+        if (exponent_of(p2) >= 400 || exponent_of(p1) >= 400) { p1 *= 0x1p-400; p2 *= 0x1p-400; e += 400; }
       } else {
         p2 = p1;
         p1 = 0.0;
@@ -637,7 +637,7 @@ void launch_df_tables(const double *x, const double2 *rec, int lmax, int RP, dou
                       float4 *sv, cudaStream_t s) {
   rescale_coeffs_kernel<<<lmax + 1, 32, 0, s>>>(rec, lmax, g, A);
   const long long n = (long long)(lmax + 1) * RP;
-  start_values_df_kernel<<<(int)((n + 255) / 256), 256, 0, s>>>(x, rec, g, lmax, RP, ls, sv);
+  start_values_df_kernel<<<(int)((n + 255) / 256), 256, (size_t)(lmax + 1) * sizeof(double), s>>>(x, rec, g, lmax, RP, ls, sv);
 }
 
 }  // namespace wfk

@@ -84,26 +84,41 @@ Layout layout_for(int nside, int lmax) {
   return L;
 }
 
+// Offsets of the tables of length 4c (c = 1 .. nside) among the lengths below
+// it, in closed form: the lengths 4c' with c' a power of two (2^0 .. 2^J, J =
+// floor(log2(c - 1))) need no chirp, and a length with 2^j < c' < 2^(j+1) has a
+// Bluestein size of 2^(j+4).
+struct LenOff { long long hs, ch, B; };
+__device__ __forceinline__ LenOff length_offsets(int c) {
+  LenOff o{2LL * c * (c - 1), 0, 0};
+  if (c < 2) return o;
+  const int J = 31 - __clz(c - 1);
+  o.ch = o.hs - 4LL * ((2LL << J) - 1);
+  for (int j = 0; j < J; ++j) o.B += ((1LL << j) - 1) << (j + 4);
+  o.B += (long long)(c - 1 - (1 << J)) << (J + 4);
+  return o;
+}
+
 // Ring geometry, per-length FFT tables and ring-pair latitudes for one nside,
-// in the layout the ring and Legendre kernels read.
-__global__ void noalloc_geometry_kernel(int nside, int maxM, RingDev *rings, double2 *hs, double2 *chirp,
-                                        double2 *tw, double *x) {
+// in the layout the ring and Legendre kernels read. One CTA per length 4c
+// (its half-shift and chirp tables), its first threads write the two rings of
+// that length (the belt's CTA: all of them), and the CTAs share the twiddles
+// and latitudes. Bound by the sincospi of the FP64 pipe: as one grid that
+// walked the lengths one after another, with the offsets summed ring by ring,
+// this took 282 us at Nside 64, more than the rest of the call's kernels each.
+__global__ void __launch_bounds__(256) noalloc_geometry_kernel(int nside, int maxM, RingDev *rings, double2 *hs,
+                                                               double2 *chirp, double2 *tw, double *x) {
+  const int c = blockIdx.x + 1;
   const int R = 4 * nside - 1;
-  const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  // per-length offsets by prefix sums over lengths 4i, i = 1 .. nside
-  for (long long r = gid; r < R; r += stride) {
-    const int i = (int)r + 1;
+  const long long n = 4LL * c;
+  const bool pow2 = (n & (n - 1)) == 0;
+  const LenOff off = length_offsets(c);
+  // rings of this length: the polar pair c, 4 nside - c; the belt nside .. 3 nside
+  const int nr = c < nside ? 2 : 2 * nside + 1;
+  for (int t = threadIdx.x; t < nr; t += blockDim.x) {
+    const int i = c < nside ? (t ? 4 * nside - c : c) : nside + t;
+    const int r = i - 1;
     const int ip = i < 4 * nside - i ? i : 4 * nside - i;
-    const int cls = ip < nside ? ip : nside;
-    long long hs_off = 0, ch_off = 0, B_off = 0;
-    for (int c = 1; c < cls; ++c) {
-      const long long n = 4LL * c;
-      hs_off += n;
-      if ((n & (n - 1)) != 0) { ch_off += n; B_off += 1LL << ilog2_dev(2 * n - 1); }
-    }
-    const long long n = 4LL * cls;
-    const bool pow2 = (n & (n - 1)) == 0;
     RingDev g{};
     g.n = (int)n;
     const long long npix = 12LL * nside * nside;
@@ -111,33 +126,27 @@ __global__ void noalloc_geometry_kernel(int nside, int maxM, RingDev *rings, dou
     else if (i <= 3 * nside) g.off = 2LL * nside * (nside - 1) + (long long)(i - nside) * 4 * nside;
     else g.off = npix - 2LL * ip * (ip + 1);
     g.shifted = ip < nside ? 1 : (((i - nside) % 2) == 0 ? 1 : 0);
-    g.pair = (int)(r < R - 1 - r ? r : R - 1 - r);
+    g.pair = r < R - 1 - r ? r : R - 1 - r;
     g.side = r > R - 1 - r ? 1 : 0;
     g.logM = pow2 ? ilog2_dev(n) : ilog2_dev(2 * n - 1);
     g.blue = pow2 ? 0 : 1;
-    g.hs_off = hs_off;
-    g.ch_off = pow2 ? 0 : ch_off;
-    g.B_off = pow2 ? 0 : B_off;
+    g.hs_off = off.hs;
+    g.ch_off = pow2 ? 0 : off.ch;
+    g.B_off = pow2 ? 0 : off.B;
     rings[r] = g;
   }
-  // half-shift and chirp tables, length by length
-  long long hs_off = 0, ch_off = 0;
-  for (int c = 1; c <= nside; ++c) {
-    const long long n = 4LL * c;
-    const bool pow2 = (n & (n - 1)) == 0;
-    for (long long q = gid; q < n; q += stride) {
-      double s, co;
-      sincospi((double)q / (double)n, &s, &co);
-      hs[hs_off + q] = make_double2(co, s);
-      if (!pow2) {
-        const long long jj = (q * q) % (2 * n);
-        sincospi((double)jj / (double)n, &s, &co);
-        chirp[ch_off + q] = make_double2(co, -s);
-      }
+  for (long long q = threadIdx.x; q < n; q += blockDim.x) {
+    double s, co;
+    sincospi((double)q / (double)n, &s, &co);
+    hs[off.hs + q] = make_double2(co, s);
+    if (!pow2) {
+      const long long jj = (q * q) % (2 * n);
+      sincospi((double)jj / (double)n, &s, &co);
+      chirp[off.ch + q] = make_double2(co, -s);
     }
-    hs_off += n;
-    if (!pow2) ch_off += n;
   }
+  const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long k = gid; k < maxM; k += stride) {
     double s, co;
     sincospi(2.0 * (double)k / (double)maxM, &s, &co);
@@ -216,7 +225,7 @@ extern "C" wf_status wf_map2alm_noalloc(int nside, int lmax, const double *map_d
   // the ring stage never writes the equator pair's south slot: it must read as zero
   e = cudaMemsetAsync(FT, 0, sizeof(double4_32a) * (size_t)(lmax + 1) * RP, s);
   if (e != cudaSuccess) return cuda_status(e, "cudaMemsetAsync");
-  noalloc_geometry_kernel<<<64, 256, 0, s>>>(nside, L.maxM, rings, hs, chirp, tw, x);
+  noalloc_geometry_kernel<<<nside, 256, 0, s>>>(nside, L.maxM, rings, hs, chirp, tw, x);
   noalloc_rec_kernel<<<lmax + 1, 128, 0, s>>>(lmax, rec);
   const RingClass all{ilog2_up(L.maxM), 0, R, 0};   // one launch over every ring, in ring order
   if (L.B_n > 0) launch_bluestein_setup(rings, nullptr, &all, 1, nullptr, tw, ilog2_up(L.maxM), chirp, B, s);
