@@ -189,7 +189,7 @@ __device__ __forceinline__ dfl dneg(dfl a) { return dfl{-a.h, -a.l}; }
 // spin-2 analysis in double-float: one CTA per m, a warp per l, lanes over
 // ring pairs. Shared memory holds, per ring pair, Q_N + Q_S, Q_N - Q_S, U_N + U_S,
 // U_N - U_S (the two parities' combinations of the rings' coefficients).
-__global__ void __launch_bounds__(kPolThreads) spin2_analysis_df_kernel(const Ctl *gate, const float4 *tab,
+__global__ void __launch_bounds__(kPolThreads, 3) spin2_analysis_df_kernel(const Ctl *gate, const float4 *tab,
                                                                          const int *ls, const double4_32a *FTQ,
                                                                          const double4_32a *FTU, int lmax, int RP,
                                                                          double2 *aE, double2 *aB) {
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(kPolThreads) spin2_analysis_df_kernel(const Ct
 // F+ B.im, F- E.re are summed separately over even (S0) and odd (S1) l - m;
 // the north ring takes even + odd, the south ring (parity (-1)^(l-m) for F+,
 // the opposite for F-) even - odd.
-__global__ void __launch_bounds__(kPolThreads) spin2_synthesis_df_kernel(const Ctl *gate, const float4 *tab,
+__global__ void __launch_bounds__(kPolThreads, 3) spin2_synthesis_df_kernel(const Ctl *gate, const float4 *tab,
                                                                           const int *ls, const double2 *aE,
                                                                           const double2 *aB, int lmax, int RP,
                                                                           double4_32a *FSQ, double4_32a *FSU) {
