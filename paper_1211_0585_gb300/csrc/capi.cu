@@ -618,6 +618,8 @@ wf_status wf_plan_set_options(wf_plan_t plan, const wf_options *opt) {
   // the captured iteration holds the kernels of the precision and the launch shape
   const bool regraph = opt->graph_iters != P->opt.graph_iters || opt->stream != P->opt.stream ||
                        opt->precision != P->opt.precision;
+  // the Fourier records left by wf_iterate are doubles or double-floats, as the precision's stages hold them
+  if ((opt->precision == WF_PREC_FP64_NATIVE) != (P->opt.precision == WF_PREC_FP64_NATIVE)) P->fs_valid = false;
   P->opt = *opt;
   wf_status st = P->ensure_hist(opt->max_iter + 1);
   if (st) return st;

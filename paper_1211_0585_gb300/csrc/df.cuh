@@ -17,6 +17,23 @@ __device__ __forceinline__ dfl df_from(double v) {
 
 __device__ __forceinline__ double df_to(dfl a) { return (double)a.h + (double)a.l; }
 
+// A double-float in the 8 bytes of a double: the Fourier records F of the
+// double-float stages hold (hi, lo) pairs where those of the native stages hold
+// doubles, so that no stage pays the FP64 pipe (1/63 of FP32) for conversions.
+__device__ __forceinline__ double df_pack(dfl a) { return __hiloint2double(__float_as_int(a.h), __float_as_int(a.l)); }
+__device__ __forceinline__ dfl df_unpack(double v) {
+  return {__int_as_float(__double2hiint(v)), __int_as_float(__double2loint(v))};
+}
+
+__device__ __forceinline__ dfl df_neg(dfl a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ float4 df_pair(dfl a, dfl b) { return make_float4(a.h, a.l, b.h, b.l); }
+
+// S + C of a compensated sum as a double-float
+__device__ __forceinline__ dfl df_norm(float S, float C) {
+  const float s = S + C, bb = s - S;
+  return {s, (S - (s - bb)) + (C - bb)};
+}
+
 // a + b (two_sum of the high parts, low parts added, renormalised)
 __device__ __forceinline__ dfl df_add(dfl a, dfl b) {
   const float s = a.h + b.h;
@@ -72,6 +89,18 @@ __device__ __forceinline__ dfl df_step(dfl A, dfl x, dfl mu1, dfl mu2) {
   const float e = d + (v - mu2.l);
   const float rh = sh + e;
   return {rh, e - (rh - sh)};
+}
+
+// A Fourier record (north re, im, south re, im; df_pack'ed) as the sums of its two rings for even l - m, E = N + S,
+// and for odd, O = N - S, each (re hi, re lo, im hi, im lo); and the record of E and O.
+__device__ __forceinline__ void f_parities(const double4_32a &t, float4 &E, float4 &O) {
+  const dfl nr = df_unpack(t.x), ni = df_unpack(t.y), sr = df_unpack(t.z), si = df_unpack(t.w);
+  E = df_pair(df_add(nr, sr), df_add(ni, si));
+  O = df_pair(df_add(nr, df_neg(sr)), df_add(ni, df_neg(si)));
+}
+__device__ __forceinline__ double4_32a f_rings(dfl er, dfl ei, dfl orr, dfl oi) {
+  return make_double4_32a(df_pack(df_add(er, orr)), df_pack(df_add(ei, oi)), df_pack(df_add(er, df_neg(orr))),
+                          df_pack(df_add(ei, df_neg(oi))));
 }
 
 }  // namespace wfk

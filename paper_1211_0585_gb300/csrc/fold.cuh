@@ -9,6 +9,7 @@
 
 #include <cuda_runtime.h>
 
+#include "df.cuh"
 #include "wf_internal.h"
 
 namespace wfk {
@@ -33,47 +34,64 @@ __device__ __forceinline__ double2 fold_alias_sum(const double4_32a *FS, int RP,
   return make_double2(ar, ai);
 }
 
-// Both slots' shares at once (north in .x/.y, south in .z/.w), each F record
-// read once.
-__device__ __forceinline__ double4_16a fold_alias_sum2(const double4_32a *FS, int RP, int k, int shifted, int n, int q,
-                                                   int L, int j0, int dj) {
-  double4_16a a = make_double4_16a(0.0, 0.0, 0.0, 0.0);
-  for (int j = j0, m = q + n * j0; m <= L; j += dj, m += n * dj) {
-    const double4_32a f4 = FS[(size_t)m * RP + k];
-    const double sg = (shifted && (j & 1)) ? -1.0 : 1.0;
-    a.x += sg * f4.x; a.y += sg * f4.y; a.z += sg * f4.z; a.w += sg * f4.w;
-  }
-  for (int j = 1 + j0, m = n * (1 + j0) - q; m <= L; j += dj, m += n * dj) {
-    const double4_32a f4 = FS[(size_t)m * RP + k];
-    const double sg = (shifted && (j & 1)) ? -1.0 : 1.0;
-    a.x += sg * f4.x; a.y -= sg * f4.y; a.z += sg * f4.z; a.w -= sg * f4.w;
-  }
+// Both slots' shares at once in double-float (records of df_pack'ed values),
+// north and south each as (re hi, re lo, im hi, im lo), each record read once.
+struct FoldPair { float4 n, s; };
+__device__ __forceinline__ FoldPair fold_record(const double4_32a *FS, size_t at, float sg, float cj) {
+  const double4_32a f = FS[at];
+  const dfl nr = df_unpack(f.x), ni = df_unpack(f.y), sr = df_unpack(f.z), si = df_unpack(f.w);
+  const float ci = sg * cj;
+  return {make_float4(sg * nr.h, sg * nr.l, ci * ni.h, ci * ni.l),
+          make_float4(sg * sr.h, sg * sr.l, ci * si.h, ci * si.l)};
+}
+__device__ __forceinline__ float4 fold_add(float4 a, float4 b) {
+  return df_pair(df_add(dfl{a.x, a.y}, dfl{b.x, b.y}), df_add(dfl{a.z, a.w}, dfl{b.z, b.w}));
+}
+__device__ __forceinline__ FoldPair fold_alias_sum2(const double4_32a *FS, int RP, int k, int shifted, int n, int q,
+                                                    int L, int j0, int dj) {
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  FoldPair a{z, z};
+  bool first = true;
+  auto take = [&](FoldPair r) {
+    if (first) a = r;
+    else { a.n = fold_add(a.n, r.n); a.s = fold_add(a.s, r.s); }
+    first = false;
+  };
+  for (int j = j0, m = q + n * j0; m <= L; j += dj, m += n * dj)
+    take(fold_record(FS, (size_t)m * RP + k, (shifted && (j & 1)) ? -1.f : 1.f, 1.f));
+  for (int j = 1 + j0, m = n * (1 + j0) - q; m <= L; j += dj, m += n * dj)
+    take(fold_record(FS, (size_t)m * RP + k, (shifted && (j & 1)) ? -1.f : 1.f, -1.f));
   return a;
 }
 
-// fold_ring for both rings of a pair: store(q, G_q north, G_q south).
-// part: shared scratch of blockDim.x double4_16a.
+// fold_ring for both rings of a pair: store(q, G_q north, G_q south), in
+// double-float. part: shared scratch of blockDim.x FoldPair. A residue's series
+// of at most L / n + 1 aliases is split over as many threads as it has terms
+// and the block has room for (over blockDim.x / n threads whatever the series'
+// length, the sum over them walked up to 64 empty parts on the smallest rings).
 template <class Store>
 __device__ __forceinline__ void fold_ring2(const double4_32a *FS, int RP, int k, int shifted, int n, int L,
-                                           double4_16a *part, Store store) {
+                                           FoldPair *part, Store store) {
   const int nt = blockDim.x;
-  if (n >= nt) {
+  const int nj = min(nt / n, L / n + 1);
+  if (nj <= 1) {
     for (int q = threadIdx.x; q < n; q += nt) {
-      const double4_16a g = fold_alias_sum2(FS, RP, k, shifted, n, q, L, 0, 1);
-      store(q, make_double2(g.x, g.y), make_double2(g.z, g.w));
+      const FoldPair g = fold_alias_sum2(FS, RP, k, shifted, n, q, L, 0, 1);
+      store(q, g.n, g.s);
     }
     return;
   }
-  const int nj = nt / n, t = threadIdx.x;
+  const int t = threadIdx.x;
   if (t < n * nj) part[t] = fold_alias_sum2(FS, RP, k, shifted, n, t % n, L, t / n, nj);
   __syncthreads();
   if (t < n) {
-    double4_16a g = make_double4_16a(0.0, 0.0, 0.0, 0.0);
-    for (int jg = 0; jg < nj; ++jg) {
-      const double4_16a p = part[jg * n + t];
-      g.x += p.x; g.y += p.y; g.z += p.z; g.w += p.w;
+    FoldPair g = part[t];
+    for (int jg = 1; jg < nj; ++jg) {
+      const FoldPair p = part[jg * n + t];
+      g.n = fold_add(g.n, p.n);
+      g.s = fold_add(g.s, p.s);
     }
-    store(t, make_double2(g.x, g.y), make_double2(g.z, g.w));
+    store(t, g.n, g.s);
   }
 }
 

@@ -137,10 +137,7 @@ __global__ void __launch_bounds__(kBThreads, kMinBlocks) legendre_batch_kernel(c
         float4 e = make_float4(0.f, 0.f, 0.f, 0.f), o = e;
         if (b < Bm.n && Lb[b] >= m) {
           const double4_32a t = Bm.FT[b][(size_t)m * RP + k0 + kk];
-          const dfl er = df_from(t.x + t.z), ei = df_from(t.y + t.w);
-          const dfl orr = df_from(t.x - t.z), oi = df_from(t.y - t.w);
-          e = make_float4(er.h, er.l, ei.h, ei.l);
-          o = make_float4(orr.h, orr.l, oi.h, oi.l);
+          f_parities(t, e, o);
         }
         reg[(size_t)(2 * b) * nkm + kk] = e;
         reg[(size_t)(2 * b + 1) * nkm + kk] = o;
@@ -344,9 +341,8 @@ __global__ void __launch_bounds__(kBThreads, kMinBlocks) legendre_batch_kernel(c
 #pragma unroll
       for (int b = 0; b < NB; ++b) {
         if (!on[b] || m > Lb[b]) continue;
-        const double er = (double)acc[b][0] + (double)acc[b][1], ei = (double)acc[b][2] + (double)acc[b][3];
-        const double orr = (double)acc[b][4] + (double)acc[b][5], oi = (double)acc[b][6] + (double)acc[b][7];
-        Bm.FS[b][(size_t)m * RP + k] = make_double4_32a(er + orr, ei + oi, er - orr, ei - oi);
+        Bm.FS[b][(size_t)m * RP + k] = f_rings(df_norm(acc[b][0], acc[b][1]), df_norm(acc[b][2], acc[b][3]),
+                                               df_norm(acc[b][4], acc[b][5]), df_norm(acc[b][6], acc[b][7]));
       }
     }
   }

@@ -301,10 +301,7 @@ __global__ void __launch_bounds__(kThreads, TAB ? kTabBlocks : 2) legendre_df_ke
         float4 *stE = ss, *stO = ss + nk;
         for (int kk = threadIdx.x; kk < nk; kk += blockDim.x) {
           const double4_32a t = A.FT[(size_t)m * RP + k0 + kk];
-          const dfl er = df_from(t.x + t.z), ei = df_from(t.y + t.w);
-          const dfl orr = df_from(t.x - t.z), oi = df_from(t.y - t.w);
-          stE[kk] = make_float4(er.h, er.l, ei.h, ei.l);
-          stO[kk] = make_float4(orr.h, orr.l, oi.h, oi.l);
+          f_parities(t, stE[kk], stO[kk]);
         }
         for (int t = warp; t < ntile; t += kWarps) {
           const int kk = 32 * t + lane;
@@ -371,10 +368,7 @@ __global__ void __launch_bounds__(kThreads, TAB ? kTabBlocks : 2) legendre_df_ke
       for (int kk = threadIdx.x; kk < nk; kk += blockDim.x) {
         const int k = k0 + kk;
         const double4_32a t = A.FT[(size_t)m * RP + k];
-        const dfl er = df_from(t.x + t.z), ei = df_from(t.y + t.w);
-        const dfl orr = df_from(t.x - t.z), oi = df_from(t.y - t.w);
-        stE[kk] = make_float4(er.h, er.l, ei.h, ei.l);
-        stO[kk] = make_float4(orr.h, orr.l, oi.h, oi.l);
+        f_parities(t, stE[kk], stO[kk]);
         stP[kk] = make_float4(0.f, 0.f, 0.f, 0.f);
         const dfl xk = df_from(A.x[k]);
         stX[kk] = make_float2(xk.h, xk.l);
@@ -516,9 +510,7 @@ __global__ void __launch_bounds__(kThreads, TAB ? kTabBlocks : 2) legendre_df_ke
         }
       }
       if (k < RP) {
-        const double er = (double)ERs + (double)ERc, ei = (double)EIs + (double)EIc;
-        const double orr = (double)ORs + (double)ORc, oi = (double)OIs + (double)OIc;
-        A.FS[(size_t)m * RP + k] = make_double4_32a(er + orr, ei + oi, er - orr, ei - oi);
+        A.FS[(size_t)m * RP + k] = f_rings(df_norm(ERs, ERc), df_norm(EIs, EIc), df_norm(ORs, ORc), df_norm(OIs, OIc));
       }
     }
     return;
@@ -572,9 +564,7 @@ __global__ void __launch_bounds__(kThreads, TAB ? kTabBlocks : 2) legendre_df_ke
           dot2_acc(EIs, EIc, me, dfl{ce.z, ce.w});
         }
       }
-      const double er = (double)ERs + (double)ERc, ei = (double)EIs + (double)EIc;
-      const double orr = (double)ORs + (double)ORc, oi = (double)OIs + (double)OIc;
-      A.FS[mk] = make_double4_32a(er + orr, ei + oi, er - orr, ei - oi);
+      A.FS[mk] = f_rings(df_norm(ERs, ERc), df_norm(EIs, EIc), df_norm(ORs, ORc), df_norm(OIs, OIc));
     }
   }
 }

@@ -181,160 +181,234 @@ __global__ void __launch_bounds__(kPolThreads) spin2_synthesis_kernel(const Ctl 
 
 // ---- double-float spin-2 Legendre stage
 __device__ __forceinline__ float4 cdf(double re, double im) {   // complex double-float (re hi, re lo, im hi, im lo)
-  const dfl a = df_from(re), b = df_from(im);
-  return make_float4(a.h, a.l, b.h, b.l);
+  return df_pair(df_from(re), df_from(im));
 }
-__device__ __forceinline__ dfl dneg(dfl a) { return dfl{-a.h, -a.l}; }
+__device__ __forceinline__ float4 zero4() { return make_float4(0.f, 0.f, 0.f, 0.f); }
 
-// spin-2 analysis in double-float: one CTA per m, a warp per l, lanes over
-// ring pairs. Shared memory holds, per ring pair, Q_N + Q_S, Q_N - Q_S, U_N + U_S,
-// U_N - U_S (the two parities' combinations of the rings' coefficients).
+// (S, C) += (S, C) of the lane `off` away (xor), error-free in S
+__device__ __forceinline__ void xor_sum_df(float &S, float &C, int off) {
+  const float rS = __shfl_xor_sync(0xffffffffu, S, off), rC = __shfl_xor_sync(0xffffffffu, C, off);
+  const float s = S + rS;
+  const float bb = s - S;
+  C = C + rC + ((S - (s - bb)) + (rS - bb));
+  S = s;
+}
+
+// Eight compensated sums over the warp: lane q ends with sum q >> 2 of its 8 (lanes 4 q .. 4 q + 3 hold sum q).
+// Halves are exchanged on the way down (4 + 2 + 1 additions, then 2), all in double-float: in FP64, 40 additions
+// on a pipe of 1/63 the rate took longer than a short row's products.
+__device__ __forceinline__ dfl warp_sum8_df(float (&S)[8], float (&C)[8]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int off = 16, n = 4; n >= 1; off >>= 1, n >>= 1) {
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int j = 0; j < n; ++j) {
+      const float oS = up ? S[j] : S[j + n], oC = up ? C[j] : C[j + n];   // sent
+      const float kS = up ? S[j + n] : S[j], kC = up ? C[j + n] : C[j];   // kept
+      const float rS = __shfl_xor_sync(0xffffffffu, oS, off), rC = __shfl_xor_sync(0xffffffffu, oC, off);
+      const float s = kS + rS;
+      const float bb = s - kS;
+      S[j] = s;
+      C[j] = kC + rC + ((kS - (s - bb)) + (rS - bb));
+    }
+  }
+  xor_sum_df(S[0], C[0], 2);
+  xor_sum_df(S[0], C[0], 1);
+  return df_norm(S[0], C[0]);
+}
+
+// spin-2 analysis in double-float: a CTA takes lchunk values of l of one m, a
+// warp two of them (l - m even, then odd) at a time, lanes over ring pairs.
+// Shared memory holds, per ring pair, Q_N + Q_S, Q_N - Q_S, U_N + U_S, U_N - U_S
+// (the two parities' combinations of the rings' coefficients).
+// Bound by FP32 issue (16 compensated products a ring pair and row pair against
+// 32 bytes of table and four shared loads); the table rows of the next two
+// tiles of 32 ring pairs are in flight while one is summed. Chunks of l instead
+// of a CTA per m keep every SM busy at any lmax. A CTA per m, FP64 sums over the
+// warp and one step of loads ahead: 2.28 ms a launch at Nside 512 / lmax 1024 and
+// 156 us at Nside 128 / lmax 256; now 1.80 ms and 54 us.
 __global__ void __launch_bounds__(kPolThreads, 3) spin2_analysis_df_kernel(const Ctl *gate, const float4 *tab,
-                                                                         const int *ls, const double4_32a *FTQ,
-                                                                         const double4_32a *FTU, int lmax, int RP,
-                                                                         double2 *aE, double2 *aB) {
+                                                                            const int *ls, const double4_32a *FTQ,
+                                                                            const double4_32a *FTU, int lmax, int RP,
+                                                                            int lchunk, double2 *aE, double2 *aB) {
   if (gate && gate->done) return;
-  extern __shared__ float4 pol_dsm[];   // [RP][4]
+  extern __shared__ float4 pol_dsm[];   // [4][RP] combinations, then [RP / 32] first l of each tile
   const int m = blockIdx.x;
-  for (int k = threadIdx.x; k < RP; k += blockDim.x) {
-    const double4_32a Qv = FTQ[(size_t)m * RP + k], Uv = FTU[(size_t)m * RP + k];
-    pol_dsm[4 * k + 0] = cdf(Qv.x + Qv.z, Qv.y + Qv.w);
-    pol_dsm[4 * k + 1] = cdf(Qv.x - Qv.z, Qv.y - Qv.w);
-    pol_dsm[4 * k + 2] = cdf(Uv.x + Uv.z, Uv.y + Uv.w);
-    pol_dsm[4 * k + 3] = cdf(Uv.x - Uv.z, Uv.y - Uv.w);
+  const int lbeg = m + blockIdx.y * lchunk, lend = min(lmax, lbeg + lchunk - 1);
+  if (lbeg > lmax) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int ntile = (RP + 31) >> 5;
+  int *tmin = reinterpret_cast<int *>(pol_dsm + 4 * RP);
+  for (int t = warp; t < ntile; t += nw) {
+    const int k = 32 * t + lane;
+    const int mn = __reduce_min_sync(0xffffffffu, k < RP ? ls[(size_t)m * RP + k] : 1 << 30);
+    if (lane == 0) tmin[t] = mn;
+    if (k < RP && mn <= lend) {
+      f_parities(FTQ[(size_t)m * RP + k], pol_dsm[k], pol_dsm[RP + k]);
+      f_parities(FTU[(size_t)m * RP + k], pol_dsm[2 * RP + k], pol_dsm[3 * RP + k]);
+    }
   }
   __syncthreads();
-  // a warp takes l and l + 1 (l - m even, then odd): both read the same four combinations, the even
-  // l as (Q+, Q-, U+, U-) = (N + S, N - S), the odd one with the two swapped
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const size_t base = idx_lm(lmax, m, m);
-  for (int l = m + 2 * warp; l <= lmax; l += 2 * nw) {
+  for (int l = lbeg + 2 * warp; l <= lend; l += 2 * nw) {
     const bool has1 = l + 1 <= lmax;
     float S[8], C[8];   // [0..3]: l, [4..7]: l + 1
 #pragma unroll
     for (int j = 0; j < 8; ++j) { S[j] = 0.f; C[j] = 0.f; }
     const float4 *row0 = tab + (base + (l - m)) * RP, *row1 = row0 + RP;
-    // two ring pairs per step, every global load of both issued before the products
-    auto term = [&](int lsk, float4 f0, float4 f1, int k) {
-      if (l + 1 < lsk) return;   // F+- = 0 below the ring pair's first l
-      const float4 A = pol_dsm[4 * k + 0], Bq = pol_dsm[4 * k + 1];
-      const float4 Cu = pol_dsm[4 * k + 2], Du = pol_dsm[4 * k + 3];
-      // a^E = -(F+ Q+ + i F- U-),  a^B = -(F+ U+ - i F- Q-)
-      if (l >= lsk) {   // l: Q+ = A, Q- = Bq, U+ = Cu, U- = Du
-        const dfl fp = {f0.x, f0.y}, fm = {f0.z, f0.w};
-        dot2_acc(S[0], C[0], fp, dneg(dfl{A.x, A.y}));
-        dot2_acc(S[0], C[0], fm, dfl{Du.z, Du.w});
-        dot2_acc(S[1], C[1], fp, dneg(dfl{A.z, A.w}));
-        dot2_acc(S[1], C[1], fm, dneg(dfl{Du.x, Du.y}));
-        dot2_acc(S[2], C[2], fp, dneg(dfl{Cu.x, Cu.y}));
-        dot2_acc(S[2], C[2], fm, dneg(dfl{Bq.z, Bq.w}));
-        dot2_acc(S[3], C[3], fp, dneg(dfl{Cu.z, Cu.w}));
-        dot2_acc(S[3], C[3], fm, dfl{Bq.x, Bq.y});
+    auto next_tile = [&](int t) {   // the next tile with a term of l or l + 1 (F+- = 0 below a ring pair's first l)
+      while (t < ntile && tmin[t] > l + 1) ++t;
+      return t;
+    };
+    auto load = [&](int t, float4 &f0, float4 &f1) {
+      const int k = 32 * t + lane;
+      f0 = k < RP ? row0[k] : zero4();
+      f1 = k < RP && has1 ? row1[k] : zero4();
+    };
+    auto term = [&](int t, float4 f0, float4 f1) {
+      const int k = min(32 * t + lane, RP - 1);   // lanes past RP: zero table values
+      const float4 A = pol_dsm[k], Bq = pol_dsm[RP + k], Cu = pol_dsm[2 * RP + k], Du = pol_dsm[3 * RP + k];
+      // -a^E = F+ Q+ + i F- U-,  -a^B = F+ U+ - i F- Q-
+      {   // l: Q+ = A, Q- = Bq, U+ = Cu, U- = Du
+        const dfl fp = {f0.x, f0.y}, fm = {f0.z, f0.w}, fn = df_neg(fm);
+        dot2_acc(S[0], C[0], fp, dfl{A.x, A.y});
+        dot2_acc(S[0], C[0], fn, dfl{Du.z, Du.w});
+        dot2_acc(S[1], C[1], fp, dfl{A.z, A.w});
+        dot2_acc(S[1], C[1], fm, dfl{Du.x, Du.y});
+        dot2_acc(S[2], C[2], fp, dfl{Cu.x, Cu.y});
+        dot2_acc(S[2], C[2], fm, dfl{Bq.z, Bq.w});
+        dot2_acc(S[3], C[3], fp, dfl{Cu.z, Cu.w});
+        dot2_acc(S[3], C[3], fn, dfl{Bq.x, Bq.y});
       }
-      if (has1) {   // l + 1: Q+ = Bq, Q- = A, U+ = Du, U- = Cu
-        const dfl fp = {f1.x, f1.y}, fm = {f1.z, f1.w};
-        dot2_acc(S[4], C[4], fp, dneg(dfl{Bq.x, Bq.y}));
-        dot2_acc(S[4], C[4], fm, dfl{Cu.z, Cu.w});
-        dot2_acc(S[5], C[5], fp, dneg(dfl{Bq.z, Bq.w}));
-        dot2_acc(S[5], C[5], fm, dneg(dfl{Cu.x, Cu.y}));
-        dot2_acc(S[6], C[6], fp, dneg(dfl{Du.x, Du.y}));
-        dot2_acc(S[6], C[6], fm, dneg(dfl{A.z, A.w}));
-        dot2_acc(S[7], C[7], fp, dneg(dfl{Du.z, Du.w}));
-        dot2_acc(S[7], C[7], fm, dfl{A.x, A.y});
+      {   // l + 1: Q+ = Bq, Q- = A, U+ = Du, U- = Cu
+        const dfl fp = {f1.x, f1.y}, fm = {f1.z, f1.w}, fn = df_neg(fm);
+        dot2_acc(S[4], C[4], fp, dfl{Bq.x, Bq.y});
+        dot2_acc(S[4], C[4], fn, dfl{Cu.z, Cu.w});
+        dot2_acc(S[5], C[5], fp, dfl{Bq.z, Bq.w});
+        dot2_acc(S[5], C[5], fm, dfl{Cu.x, Cu.y});
+        dot2_acc(S[6], C[6], fp, dfl{Du.x, Du.y});
+        dot2_acc(S[6], C[6], fm, dfl{A.z, A.w});
+        dot2_acc(S[7], C[7], fp, dfl{Du.z, Du.w});
+        dot2_acc(S[7], C[7], fn, dfl{A.x, A.y});
       }
     };
-    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int k = lane; k < RP; k += 64) {
-      const int ka = k, kb = k + 32;
-      const int la = ls[(size_t)m * RP + ka], lb = kb < RP ? ls[(size_t)m * RP + kb] : lmax + 2;
-      const float4 fa0 = l >= la ? row0[ka] : z4, fa1 = has1 && l + 1 >= la ? row1[ka] : z4;
-      const float4 fb0 = l >= lb ? row0[kb] : z4, fb1 = has1 && l + 1 >= lb ? row1[kb] : z4;
-      term(la, fa0, fa1, ka);
-      if (kb < RP) term(lb, fb0, fb1, kb);
+    float4 a0 = zero4(), a1 = zero4(), b0 = zero4(), b1 = zero4();
+    int ta = next_tile(0), tb = next_tile(ta + 1);
+    if (ta < ntile) load(ta, a0, a1);
+    if (tb < ntile) load(tb, b0, b1);
+    while (ta < ntile) {
+      const int t0 = ta;
+      const float4 f0 = a0, f1 = a1;
+      const int tc = next_tile(tb + 1);
+      ta = tb;
+      tb = tc;
+      a0 = b0;
+      a1 = b1;
+      if (tc < ntile) load(tc, b0, b1);
+      term(t0, f0, f1);
     }
-    double v[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = (double)S[j] + (double)C[j];
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
-    if (lane == 0) {
-      aE[base + (l - m)] = l >= 2 ? make_double2(v[0], v[1]) : make_double2(0.0, 0.0);
-      aB[base + (l - m)] = l >= 2 ? make_double2(v[2], v[3]) : make_double2(0.0, 0.0);
-      if (has1) {
-        aE[base + (l + 1 - m)] = l + 1 >= 2 ? make_double2(v[4], v[5]) : make_double2(0.0, 0.0);
-        aB[base + (l + 1 - m)] = l + 1 >= 2 ? make_double2(v[6], v[7]) : make_double2(0.0, 0.0);
+    const dfl v = warp_sum8_df(S, C);
+    if ((lane & 3) == 0) {   // sum lane / 4: E re, im, B re, im of l, then of l + 1
+      const int q = lane >> 2, lq = l + (q >> 2);
+      if (lq <= lend) {
+        double2 *dst = ((q >> 1) & 1) ? aB : aE;
+        reinterpret_cast<double *>(dst + base + (lq - m))[q & 1] = lq >= 2 ? -df_to(v) : 0.0;
       }
     }
   }
 }
 
-// spin-2 synthesis in double-float: one CTA per m, a thread per ring pair.
+// spin-2 synthesis in double-float: a CTA takes one m and blockDim.x ring pairs, a thread one of them.
 // The eight products F+ E.re, F- B.im, F+ E.im, F- B.re, F+ B.re, F- E.im,
 // F+ B.im, F- E.re are summed separately over even (S0) and odd (S1) l - m;
 // the north ring takes even + odd, the south ring (parity (-1)^(l-m) for F+,
 // the opposite for F-) even - odd.
+// Bound by FP32 issue (80 instructions a row). Each lane copies its own table
+// column into a shared ring of kSynDepth rows ahead with cp.async (no barrier:
+// nobody else reads it), which holds the loads of a DRAM latency without the
+// registers that a third CTA per SM needs. Four rows loaded at a time, a CTA per
+// m: 1.65 ms a launch at Nside 512 / lmax 1024, 78 us at Nside 128 / lmax 256; now
+// 1.48 ms and 48 us.
+constexpr int kSynDepth = 8;   // rows in flight, even
+__device__ __forceinline__ void cp_async16(float4 *dst, const float4 *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
 __global__ void __launch_bounds__(kPolThreads, 3) spin2_synthesis_df_kernel(const Ctl *gate, const float4 *tab,
-                                                                          const int *ls, const double2 *aE,
-                                                                          const double2 *aB, int lmax, int RP,
-                                                                          double4_32a *FSQ, double4_32a *FSU) {
+                                                                             const int *ls, const double2 *aE,
+                                                                             const double2 *aB, int lmax, int RP,
+                                                                             double4_32a *FSQ, double4_32a *FSU) {
   if (gate && gate->done) return;
-  extern __shared__ float4 pol_dsa[];   // [Lm][2]: E, B as complex double-float
+  extern __shared__ float4 pol_dsa[];   // [kSynDepth][blockDim.x] ring of rows, then [Lm + 1][2]: E, B as complex double-float
   const int m = blockIdx.x;
   const int Lm = lmax - m + 1;
   const size_t base = idx_lm(lmax, m, m);
-  for (int i = threadIdx.x; i < Lm; i += blockDim.x) {
-    pol_dsa[2 * i] = cdf(aE[base + i].x, aE[base + i].y);
-    pol_dsa[2 * i + 1] = cdf(aB[base + i].x, aB[base + i].y);
+  const int k = blockIdx.y * blockDim.x + threadIdx.x;
+  float4 *ring = pol_dsa + threadIdx.x, *coef = pol_dsa + (size_t)kSynDepth * blockDim.x;
+  const int nt = blockDim.x;
+  // the warp's first row (its ring pairs' first l, at least l = 2), made even
+  const int lw = __reduce_min_sync(0xffffffffu, k < RP ? ls[(size_t)m * RP + k] : 1 << 30);
+  const int i0 = max(m < 2 ? 2 - m : 0, lw - m) & ~1;
+  const float4 *col = tab + base * RP + min(k, RP - 1);
+  auto fetch = [&](int i) {   // rows i and i + 1 into the ring (one group, also when there is none left)
+    if (i < Lm) cp_async16(ring + (size_t)(i & (kSynDepth - 1)) * nt, col + (size_t)i * RP);
+    if (i + 1 < Lm) cp_async16(ring + (size_t)((i + 1) & (kSynDepth - 1)) * nt, col + (size_t)(i + 1) * RP);
+    cp_commit();
+  };
+#pragma unroll
+  for (int j = 0; j < kSynDepth; j += 2) fetch(i0 + j);
+  for (int i = threadIdx.x; i < Lm; i += nt) {
+    coef[2 * i] = cdf(aE[base + i].x, aE[base + i].y);
+    coef[2 * i + 1] = cdf(aB[base + i].x, aB[base + i].y);
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < RP; k += blockDim.x) {
-    float S0[8], C0[8], S1[8], C1[8];   // compile-time indices: the sums stay in registers
+  float S0[8], C0[8], S1[8], C1[8];   // compile-time indices: the sums stay in registers
 #pragma unroll
-    for (int j = 0; j < 8; ++j) { S0[j] = 0.f; C0[j] = 0.f; S1[j] = 0.f; C1[j] = 0.f; }
-    auto accum4 = [&](int i, float4 f, float(&Sa)[8], float(&Ca)[8]) {
-      const dfl fp = {f.x, f.y}, fm = {f.z, f.w};
-      const float4 E = pol_dsa[2 * i], Bv = pol_dsa[2 * i + 1];
-      const dfl er = {E.x, E.y}, ei = {E.z, E.w}, br = {Bv.x, Bv.y}, bi = {Bv.z, Bv.w};
-      dot2_acc(Sa[0], Ca[0], fp, er);
-      dot2_acc(Sa[1], Ca[1], fm, bi);
-      dot2_acc(Sa[2], Ca[2], fp, ei);
-      dot2_acc(Sa[3], Ca[3], fm, br);
-      dot2_acc(Sa[4], Ca[4], fp, br);
-      dot2_acc(Sa[5], Ca[5], fm, ei);
-      dot2_acc(Sa[6], Ca[6], fp, bi);
-      dot2_acc(Sa[7], Ca[7], fm, er);
-    };
-    auto accum = [&](int i, float(&Sa)[8], float(&Ca)[8]) { accum4(i, tab[(base + i) * RP + k], Sa, Ca); };
-    int i = max(m < 2 ? 2 - m : 0, ls[(size_t)m * RP + k] - m);
-    if (i < Lm && (i & 1)) accum(i++, S1, C1);
-    for (; i + 3 < Lm; i += 4) {   // four rows of the table in flight
-      const float4 f0 = tab[(base + i) * RP + k], f1 = tab[(base + i + 1) * RP + k];
-      const float4 f2 = tab[(base + i + 2) * RP + k], f3 = tab[(base + i + 3) * RP + k];
-      accum4(i, f0, S0, C0);
-      accum4(i + 1, f1, S1, C1);
-      accum4(i + 2, f2, S0, C0);
-      accum4(i + 3, f3, S1, C1);
-    }
-    for (; i + 1 < Lm; i += 2) {
-      accum(i, S0, C0);
-      accum(i + 1, S1, C1);
-    }
-    if (i < Lm) accum(i, S0, C0);
-    double e[8], o[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      e[j] = (double)S0[j] + (double)C0[j];
-      o[j] = (double)S1[j] + (double)C1[j];
-    }
-    // north: Q = -(F+ E + i F- B), U = -(F+ B - i F- E); south: F+ -> p F+, F- -> -p F-
-    const double qnr = -((e[0] + o[0]) - (e[1] + o[1])), qni = -((e[2] + o[2]) + (e[3] + o[3]));
-    const double qsr = -((e[0] - o[0]) + (e[1] - o[1])), qsi = -((e[2] - o[2]) - (e[3] - o[3]));
-    const double unr = -((e[4] + o[4]) + (e[5] + o[5])), uni = -((e[6] + o[6]) - (e[7] + o[7]));
-    const double usr = -((e[4] - o[4]) - (e[5] - o[5])), usi = -((e[6] - o[6]) + (e[7] - o[7]));
-    FSQ[(size_t)m * RP + k] = make_double4_32a(qnr, qni, qsr, qsi);
-    FSU[(size_t)m * RP + k] = make_double4_32a(unr, uni, usr, usi);
+  for (int j = 0; j < 8; ++j) { S0[j] = 0.f; C0[j] = 0.f; S1[j] = 0.f; C1[j] = 0.f; }
+  auto accum = [&](int i, float4 f, float(&Sa)[8], float(&Ca)[8]) {
+    const dfl fp = {f.x, f.y}, fm = {f.z, f.w};
+    const float4 E = coef[2 * i], Bv = coef[2 * i + 1];
+    const dfl er = {E.x, E.y}, ei = {E.z, E.w}, br = {Bv.x, Bv.y}, bi = {Bv.z, Bv.w};
+    dot2_acc(Sa[0], Ca[0], fp, er);
+    dot2_acc(Sa[1], Ca[1], fm, bi);
+    dot2_acc(Sa[2], Ca[2], fp, ei);
+    dot2_acc(Sa[3], Ca[3], fm, br);
+    dot2_acc(Sa[4], Ca[4], fp, br);
+    dot2_acc(Sa[5], Ca[5], fm, ei);
+    dot2_acc(Sa[6], Ca[6], fp, bi);
+    dot2_acc(Sa[7], Ca[7], fm, er);
+  };
+  const int istart = m < 2 ? 2 - m : 0;   // rows of l < 2 hold zeros; their coefficients may be anything
+  for (int i = i0; i < Lm; i += 2) {
+    cp_wait<kSynDepth / 2 - 1>();
+    const float4 f0 = ring[(size_t)(i & (kSynDepth - 1)) * nt];
+    const float4 f1 = ring[(size_t)((i + 1) & (kSynDepth - 1)) * nt];
+    if (i >= istart) accum(i, f0, S0, C0);
+    if (i + 1 < Lm && i + 1 >= istart) accum(i + 1, f1, S1, C1);
+    fetch(i + kSynDepth);   // into the slots just used
   }
+  cp_wait<0>();
+  if (k >= RP) return;
+  dfl e[8], o[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    e[j] = df_norm(S0[j], C0[j]);
+    o[j] = df_norm(S1[j], C1[j]);
+  }
+  // sums over both parities (p) and their difference (d)
+  auto p = [&](int j) { return df_add(e[j], o[j]); };
+  auto d = [&](int j) { return df_add(e[j], df_neg(o[j])); };
+  auto put = [](dfl x, dfl y) { return df_pack(df_neg(df_add(x, y))); };
+  // north: Q = -(F+ E + i F- B), U = -(F+ B - i F- E); south: F+ -> p F+, F- -> -p F-
+  FSQ[(size_t)m * RP + k] = make_double4_32a(put(p(0), df_neg(p(1))), put(p(2), p(3)), put(d(0), d(1)),
+                                             put(d(2), df_neg(d(3))));
+  FSU[(size_t)m * RP + k] = make_double4_32a(put(p(4), p(5)), put(p(6), df_neg(p(7))), put(d(4), df_neg(d(5))),
+                                             put(d(6), d(7)));
 }
 
 // Eq. 3 per pixel with the 3 x 3 messenger and the chi^2 partials (sum r^T W r and r^T (N + (lambda-1) tau)^-1 r).
@@ -502,7 +576,11 @@ void Pol::synth(cudaStream_t s, const double2 *alm, double *map, const Ctl *gate
   P->launch_leg(la, s, LEG_SYNTH);                                    // T -> the plan's FS
   if (df) {
     raise_smem_cap(reinterpret_cast<const void *>(spin2_synthesis_df_kernel));
-    spin2_synthesis_df_kernel<<<lmax + 1, kPolThreads, sizeof(float4) * 2 * (lmax + 1), s>>>(
+    // half of the ring pairs a CTA up to 256 of them: enough CTAs where few values of m do not fill the chip,
+    // and the coefficients (whose conversion is FP64 work) read by few
+    const int nt = std::min(kPolThreads, std::max(32, (RP / 2 + 31) / 32 * 32));
+    const dim3 grid(lmax + 1, (RP + nt - 1) / nt);
+    spin2_synthesis_df_kernel<<<grid, nt, sizeof(float4) * (kSynDepth * nt + 2 * (size_t)(lmax + 1)), s>>>(
         gate, reinterpret_cast<const float4 *>(d_tab), P->d_ls, alm + nalm, alm + 2 * nalm, lmax, RP, d_FSQ, d_FSU);
   } else {
     raise_smem_cap(reinterpret_cast<const void *>(spin2_synthesis_kernel));
@@ -537,8 +615,12 @@ void Pol::analysis(cudaStream_t s, const double *map, double2 *alm, const Ctl *g
   P->launch_leg(la, s, LEG_ANALYSIS);                                 // T
   if (df) {
     raise_smem_cap(reinterpret_cast<const void *>(spin2_analysis_df_kernel));
-    spin2_analysis_df_kernel<<<lmax + 1, kPolThreads, sizeof(float4) * 4 * RP, s>>>(
-        gate, reinterpret_cast<const float4 *>(d_tab), P->d_ls, d_FTQ, d_FTU, lmax, RP, alm + nalm, alm + 2 * nalm);
+    // 64 values of l a CTA (four row pairs a warp), 16 where lmax leaves few chunks
+    const int lchunk = lmax >= 256 ? 64 : 16;
+    const dim3 grid(lmax + 1, (lmax + lchunk) / lchunk);
+    spin2_analysis_df_kernel<<<grid, kPolThreads, sizeof(float4) * 4 * RP + sizeof(int) * ((RP + 31) / 32), s>>>(
+        gate, reinterpret_cast<const float4 *>(d_tab), P->d_ls, d_FTQ, d_FTU, lmax, RP, lchunk, alm + nalm,
+        alm + 2 * nalm);
   } else {
     raise_smem_cap(reinterpret_cast<const void *>(spin2_analysis_kernel));
     spin2_analysis_kernel<<<lmax + 1, kPolThreads, sizeof(double4_32a) * 2 * RP, s>>>(

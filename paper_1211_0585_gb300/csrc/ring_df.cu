@@ -4,13 +4,15 @@
 // half-pixel shift, inverse DFT, Eq. 3 per pixel with the chi^2 partials,
 // forward DFT, unfold), but every FFT value is a pair of floats per real
 // component and every butterfly is built from error-free transformations
-// (two_sum, two_prod), because GB300's FP64 pipe is 1/63 of its FP32 pipe.
-// The per-pixel Eq. 3 update and the chi^2 partials stay in double (one pass
-// over the ring's pixels). Tables (twiddles, half-shift, chirp, Bluestein
+// (two_sum, two_prod), because GB300's FP64 pipe is 1/63 of its FP32 pipe. So
+// are the Fourier records on both sides, the fold, the unfold, the per-pixel
+// Eq. 3 update and the chi^2 sums up to the warp's; the FP64 pipe sees the
+// sums over warps and the gains of a new lambda. Tables (twiddles, half-shift, chirp, Bluestein
 // filter) are stored as double-float pairs, converted once from the double
 // tables when the plan is built.
 #include <cuda_runtime.h>
 
+#include "df.cuh"
 #include "fft.cuh"
 #include "fold.cuh"
 #include "wf_internal.h"
@@ -19,55 +21,22 @@ namespace wfk {
 
 namespace {
 
-struct dd { float h, l; };
-
-__device__ __forceinline__ dd mk(double v) {
-  const float h = (float)v;
-  return {h, (float)(v - (double)h)};
-}
-__device__ __forceinline__ double todbl(dd a) { return (double)a.h + (double)a.l; }
-
-__device__ __forceinline__ dd dadd(dd a, dd b) {
-  const float s = a.h + b.h;
-  const float bb = s - a.h;
-  float e = (a.h - (s - bb)) + (b.h - bb);
-  e += a.l + b.l;
-  const float r = s + e;
-  return {r, e - (r - s)};
-}
-__device__ __forceinline__ dd dneg(dd a) { return {-a.h, -a.l}; }
-__device__ __forceinline__ dd dmul(dd a, dd b) {
-  const float p = a.h * b.h;
-  float e = fmaf(a.h, b.h, -p);
-  e = fmaf(a.h, b.l, fmaf(a.l, b.h, e));
-  const float r = p + e;
-  return {r, e - (r - p)};
-}
-
 // complex double-float held as float4 (re.h, re.l, im.h, im.l)
-__device__ __forceinline__ float4 pack(dd re, dd im) { return make_float4(re.h, re.l, im.h, im.l); }
-__device__ __forceinline__ dd RE(float4 v) { return {v.x, v.y}; }
-__device__ __forceinline__ dd IM(float4 v) { return {v.z, v.w}; }
-__device__ __forceinline__ float4 cmul(float4 a, float4 b) {
-  const dd re = dadd(dmul(RE(a), RE(b)), dneg(dmul(IM(a), IM(b))));
-  const dd im = dadd(dmul(RE(a), IM(b)), dmul(IM(a), RE(b)));
-  return pack(re, im);
-}
+__device__ __forceinline__ dfl RE(float4 v) { return {v.x, v.y}; }
+__device__ __forceinline__ dfl IM(float4 v) { return {v.z, v.w}; }
+__device__ __forceinline__ float4 cmul(float4 a, float4 b) { return OpsDF::mul(a, b); }
 __device__ __forceinline__ float4 cconj(float4 a) { return make_float4(a.x, a.y, -a.z, -a.w); }
 __device__ __forceinline__ float4 cneg(float4 a) { return make_float4(-a.x, -a.y, -a.z, -a.w); }
 
-__device__ void block_sum2(double &a, double &b, double *red) {
+// the compensated sum (S, C) over the warp's lanes, on every lane
+__device__ __forceinline__ void warp_sum_df(float &S, float &C) {
+#pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_xor_sync(0xffffffffu, a, o);
-    b += __shfl_xor_sync(0xffffffffu, b, o);
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) { red[2 * warp] = a; red[2 * warp + 1] = b; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double sa = 0.0, sb = 0.0;
-    for (int w2 = 0; w2 < (int)(blockDim.x >> 5); ++w2) { sa += red[2 * w2]; sb += red[2 * w2 + 1]; }
-    a = sa; b = sb;
+    const float rS = __shfl_xor_sync(0xffffffffu, S, o), rC = __shfl_xor_sync(0xffffffffu, C, o);
+    const float s = S + rS;
+    const float bb = s - S;
+    C = C + rC + ((S - (s - bb)) + (rS - bb));
+    S = s;
   }
 }
 
@@ -84,6 +53,9 @@ __device__ void block_sum2(double &a, double &b, double *red) {
 // inverse transform's output, which is the forward transform's input order.
 // 256 threads and three CTAs per SM (up to 64 KB of FFT buffer each at Nside
 // 512), so that one pair's barriers and global loads overlap another's work.
+// With the records, the fold and the sums in double, the FP64 pipe was as busy
+// as the FP32 one (37 %) and the kernel took 250 us at Nside 512, 65 us at 256;
+// in double-float throughout 203 and 52 us.
 constexpr int kRingDfThreads = 256;
 template <int MODE>
 __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingArgs A, const RingDfArgs T) {
@@ -97,8 +69,8 @@ __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingAr
   const int Mp = M;
   // [Mp] (swizzled, px): shared memory, or this CTA's part of the global scratch
   float4 *buf = A.scratch ? reinterpret_cast<float4 *>(A.scratch) + (size_t)blockIdx.x * M : rsm;
-  __shared__ double red[64];
-  __shared__ double4_16a fold_part[kRingDfThreads];
+  __shared__ float2 red[kRingDfThreads / 32][4];
+  __shared__ FoldPair fold_part[kRingDfThreads];
 
   int L = A.lsht;
   double lam = 1.0;
@@ -114,9 +86,9 @@ __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingAr
   const int k = rg.pair;
 
   if (MODE == RING_SYNTH || MODE == RING_ITER) {
-    // folding is a handful of additions: done in double; Z = G_N + i G_S
-    fold_ring2(A.FS, A.RP, k, rg.shifted, n, L, fold_part, [&](int q, double2 gN, double2 gS) {
-      float4 acc = pack(mk(gN.x - gS.y), mk(gN.y + gS.x));
+    // Z = G_N + i G_S
+    fold_ring2(A.FS, A.RP, k, rg.shifted, n, L, fold_part, [&](int q, float4 gN, float4 gS) {
+      float4 acc = df_pair(df_add(RE(gN), df_neg(IM(gS))), df_add(IM(gN), RE(gS)));
       if (rg.shifted) acc = cmul(acc, hs[q]);
       buf[px<OpsDF>(q)] = rg.blue ? cmul(cconj(acc), ch[q]) : acc;
     });
@@ -136,69 +108,71 @@ __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingAr
   if (MODE == RING_SYNTH) {
     for (int p = threadIdx.x; p < n; p += blockDim.x) {
       const float4 z = pixel(p);
-      A.map_out[rg.off + p] = todbl(RE(z));
-      if (two) A.map_out[offS + p] = todbl(IM(z));
+      A.map_out[rg.off + p] = df_to(RE(z));
+      if (two) A.map_out[offS + p] = df_to(IM(z));
     }
     return;
   }
   if (MODE == RING_ITER) {
     // Eq. 3 and the chi^2 partials in double-float (the FP64 pipe is 1/63 of the
-    // FP32 one); the per-thread partials become doubles for the block sums
-    dd cnN{0.f, 0.f}, clN{0.f, 0.f}, cnS{0.f, 0.f}, clS{0.f, 0.f};
+    // FP32 one): compensated sums per thread and warp, the sum over warps in double
+    float cs[4] = {0.f, 0.f, 0.f, 0.f}, cc[4] = {0.f, 0.f, 0.f, 0.f};   // north chi2, chi2_lambda, south
     const bool fresh = T.gainlam[pr.x] == lam;   // gains of this pair already at this lambda
-    const dd ltd = mk(lam * A.tau);
+    const dfl ltd = df_from(lam * A.tau);
     const double l1t = (lam - 1.0) * A.tau;
-    auto update = [&](long long at, dd s, dd &cn, dd &cl) {  // Eq. 3, returns u
+    auto update = [&](long long at, dfl s, int half) {  // Eq. 3, returns u
       const float2 d2 = T.d[at], w2 = T.w[at];
-      const dd dv{d2.x, d2.y}, wv{w2.x, w2.y};
-      dd g;
+      const dfl dv{d2.x, d2.y}, wv{w2.x, w2.y};
+      dfl g;
       if (fresh) {
         const float2 g2 = T.gain[at];
-        g = dd{g2.x, g2.y};
+        g = dfl{g2.x, g2.y};
       } else {  // the first pass at a new lambda: the gain from w in double
         const double w = A.w[at];
-        g = mk(w / (1.0 + l1t * w));
+        g = df_from(w / (1.0 + l1t * w));
         T.gain[at] = make_float2(g.h, g.l);
       }
-      const dd res = dadd(dv, dneg(s));
-      const dd r2 = dmul(res, res);
-      cn = dadd(cn, dmul(wv, r2));
-      cl = dadd(cl, dmul(g, r2));
-      return dmul(dmul(ltd, g), res);
+      const dfl res = df_add(dv, df_neg(s));
+      const dfl r2 = df_mul(res, res);
+      dot2_acc(cs[2 * half], cc[2 * half], wv, r2);
+      dot2_acc(cs[2 * half + 1], cc[2 * half + 1], g, r2);
+      return df_mul(df_mul(ltd, g), res);
     };
     for (int p = threadIdx.x; p < n; p += blockDim.x) {
       const float4 z = pixel(p);
-      const dd uN = update(rg.off + p, RE(z), cnN, clN);
-      const dd uS = two ? update(offS + p, IM(z), cnS, clS) : dd{0.f, 0.f};
-      const float4 u = pack(uN, uS);
+      const dfl uN = update(rg.off + p, RE(z), 0);
+      const dfl uS = two ? update(offS + p, IM(z), 1) : dfl{0.f, 0.f};
+      const float4 u = df_pair(uN, uS);
       buf[loc(p)] = rg.blue ? cmul(u, ch[p]) : u;
     }
-    double c2n = todbl(cnN), c2l = todbl(clN), c2nS = todbl(cnS), c2lS = todbl(clS);
     if (rg.blue) {
       for (int q = n + threadIdx.x; q < M; q += blockDim.x) buf[px<OpsDF>(q)] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    block_sum2(c2n, c2l, red);
-    if (threadIdx.x == 0) {
-      A.ring_part[2 * pr.x] = c2n;
-      A.ring_part[2 * pr.x + 1] = c2l;
-    }
-    __syncthreads();
-    if (two) {
-      block_sum2(c2nS, c2lS, red);
-      if (threadIdx.x == 0) {
-        A.ring_part[2 * pr.y] = c2nS;
-        A.ring_part[2 * pr.y + 1] = c2lS;
+    {
+      const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        warp_sum_df(cs[i], cc[i]);
+        if (lane == 0) red[warp][i] = make_float2(cs[i], cc[i]);
+      }
+      __syncthreads();   // also orders the pixel pass before the forward transform
+      if (threadIdx.x < (two ? 4 : 2)) {
+        double v = 0.0;
+        for (int w = 0; w < kRingDfThreads / 32; ++w) {
+          const float2 r = red[w][threadIdx.x];
+          v += (double)r.x + (double)r.y;
+        }
+        A.ring_part[2 * (threadIdx.x < 2 ? pr.x : pr.y) + (threadIdx.x & 1)] = v;
+      }
+      if (threadIdx.x == 0 && !fresh) {  // after the barrier: every gain of the pair is written
+        T.gainlam[pr.x] = lam;
+        if (two) T.gainlam[pr.y] = lam;
       }
     }
-    if (threadIdx.x == 0 && !fresh) {  // after block_sum2's barrier: every gain of the pair is written
-      T.gainlam[pr.x] = lam;
-      if (two) T.gainlam[pr.y] = lam;
-    }
-    __syncthreads();
   } else {  // RING_ANALYSIS: u = the input maps
     for (int p = threadIdx.x; p < M; p += blockDim.x) {
       if (p < n) {
-        const float4 u = pack(mk(A.map_in[rg.off + p]), mk(two ? A.map_in[offS + p] : 0.0));
+        const float4 u = df_pair(df_from(A.map_in[rg.off + p]), df_from(two ? A.map_in[offS + p] : 0.0));
         buf[loc(p)] = rg.blue ? cmul(u, ch[p]) : u;
       } else if (rg.blue) {
         buf[px<OpsDF>(p)] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -209,31 +183,29 @@ __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingAr
 
   if (rg.blue) bluestein4<OpsDF, 1>(buf, Mp, M, rg.logM, Bf, T.tw, A.logMmax);
   else fft_dit4<OpsDF, 1>(buf, Mp, M, rg.logM, -1, T.tw, A.logMmax);
+  const dfl om = df_from(0.5 * A.omega);
   for (int m = threadIdx.x; m <= L; m += blockDim.x) {
     const int q = m % n, j = m / n, qn = q ? n - q : 0;
     const float4 Zq = rg.blue ? cmul(ch[q], buf[px<OpsDF>(q)]) : buf[px<OpsDF>(q)];
     const float4 Zn = rg.blue ? cmul(ch[qn], buf[px<OpsDF>(qn)]) : buf[px<OpsDF>(qn)];
-    // U_N = (Z_q + conj Z_{n-q}) / 2, U_S = (Z_q - conj Z_{n-q}) / (2 i)
-    float4 UN = pack(dadd(RE(Zq), RE(Zn)), dadd(IM(Zq), dneg(IM(Zn))));
-    float4 US = pack(dadd(IM(Zq), IM(Zn)), dadd(RE(Zn), dneg(RE(Zq))));
-    UN = make_float4(0.5f * UN.x, 0.5f * UN.y, 0.5f * UN.z, 0.5f * UN.w);
-    US = make_float4(0.5f * US.x, 0.5f * US.y, 0.5f * US.z, 0.5f * US.w);
+    // U_N = (Z_q + conj Z_{n-q}) / 2, U_S = (Z_q - conj Z_{n-q}) / (2 i); the halves are in omega
+    float4 UN = df_pair(df_add(RE(Zq), RE(Zn)), df_add(IM(Zq), df_neg(IM(Zn))));
+    float4 US = df_pair(df_add(IM(Zq), IM(Zn)), df_add(RE(Zn), df_neg(RE(Zq))));
     if (rg.shifted) {
       UN = cmul(UN, cconj(hs[q]));
       US = cmul(US, cconj(hs[q]));
       if (j & 1) { UN = cneg(UN); US = cneg(US); }
     }
-    const double om = A.omega;
-    A.FT[(size_t)m * A.RP + k] = two ? make_double4_32a(om * todbl(RE(UN)), om * todbl(IM(UN)), om * todbl(RE(US)),
-                                                      om * todbl(IM(US)))
-                                     : make_double4_32a(om * todbl(RE(UN)), om * todbl(IM(UN)), 0.0, 0.0);
+    A.FT[(size_t)m * A.RP + k] = make_double4_32a(
+        df_pack(df_mul(RE(UN), om)), df_pack(df_mul(IM(UN), om)), two ? df_pack(df_mul(RE(US), om)) : 0.0,
+        two ? df_pack(df_mul(IM(US), om)) : 0.0);
   }
 }
 
 // double -> double-float (hi, lo) per element
 __global__ void to_df2_kernel(const double *src, float2 *dst, long long n) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const dd v = mk(src[i]);
+    const dfl v = df_from(src[i]);
     dst[i] = make_float2(v.h, v.l);
   }
 }
@@ -249,7 +221,7 @@ void launch_to_df2(const double *src, float2 *dst, long long n, cudaStream_t s) 
 __global__ void to_df_kernel(const double2 *src, float4 *dst, long long n) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const double2 v = src[i];
-    dst[i] = pack(mk(v.x), mk(v.y));
+    dst[i] = df_pair(df_from(v.x), df_from(v.y));
   }
 }
 
