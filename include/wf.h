@@ -187,7 +187,7 @@ wf_status wf_plan_legendre_table(wf_plan_t plan, int lsht, int64_t *held, int64_
 /* Kernel launches in one messenger iteration of the plan's single-solve path
  * (WF_PREC_FP64 or WF_PREC_FP64_NATIVE): the ring stage (one launch, or at
  * Nside 2048 two: the rings whose FFT buffers exceed shared memory run apart),
- * the Legendre stage and the controller. Used to count device launches; *n
+ * the Legendre stage (one launch, two with a lambda table) and the controller. Used to count device launches; *n
  * must not be NULL. */
 wf_status wf_plan_kernels_per_iteration(wf_plan_t plan, int *n);
 

@@ -2,7 +2,7 @@
 // table. Right-hand sides go in groups of up to kLegBatchMax maps that
 // iterate together: each map runs its own ring stage (Eq. 3 with its own data
 // and cached gains) and its own controller (Sect. 3 schedule and stop rule),
-// and one launch of legendre_batch_kernel does every map's Legendre stage,
+// and one pass of the table kernels (legendre_tab.cu) does every map's Legendre stage,
 // reading each table row once for the group. A map that has stopped is skipped
 // by every kernel until the group's last map stops. The first map of a group
 // uses the plan's own buffers; the others use plans of the same shape that
@@ -61,6 +61,7 @@ wf_status make_batch(Plan *P, int nb) {
     o.legendre_table_bytes = 0;   // the plan's table serves every map
     wf_plan_t q = nullptr;
     wf_status st = wf_plan_create(P->nside, P->lmax, P->h_cl.data(), unit.data(), nullptr, &o, &q);
+    if (!st) st = static_cast<Plan *>(q)->alloc_tab_work();   // no table of its own, but its part of the launches
     if (!st) st = plan_rebind(static_cast<Plan *>(q), P->h_cl.data(), w.data(), P->tau, P->n_obs);
     if (st) { if (q) wf_plan_destroy(q); delete F; return st; }
     F->sub.push_back(static_cast<Plan *>(q));
@@ -97,13 +98,9 @@ wf_status solve_fp64_batch(Plan *P, int nrhs, const double *d, int d_on_device, 
   LegBatchMaps bm{};
   bm.n = nb;
   for (int b = 0; b < nb; ++b) {
-    bm.FT[b] = M[b]->d_FT;
-    bm.FS[b] = M[b]->d_FS;
-    bm.alm[b] = M[b]->d_s;
-    bm.m_part[b] = M[b]->d_m_part;
-    bm.ctl[b] = M[b]->d_ctl;
-    bm.cl[b] = M[b]->d_cl;
-    bm.tau[b] = M[b]->tau;
+    M[b]->tab_map(bm, b);
+    bm.part[b] = M[b]->d_part;
+    bm.coef[b] = M[b]->d_coef;
   }
   const int gi = P->opt.graph_iters;
   std::vector<const void *> hist(nb);
@@ -115,7 +112,7 @@ wf_status solve_fp64_batch(Plan *P, int nrhs, const double *d, int d_on_device, 
     FB_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
     for (int i = 0; i < gi; ++i) {
       for (int b = 0; b < nb; ++b) M[b]->launch_rng(M[b]->ring_args(), s, RING_ITER);
-      launch_legendre_batch(P->leg_args(), P->legdf_args(), bm, nb, s);
+      launch_legendre_tab(P->leg_args(), P->legdf_args(), bm, nb, s, LEG_ITER);
       for (int b = 0; b < nb; ++b)
         launch_control(M[b]->d_ctl, M[b]->d_ring_part, M[b]->R, M[b]->d_m_part, M[b]->lmax, M[b]->d_cl,
                        M[b]->d_hist, M[b]->hist_cap, s);

@@ -296,9 +296,10 @@ static wf_status build_legendre(Plan *P) {
       leg_tab_smem(lmax, P->RP) <= kTabSmemLimit) {
     std::vector<long long> poff(lmax + 1);
     long long r = 0;
-    for (int m = 0; m <= lmax; ++m) { poff[m] = r; r += (lmax - m + 2) / 2; }
+    for (int m = 0; m <= lmax; ++m) { poff[m] = r; r += tab_rows(lmax, m); }
     if ((st = P->dalloc((void **)&P->d_poff, sizeof(long long) * poff.size()))) return st;
     if ((st = P->dalloc((void **)&P->d_tab, tab_bytes))) return st;
+    if ((st = P->alloc_tab_work())) return st;
     WF_CUDA(cudaMemcpyAsync(P->d_poff, poff.data(), sizeof(long long) * poff.size(), cudaMemcpyHostToDevice,
                             P->stream));
     if (P->RP % 32) WF_CUDA(cudaMemsetAsync(P->d_tab, 0, tab_bytes, P->stream));  // columns past RP
@@ -308,6 +309,11 @@ static wf_status build_legendre(Plan *P) {
   WF_CUDA(cudaStreamSynchronize(P->stream));
   WF_CUDA(cudaGetLastError());
   return WF_OK;
+}
+
+wf_status Plan::alloc_tab_work() {
+  wf_status st = dalloc((void **)&d_coef, sizeof(float4) * nalm);
+  return st ? st : dalloc((void **)&d_part, sizeof(double) * 3 * (size_t)(lmax + 1) * tab_chunks(lmax));
 }
 
 wf_status Plan::alloc_work() {
@@ -390,7 +396,7 @@ RingArgs Plan::ring_args() const {
 LegArgs Plan::leg_args() const {
   LegArgs a{};
   a.x = d_x; a.rec = d_rec; a.ls = d_ls; a.sv = d_sv; a.cl = d_cl; a.FT = d_FT; a.FS = d_FS; a.alm = d_s;
-  a.m_part = d_m_part; a.ctl = d_ctl; a.lsht = lmax; a.lmax = lmax; a.RP = RP; a.omega = omega; a.tau = tau;
+  a.m_part = d_m_part; a.part = d_part; a.coef = d_coef; a.ctl = d_ctl; a.lsht = lmax; a.lmax = lmax; a.RP = RP; a.omega = omega; a.tau = tau;
   return a;
 }
 
@@ -568,8 +574,9 @@ wf_status wf_plan_info(wf_plan_t plan, int64_t *npix, int64_t *nalm, double *tau
 
 wf_status wf_plan_kernels_per_iteration(wf_plan_t plan, int *n) {
   if (!plan || !n) { set_error("wf_plan_kernels_per_iteration: NULL argument"); return WF_EINVAL; }
-  // the ring stage (one launch per single-solve ring class), Legendre stage, controller
-  *n = (int)static_cast<const Plan *>(plan)->rsingle.size() + 2;
+  // the ring stage (one launch per single-solve ring class), Legendre stage (two over the table), controller
+  const Plan *P = static_cast<const Plan *>(plan);
+  *n = (int)P->rsingle.size() + (P->d_tab && P->opt.precision != WF_PREC_FP64_NATIVE ? 3 : 2);
   return WF_OK;
 }
 

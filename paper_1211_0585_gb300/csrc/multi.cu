@@ -165,7 +165,7 @@ void Multi::enqueue_iteration(cudaStream_t s) {
       }
       LegArgs la = P0->leg_args();
       la.lsht = lmax;
-      launch_legendre_batch(la, P0->legdf_args(), syn, nb, s, LEG_SYNTH);
+      launch_legendre_tab(la, P0->legdf_args(), syn, nb, s, LEG_SYNTH);
       for (int b = 0; b < nb; ++b) {
         const int k = k0 + b;
         RingArgs ra = P[k]->ring_args();   // map k's data, noise, gains and Fourier buffers
@@ -173,7 +173,7 @@ void Multi::enqueue_iteration(cudaStream_t s) {
         ra.ring_part = d_ring_part + (size_t)k * 2 * R;
         P[k]->launch_rng(ra, s, RING_ITER);
       }
-      launch_legendre_batch(la, P0->legdf_args(), ana, nb, s, LEG_ANALYSIS);
+      launch_legendre_tab(la, P0->legdf_args(), ana, nb, s, LEG_ANALYSIS);
     }
     multi_eq4_kernel<<<lmax + 1, 128, 0, s>>>(d_ctl, K, lmax, nalm, omega, d_beam, d_tau, d_cl, d_ta, d_s, d_m_part);
     launch_control(d_ctl, d_ring_part, K * R, d_m_part, lmax, d_lamcl, d_hist, hist_cap, s);

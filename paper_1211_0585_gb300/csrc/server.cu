@@ -194,7 +194,8 @@ wf_options fp64_plan_options(size_t budget) {
 }
 
 // an FP64 plan: its Fourier arrays (two 32-byte double-float complexes per (m,
-// ring pair)), recurrence tables (40 bytes per (m, ring pair), 48 per a_lm), the
+// ring pair)), recurrence tables (40 bytes per (m, ring pair), 64 per a_lm with the
+// synthesis coefficients), the
 // per-pixel buffers and ring FFT tables (about 176 bytes per pixel in all), the
 // posterior-gradient buffers, plus the precomputed lambda table when it is
 // within the pool's limit
@@ -204,7 +205,7 @@ size_t fp64_bytes(size_t budget, int nside, int lmax) {
   const size_t npix = 12 * (size_t)nside * nside, nalm = (size_t)(lmax + 1) * (lmax + 2) / 2;
   const size_t nmk = (size_t)(lmax + 1) * 2 * nside;
   const size_t posterior = 2 * npix * sizeof(double) + 2 * nalm * 16;  // rel_posterior_grad buffers
-  return nmk * (64 + 40) + nalm * 48 + npix * 176 + posterior + (tab <= o.legendre_table_bytes ? tab : 0);
+  return nmk * (64 + 40) + nalm * 64 + npix * 176 + posterior + (tab <= o.legendre_table_bytes ? tab : 0);
 }
 
 size_t bytes_in_use(wf_server_s *S) {

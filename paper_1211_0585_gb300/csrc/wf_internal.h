@@ -124,6 +124,8 @@ struct LegArgs {
   double2 *alm;           // state / output a_lm
   const double2 *alm_in;  // LEG_SYNTH input
   double *m_part;         // LEG_ITER: [lmax+1][3] chi2_S, incr2, norm2
+  double *part;           // LEG_ITER, table form: [lmax+1][tab_chunks(lmax)][3]
+  float4 *coef;           // LEG_ITER, table form: [nalm] the new state in double-float
   const Ctl *ctl;
   const Ctl *gate;        // LEG_SYNTH / LEG_ANALYSIS inside a controlled iteration: skip once gate->done
                           // (nullptr for the standalone transforms)
@@ -141,26 +143,29 @@ struct LegDfArgs {
   const long long *poff;  // [lmax+1] first table row of each m
 };
 
-// Per-map buffers of the batched FP64 Legendre stage (legendre_batch.cu): up to
+// Legendre stage over the precomputed table (legendre_tab.cu), for up to
 // kLegBatchMax maps of one shape, each with its own Fourier arrays, state, C_l,
 // tau, partial sums and controller.
 constexpr int kLegBatchMax = 2;
-constexpr int kSynRowsB = 4;      // batched synthesis: table rows per load batch
+constexpr int kTabRows = 96;      // table rows (two l each) of an analysis CTA
 struct LegBatchMaps {
   int n;                          // maps in use (the rest are skipped)
   const double4_32a *FT[kLegBatchMax];
   double4_32a *FS[kLegBatchMax];
-  double2 *alm[kLegBatchMax];
-  double *m_part[kLegBatchMax];
-  const Ctl *ctl[kLegBatchMax];
+  double2 *alm[kLegBatchMax];     // state; the standalone transforms' a_lm in (synthesis) or t_l out (analysis)
+  const Ctl *ctl[kLegBatchMax];   // controller; standalone transforms: skip the map once done (nullptr: never)
+  // an iteration's, nullptr for the standalone transforms
+  double *m_part[kLegBatchMax];   // [lmax+1][3] chi2_S, incr2, norm2
+  double *part[kLegBatchMax];     // [lmax+1][tab_chunks(lmax)][3] the same by chunk of rows
+  float4 *coef[kLegBatchMax];     // [nalm] the new state as double-floats (re hi, re lo, im hi, im lo)
   const double *cl[kLegBatchMax];
   double tau[kLegBatchMax];
 };
-size_t leg_batch_smem(int nb, int lmax, int RP);
-// mode: LEG_ITER (NB independent iterations), LEG_SYNTH or LEG_ANALYSIS (NB maps' transforms, a_lm in / t_l out
-// through Bm.alm); the table form only
-void launch_legendre_batch(const LegArgs &a, const LegDfArgs &d, const LegBatchMaps &bm, int nb, cudaStream_t s,
-                           int mode = LEG_ITER);
+// chunks of kTabRows rows of the longest column (m = 0)
+int tab_chunks(int lmax);
+// mode: LEG_ITER (nb independent iterations), LEG_SYNTH or LEG_ANALYSIS; nb = 1 or 2
+void launch_legendre_tab(const LegArgs &a, const LegDfArgs &d, const LegBatchMaps &bm, int nb, cudaStream_t s,
+                         int mode);
 
 // Double-float copies of the ring-stage tables (ring_df.cu): float4 =
 // (re hi, re lo, im hi, im lo).
@@ -257,10 +262,10 @@ void launch_legendre_df(const LegArgs &a, const LegDfArgs &d, cudaStream_t s, in
 void launch_posterior_maps(const double *d, const double *w, double *ya, double *wd, long long npix, cudaStream_t s);
 void launch_posterior_norms(const double2 *a, const double2 *ta, const double2 *tb, const double *cl, int lmax,
                             double inv_omega, double *part, cudaStream_t s);
-// rows of the precomputed double-float lambda table (sum over m of ceil((lmax - m + 1) / 2)),
-// each RP float4
+// rows of the precomputed double-float lambda table: of one m (two l each), and of all
+__host__ __device__ inline int tab_rows(int lmax, int m) { return (lmax - m + 2) / 2; }
 size_t lam_table_rows(int lmax);
-// dynamic shared memory of the table form of the Legendre kernel
+// largest dynamic shared memory of the table form's kernels
 size_t leg_tab_smem(int lmax, int RP);
 void launch_lam_table(const double *x, const double2 *rec, const int *ls64, const double2 *sv64, const int *ls_df,
                       const long long *poff, int lmax, int RP, float4 *tab, cudaStream_t s);

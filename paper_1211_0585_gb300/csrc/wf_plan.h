@@ -57,6 +57,8 @@ struct Plan : wf_plan_s {
   float4 *d_tab = nullptr;              // precomputed lambda (FP64 path, when it fits opt.legendre_table_bytes)
   long long *d_poff = nullptr;
   size_t tab_bytes = 0;
+  float4 *d_coef = nullptr;             // table form: the synthesis coefficients and the partial sums by chunk of rows
+  double *d_part = nullptr;
   // working state
   double4_32a *d_FS = nullptr, *d_FT = nullptr;
   double *d_ring_part = nullptr, *d_m_part = nullptr;
@@ -83,6 +85,7 @@ struct Plan : wf_plan_s {
   ~Plan() override;
   wf_status dalloc(void **p, size_t bytes);
   wf_status alloc_work();
+  wf_status alloc_tab_work();           // d_coef, d_part
   wf_status ensure_hist(int cap);
   cudaStream_t run_stream() const;
   RingArgs ring_args() const;
@@ -97,6 +100,11 @@ struct Plan : wf_plan_s {
   void launch_rng(const RingArgs &a, cudaStream_t s, int mode) const {
     if (opt.precision == WF_PREC_FP64_NATIVE) launch_ring(a, rsingle.data(), (int)rsingle.size(), s, mode);
     else launch_ring_df(a, ringdf_args(), psingle.data(), (int)psingle.size(), s, mode);
+  }
+  // this plan's map in slot b of a launch of the table form
+  void tab_map(LegBatchMaps &bm, int b) const {
+    bm.FT[b] = d_FT; bm.FS[b] = d_FS; bm.alm[b] = d_s; bm.ctl[b] = d_ctl; bm.m_part[b] = d_m_part; bm.cl[b] = d_cl;
+    bm.tau[b] = tau;
   }
   // the Legendre stage of the plan's precision
   void launch_leg(const LegArgs &a, cudaStream_t s, int mode) const {
