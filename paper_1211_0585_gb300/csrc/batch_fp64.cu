@@ -1,7 +1,7 @@
 // Batched FP64 solves: wf_solve_batch on a WF_PREC_FP64 plan with a lambda
 // table. Right-hand sides go in groups of up to kLegBatchMax maps that
-// iterate together: each map runs its own ring stage (Eq. 3 with its own data
-// and cached gains) and its own controller (Sect. 3 schedule and stop rule),
+// iterate together: each map has its own ring stage (Eq. 3 with its own data
+// and cached gains, the group's in one launch) and its own controller (Sect. 3 schedule and stop rule),
 // and one pass of the table kernels (legendre_tab.cu) does every map's Legendre stage,
 // reading each table row once for the group. A map that has stopped is skipped
 // by every kernel until the group's last map stops. The first map of a group
@@ -108,14 +108,20 @@ wf_status solve_fp64_batch(Plan *P, int nrhs, const double *d, int d_on_device, 
   if (!F->graph || F->graph_iters != gi || F->graph_hist != hist) {
     if (F->graph) cudaGraphExecDestroy(F->graph);
     F->graph = nullptr;
+    std::vector<RingArgs> ra;
+    std::vector<RingDfArgs> rd;
+    std::vector<CtlMap> rc;
+    for (int b = 0; b < nb; ++b) {
+      rc.push_back(M[b]->ctl_map());
+      ra.push_back(M[b]->ring_args());
+      rd.push_back(M[b]->ringdf_args());
+    }
     cudaGraph_t g;
     FB_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
     for (int i = 0; i < gi; ++i) {
-      for (int b = 0; b < nb; ++b) M[b]->launch_rng(M[b]->ring_args(), s, RING_ITER);
+      P->launch_rng_maps(ra.data(), rd.data(), nb, s, RING_ITER);
       launch_legendre_tab(P->leg_args(), P->legdf_args(), bm, nb, s, LEG_ITER);
-      for (int b = 0; b < nb; ++b)
-        launch_control(M[b]->d_ctl, M[b]->d_ring_part, M[b]->R, M[b]->d_m_part, M[b]->lmax, M[b]->d_cl,
-                       M[b]->d_hist, M[b]->hist_cap, s);
+      launch_control(rc.data(), nb, P->R, P->lmax, s);
     }
     FB_CUDA(cudaStreamEndCapture(s, &g));
     cudaError_t e = cudaGraphInstantiate(&F->graph, g, 0);

@@ -403,7 +403,8 @@ LegArgs Plan::leg_args() const {
 void Plan::enqueue_iteration(cudaStream_t s) {
   launch_rng(ring_args(), s, RING_ITER);
   launch_leg(leg_args(), s, LEG_ITER);
-  launch_control(d_ctl, d_ring_part, R, d_m_part, lmax, d_cl, d_hist, hist_cap, s);
+  const CtlMap c = ctl_map();
+  launch_control(&c, 1, R, lmax, s);
 }
 
 Ctl Plan::make_ctl(int mode, double lambda, int lsht, int n_fixed) const {
@@ -739,7 +740,8 @@ wf_status wf_profile_iterations(wf_plan_t plan, const double *d_dev, double *s_d
     cudaEventRecord(ev[4 * i + 1], s);
     P->launch_leg(P->leg_args(), s, LEG_ITER);
     cudaEventRecord(ev[4 * i + 2], s);
-    launch_control(P->d_ctl, P->d_ring_part, P->R, P->d_m_part, P->lmax, P->d_cl, P->d_hist, P->hist_cap, s);
+    const CtlMap cm = P->ctl_map();
+    launch_control(&cm, 1, P->R, P->lmax, s);
     cudaEventRecord(ev[4 * i + 3], s);
   }
   WF_CUDA(cudaGetLastError());

@@ -95,14 +95,19 @@ __global__ void multi_beam_kernel(const Ctl *ctl, int K, int lmax, long long nal
 }
 
 // Eq. 4 with K messengers, the prior chi^2 of the input state, the increment
-// and norm partials per m (the layout the controller reads)
+// and norm partials per m (the layout the controller reads). Bound by the FP64
+// pipe, so two divisions an l: 1 / C_l and the reciprocal of the denominator,
+// and g_k once a CTA (with 1 / C_l, two quotients, the chi^2's and every g_k a
+// division each: 38 us at Nside 256 / lmax 512 with three maps; now 21)
 __global__ void multi_eq4_kernel(const Ctl *ctl, int K, int lmax, long long nalm, double omega, const double *beam,
                                  const double *tau, const double *cl, const double2 *ta, double2 *s,
                                  double *m_part) {
   __shared__ double red[3][32];
+  __shared__ double gk[kMultiMax];
   if (ctl->done) return;
   const int m = blockIdx.x;
-  const double lam = ctl->lambda;
+  if (threadIdx.x < K) gk[threadIdx.x] = 1.0 / (ctl->lambda * tau[threadIdx.x] * omega);
+  __syncthreads();
   const double wgt = (m == 0) ? 1.0 : 2.0;
   double c2 = 0.0, inc = 0.0, nrm = 0.0;
   for (int l = m + threadIdx.x; l <= lmax; l += blockDim.x) {
@@ -111,17 +116,18 @@ __global__ void multi_eq4_kernel(const Ctl *ctl, int K, int lmax, long long nalm
     const double c = cl[l];
     double2 sn = make_double2(0.0, 0.0);
     if (c > 0.0) {
-      double nx = 0.0, ny = 0.0, den = 1.0 / c;
+      const double ic = 1.0 / c;
+      double nx = 0.0, ny = 0.0, den = ic;
       for (int k = 0; k < K; ++k) {
-        const double b = beam[(size_t)k * (lmax + 1) + l];
-        const double g = 1.0 / (lam * tau[k] * omega);
+        const double b = beam[(size_t)k * (lmax + 1) + l], gb = gk[k] * b;
         const double2 t = ta[(size_t)k * nalm + q];
-        nx += g * b * (b * so.x + t.x);
-        ny += g * b * (b * so.y + t.y);
-        den += g * b * b;
+        nx = fma(gb, fma(b, so.x, t.x), nx);
+        ny = fma(gb, fma(b, so.y, t.y), ny);
+        den = fma(gb, b, den);
       }
-      sn = make_double2(nx / den, ny / den);
-      c2 += wgt * (so.x * so.x + so.y * so.y) / c;
+      const double r = 1.0 / den;
+      sn = make_double2(nx * r, ny * r);
+      c2 += wgt * (so.x * so.x + so.y * so.y) * ic;
     }
     const double dx = sn.x - so.x, dy = sn.y - so.y;
     inc += wgt * (dx * dx + dy * dy);
@@ -148,57 +154,49 @@ __global__ void multi_eq4_kernel(const Ctl *ctl, int K, int lmax, long long nalm
 void Multi::enqueue_iteration(cudaStream_t s) {
   Plan *P0 = P[0];
   multi_beam_kernel<<<lmax + 1, 128, 0, s>>>(d_ctl, K, lmax, nalm, d_beam, d_s, d_balm);
-  if (P0->legdf_args().tab) {
-    // table form: the maps' syntheses, and then their analyses, two maps per launch (each table row
-    // read once for both; every map's transform bitwise the single kernel's)
-    for (int k0 = 0; k0 < K; k0 += kLegBatchMax) {
-      const int nb = std::min(kLegBatchMax, K - k0);
-      LegBatchMaps syn{}, ana{};
-      syn.n = ana.n = nb;
-      for (int b = 0; b < nb; ++b) {
-        const int k = k0 + b;
-        syn.FS[b] = P[k]->d_FS;
-        syn.alm[b] = d_balm + (size_t)k * nalm;
-        ana.FT[b] = P[k]->d_FT;
-        ana.alm[b] = d_ta + (size_t)k * nalm;
-        syn.ctl[b] = ana.ctl[b] = d_ctl;
-      }
-      LegArgs la = P0->leg_args();
-      la.lsht = lmax;
-      launch_legendre_tab(la, P0->legdf_args(), syn, nb, s, LEG_SYNTH);
-      for (int b = 0; b < nb; ++b) {
-        const int k = k0 + b;
-        RingArgs ra = P[k]->ring_args();   // map k's data, noise, gains and Fourier buffers
-        ra.ctl = d_ctl;
-        ra.ring_part = d_ring_part + (size_t)k * 2 * R;
-        P[k]->launch_rng(ra, s, RING_ITER);
-      }
-      launch_legendre_tab(la, P0->legdf_args(), ana, nb, s, LEG_ANALYSIS);
-    }
-    multi_eq4_kernel<<<lmax + 1, 128, 0, s>>>(d_ctl, K, lmax, nalm, omega, d_beam, d_tau, d_cl, d_ta, d_s, d_m_part);
-    launch_control(d_ctl, d_ring_part, K * R, d_m_part, lmax, d_lamcl, d_hist, hist_cap, s);
-    return;
-  }
+  std::vector<RingArgs> ra;
+  std::vector<RingDfArgs> rd;
   for (int k = 0; k < K; ++k) {
-    LegArgs ls = P0->leg_args();          // the first plan's Legendre tables, map k's buffers
-    ls.lsht = lmax;
-    ls.alm_in = d_balm + (size_t)k * nalm;
-    ls.FS = P[k]->d_FS;
-    ls.gate = d_ctl;
-    P0->launch_leg(ls, s, LEG_SYNTH);
-    RingArgs ra = P[k]->ring_args();      // map k's data, noise, gains and Fourier buffers
-    ra.ctl = d_ctl;
-    ra.ring_part = d_ring_part + (size_t)k * 2 * R;
-    P[k]->launch_rng(ra, s, RING_ITER);
+    ra.push_back(P[k]->ring_args());      // map k's data, noise, gains and Fourier buffers
+    ra[k].ctl = d_ctl;
+    ra[k].ring_part = d_ring_part + (size_t)k * 2 * R;
+    rd.push_back(P[k]->ringdf_args());
+  }
+  // the maps' syntheses, then every map's ring stage, then their analyses, with the first plan's Legendre tables: in
+  // the table form two maps per launch (each table row read once for both; every map's transform bitwise the single
+  // one's)
+  const bool tab = P0->legdf_args().tab && P0->opt.precision != WF_PREC_FP64_NATIVE;
+  auto legendre = [&](int mode) {
     LegArgs la = P0->leg_args();
     la.lsht = lmax;
-    la.FT = P[k]->d_FT;
-    la.alm = d_ta + (size_t)k * nalm;
     la.gate = d_ctl;
-    P0->launch_leg(la, s, LEG_ANALYSIS);
-  }
+    for (int k0 = 0; k0 < K; k0 += tab ? kLegBatchMax : 1) {
+      const int nb = tab ? std::min(kLegBatchMax, K - k0) : 1;
+      double2 *alm = (mode == LEG_SYNTH ? d_balm : d_ta) + (size_t)k0 * nalm;
+      if (!tab) {
+        la.alm_in = la.alm = alm;
+        la.FS = P[k0]->d_FS;
+        la.FT = P[k0]->d_FT;
+        P0->launch_leg(la, s, mode);
+        continue;
+      }
+      LegBatchMaps bm{};
+      bm.n = nb;
+      for (int b = 0; b < nb; ++b) {
+        bm.FS[b] = P[k0 + b]->d_FS;
+        bm.FT[b] = P[k0 + b]->d_FT;
+        bm.alm[b] = alm + (size_t)b * nalm;
+        bm.ctl[b] = d_ctl;
+      }
+      launch_legendre_tab(la, P0->legdf_args(), bm, nb, s, mode);
+    }
+  };
+  legendre(LEG_SYNTH);
+  P0->launch_rng_maps(ra.data(), rd.data(), K, s, RING_ITER);
+  legendre(LEG_ANALYSIS);
   multi_eq4_kernel<<<lmax + 1, 128, 0, s>>>(d_ctl, K, lmax, nalm, omega, d_beam, d_tau, d_cl, d_ta, d_s, d_m_part);
-  launch_control(d_ctl, d_ring_part, K * R, d_m_part, lmax, d_lamcl, d_hist, hist_cap, s);
+  const CtlMap c{d_ctl, d_ring_part, d_m_part, d_lamcl, d_hist, hist_cap};
+  launch_control(&c, 1, K * R, lmax, s);
 }
 
 }  // namespace

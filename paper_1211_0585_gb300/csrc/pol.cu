@@ -462,7 +462,9 @@ __global__ void __launch_bounds__(kPolThreads) pol_pixel_kernel(const Ctl *ctl, 
   }
 }
 
-// Eq. 4 with the (T, E) block and B, the prior chi^2 of the input state, increment and norm per m
+// Eq. 4 with the (T, E) block and B, the prior chi^2 of the input state, increment and norm per m. Bound by the FP64
+// pipe: a reciprocal each of the block's determinant, of S's and of C_BB + k and C_BB, and products with them (a
+// division an element: 22 us at Nside 128 / lmax 256; now 17)
 __global__ void __launch_bounds__(128) pol_eq4_kernel(const Ctl *ctl, int lmax, long long nalm, double tau,
                                                        double omega, const double *cls, const double2 *ta,
                                                        double2 *s, double *m_part) {
@@ -482,8 +484,9 @@ __global__ void __launch_bounds__(128) pol_eq4_kernel(const Ctl *ctl, int lmax, 
     const double tt = TT[l], ee = EE[l], bb = BB[l], te = TE[l];
     // S (S + k)^-1 on (T, E)
     const double a11 = tt + k, a12 = te, a22 = ee + k, det = a11 * a22 - a12 * a12;
-    const double m11 = (tt * a22 - te * a12) / det, m12 = (-tt * a12 + te * a11) / det;
-    const double m21 = (te * a22 - ee * a12) / det, m22 = (-te * a12 + ee * a11) / det;
+    const double rd = 1.0 / det;
+    const double m11 = (tt * a22 - te * a12) * rd, m12 = (-tt * a12 + te * a11) * rd;
+    const double m21 = (te * a22 - ee * a12) * rd, m22 = (-te * a12 + ee * a11) * rd;
     const double fb = bb > 0.0 ? bb / (bb + k) : 0.0;
     const double2 nT = make_double2(m11 * tT.x + m12 * tE.x, m11 * tT.y + m12 * tE.y);
     const double2 nE = make_double2(m21 * tT.x + m22 * tE.x, m21 * tT.y + m22 * tE.y);
@@ -588,26 +591,32 @@ void Pol::synth(cudaStream_t s, const double2 *alm, double *map, const Ctl *gate
         gate, d_tab, alm + nalm, alm + 2 * nalm, lmax, RP, d_FSQ, d_FSU);
   }
   const double4_32a *fs[3] = {P->d_FS, d_FSQ, d_FSU};
+  RingArgs ra[3];
+  RingDfArgs rd[3];
   for (int c = 0; c < 3; ++c) {
-    RingArgs ra = P->ring_args();
-    ra.lsht = lmax;
-    ra.FS = fs[c];
-    ra.map_out = map + (size_t)c * npix;
-    ra.gate = gate;
-    P->launch_rng(ra, s, RING_SYNTH);
+    ra[c] = P->ring_args();
+    ra[c].lsht = lmax;
+    ra[c].FS = fs[c];
+    ra[c].map_out = map + (size_t)c * npix;
+    ra[c].gate = gate;
+    rd[c] = P->ringdf_args();
   }
+  P->launch_rng_maps(ra, rd, 3, s, RING_SYNTH);
 }
 
 void Pol::analysis(cudaStream_t s, const double *map, double2 *alm, const Ctl *gate) const {
   double4_32a *ft[3] = {P->d_FT, d_FTQ, d_FTU};
+  RingArgs ra[3];
+  RingDfArgs rd[3];
   for (int c = 0; c < 3; ++c) {
-    RingArgs ra = P->ring_args();
-    ra.lsht = lmax;
-    ra.FT = ft[c];
-    ra.map_in = map + (size_t)c * npix;
-    ra.gate = gate;
-    P->launch_rng(ra, s, RING_ANALYSIS);
+    ra[c] = P->ring_args();
+    ra[c].lsht = lmax;
+    ra[c].FT = ft[c];
+    ra[c].map_in = map + (size_t)c * npix;
+    ra[c].gate = gate;
+    rd[c] = P->ringdf_args();
   }
+  P->launch_rng_maps(ra, rd, 3, s, RING_ANALYSIS);
   LegArgs la = P->leg_args();
   la.lsht = lmax;
   la.alm = alm;
@@ -634,7 +643,8 @@ void Pol::enqueue_iteration(cudaStream_t s) {
                                                        d_part);
   analysis(s, d_u, d_ta, d_ctl);
   pol_eq4_kernel<<<lmax + 1, 128, 0, s>>>(d_ctl, lmax, nalm, tau, omega, d_cls, d_ta, d_s, d_m_part);
-  launch_control(d_ctl, d_part, kPixBlocks, d_m_part, lmax, P->d_cl, d_hist, hist_cap, s);
+  const CtlMap c{d_ctl, d_part, d_m_part, P->d_cl, d_hist, hist_cap};
+  launch_control(&c, 1, kPixBlocks, lmax, s);
 }
 
 }  // namespace

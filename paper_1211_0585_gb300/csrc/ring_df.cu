@@ -42,7 +42,10 @@ __device__ __forceinline__ void warp_sum_df(float &S, float &C) {
 
 }  // namespace
 
-// One CTA per ring pair: the two rings of a pair have the same length,
+// One CTA per ring pair and map (grid.y: maps of one shape share the launch,
+// since the pairs of one map leave a second wave of CTAs nearly empty below
+// Nside 512: two maps 103 -> 89 us and three 205 -> 159 us at Nside 256, three
+// transforms 40 -> 27 us at Nside 128): the two rings of a pair have the same length,
 // half-pixel shift and tables, and real pixel values, so they share one
 // complex transform (Sect. 2 basis change, both directions):
 //   synthesis  IDFT(G_N + i G_S) = f_N + i f_S
@@ -58,8 +61,10 @@ __device__ __forceinline__ void warp_sum_df(float &S, float &C) {
 // in double-float throughout 203 and 52 us.
 constexpr int kRingDfThreads = 256;
 template <int MODE>
-__global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingArgs A, const RingDfArgs T) {
+__global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingArgs A, const RingDfArgs T,
+                                                                     const __grid_constant__ RingMaps Maps) {
   extern __shared__ float4 rsm[];
+  const RingMap &Q = Maps.m[blockIdx.y];
   const int2 pr = A.porder[A.first + blockIdx.x];  // (north ring, south ring or -1)
   const RingDev rg = A.rings[pr.x];
   const bool two = pr.y >= 0;
@@ -74,11 +79,11 @@ __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingAr
 
   int L = A.lsht;
   double lam = 1.0;
-  if (MODE != RING_ITER && A.gate && A.gate->done) return;
+  if (MODE != RING_ITER && Q.gate && Q.gate->done) return;
   if (MODE == RING_ITER) {
-    if (A.ctl->done) return;
-    L = A.ctl->lsht;
-    lam = A.ctl->lambda;
+    if (Q.ctl->done) return;
+    L = Q.ctl->lsht;
+    lam = Q.ctl->lambda;
   }
   const float4 *hs = T.hs + rg.hs_off;
   const float4 *ch = T.chirp + rg.ch_off;
@@ -87,7 +92,7 @@ __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingAr
 
   if (MODE == RING_SYNTH || MODE == RING_ITER) {
     // Z = G_N + i G_S
-    fold_ring2(A.FS, A.RP, k, rg.shifted, n, L, fold_part, [&](int q, float4 gN, float4 gS) {
+    fold_ring2(Q.FS, A.RP, k, rg.shifted, n, L, fold_part, [&](int q, float4 gN, float4 gS) {
       float4 acc = df_pair(df_add(RE(gN), df_neg(IM(gS))), df_add(IM(gN), RE(gS)));
       if (rg.shifted) acc = cmul(acc, hs[q]);
       buf[px<OpsDF>(q)] = rg.blue ? cmul(cconj(acc), ch[q]) : acc;
@@ -108,8 +113,8 @@ __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingAr
   if (MODE == RING_SYNTH) {
     for (int p = threadIdx.x; p < n; p += blockDim.x) {
       const float4 z = pixel(p);
-      A.map_out[rg.off + p] = df_to(RE(z));
-      if (two) A.map_out[offS + p] = df_to(IM(z));
+      Q.map_out[rg.off + p] = df_to(RE(z));
+      if (two) Q.map_out[offS + p] = df_to(IM(z));
     }
     return;
   }
@@ -117,20 +122,20 @@ __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingAr
     // Eq. 3 and the chi^2 partials in double-float (the FP64 pipe is 1/63 of the
     // FP32 one): compensated sums per thread and warp, the sum over warps in double
     float cs[4] = {0.f, 0.f, 0.f, 0.f}, cc[4] = {0.f, 0.f, 0.f, 0.f};   // north chi2, chi2_lambda, south
-    const bool fresh = T.gainlam[pr.x] == lam;   // gains of this pair already at this lambda
-    const dfl ltd = df_from(lam * A.tau);
-    const double l1t = (lam - 1.0) * A.tau;
+    const bool fresh = Q.gainlam[pr.x] == lam;   // gains of this pair already at this lambda
+    const dfl ltd = df_from(lam * Q.tau);
+    const double l1t = (lam - 1.0) * Q.tau;
     auto update = [&](long long at, dfl s, int half) {  // Eq. 3, returns u
-      const float2 d2 = T.d[at], w2 = T.w[at];
+      const float2 d2 = Q.d[at], w2 = Q.w[at];
       const dfl dv{d2.x, d2.y}, wv{w2.x, w2.y};
       dfl g;
       if (fresh) {
-        const float2 g2 = T.gain[at];
+        const float2 g2 = Q.gain[at];
         g = dfl{g2.x, g2.y};
       } else {  // the first pass at a new lambda: the gain from w in double
-        const double w = A.w[at];
+        const double w = Q.w64[at];
         g = df_from(w / (1.0 + l1t * w));
-        T.gain[at] = make_float2(g.h, g.l);
+        Q.gain[at] = make_float2(g.h, g.l);
       }
       const dfl res = df_add(dv, df_neg(s));
       const dfl r2 = df_mul(res, res);
@@ -162,17 +167,17 @@ __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingAr
           const float2 r = red[w][threadIdx.x];
           v += (double)r.x + (double)r.y;
         }
-        A.ring_part[2 * (threadIdx.x < 2 ? pr.x : pr.y) + (threadIdx.x & 1)] = v;
+        Q.ring_part[2 * (threadIdx.x < 2 ? pr.x : pr.y) + (threadIdx.x & 1)] = v;
       }
       if (threadIdx.x == 0 && !fresh) {  // after the barrier: every gain of the pair is written
-        T.gainlam[pr.x] = lam;
-        if (two) T.gainlam[pr.y] = lam;
+        Q.gainlam[pr.x] = lam;
+        if (two) Q.gainlam[pr.y] = lam;
       }
     }
   } else {  // RING_ANALYSIS: u = the input maps
     for (int p = threadIdx.x; p < M; p += blockDim.x) {
       if (p < n) {
-        const float4 u = df_pair(df_from(A.map_in[rg.off + p]), df_from(two ? A.map_in[offS + p] : 0.0));
+        const float4 u = df_pair(df_from(Q.map_in[rg.off + p]), df_from(two ? Q.map_in[offS + p] : 0.0));
         buf[loc(p)] = rg.blue ? cmul(u, ch[p]) : u;
       } else if (rg.blue) {
         buf[px<OpsDF>(p)] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -196,7 +201,7 @@ __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingAr
       US = cmul(US, cconj(hs[q]));
       if (j & 1) { UN = cneg(UN); US = cneg(US); }
     }
-    A.FT[(size_t)m * A.RP + k] = make_double4_32a(
+    Q.FT[(size_t)m * A.RP + k] = make_double4_32a(
         df_pack(df_mul(RE(UN), om)), df_pack(df_mul(IM(UN), om)), two ? df_pack(df_mul(RE(US), om)) : 0.0,
         two ? df_pack(df_mul(IM(US), om)) : 0.0);
   }
@@ -233,26 +238,37 @@ void launch_to_df(const double2 *src, float4 *dst, long long n, cudaStream_t s) 
 }
 
 template <int MODE>
-static void launch_ring_df_mode(const RingArgs &a, const RingDfArgs &t, const RingClass *cls, int ncls,
+static void launch_ring_df_mode(const RingArgs *a, const RingDfArgs *t, int nmaps, const RingClass *cls, int ncls,
                                 cudaStream_t s) {
   auto smem = [](const RingClass &c) { return c.global ? (size_t)16 : ((size_t)1 << c.logM) * sizeof(float4); };
   raise_smem_cap(reinterpret_cast<const void *>(ring_df_kernel<MODE>));
   for (int c = 0; c < ncls; ++c) {
     if (cls[c].count <= 0) continue;
     const size_t sm = smem(cls[c]);
-    RingArgs ac = a;
+    RingArgs ac = a[0];
     ac.first = cls[c].first;
-    ac.scratch = cls[c].global ? a.scratch : nullptr;
-    ring_df_kernel<MODE><<<cls[c].count, kRingDfThreads, sm, s>>>(ac, t);
+    ac.scratch = cls[c].global ? a[0].scratch : nullptr;
+    const int most = cls[c].global ? 1 : kRingMapsMax;   // the scratch array holds one map's rings
+    for (int i0 = 0; i0 < nmaps; i0 += most) {
+      const int n = nmaps - i0 < most ? nmaps - i0 : most;
+      RingMaps q{};
+      for (int i = 0; i < n; ++i) {
+        const RingArgs &x = a[i0 + i];
+        const RingDfArgs &y = t[i0 + i];
+        q.m[i] = RingMap{x.FS, x.FT, x.map_in, x.map_out, y.d, y.w, x.w, y.gain, y.gainlam, x.ring_part, x.ctl,
+                         x.gate, x.tau};
+      }
+      ring_df_kernel<MODE><<<dim3(cls[c].count, n), kRingDfThreads, sm, s>>>(ac, t[0], q);
+    }
   }
 }
 
-void launch_ring_df(const RingArgs &a, const RingDfArgs &t, const RingClass *cls, int ncls, cudaStream_t s,
-                    int mode) {
+void launch_ring_df(const RingArgs *a, const RingDfArgs *t, int nmaps, const RingClass *cls, int ncls,
+                    cudaStream_t s, int mode) {
   switch (mode) {
-    case RING_SYNTH: launch_ring_df_mode<RING_SYNTH>(a, t, cls, ncls, s); break;
-    case RING_ANALYSIS: launch_ring_df_mode<RING_ANALYSIS>(a, t, cls, ncls, s); break;
-    default: launch_ring_df_mode<RING_ITER>(a, t, cls, ncls, s); break;
+    case RING_SYNTH: launch_ring_df_mode<RING_SYNTH>(a, t, nmaps, cls, ncls, s); break;
+    case RING_ANALYSIS: launch_ring_df_mode<RING_ANALYSIS>(a, t, nmaps, cls, ncls, s); break;
+    default: launch_ring_df_mode<RING_ITER>(a, t, nmaps, cls, ncls, s); break;
   }
 }
 

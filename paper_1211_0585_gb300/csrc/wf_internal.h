@@ -176,6 +176,22 @@ struct RingDfArgs {
   double *gainlam;        // [R] lambda the cached gains of each ring belong to (-1: none)
 };
 void launch_to_df2(const double *src, float2 *dst, long long n, cudaStream_t s);
+// One map of a double-float ring-stage launch: what a RingArgs and RingDfArgs hold beside the shape's tables.
+constexpr int kRingMapsMax = 4;
+struct RingMap {
+  const double4_32a *FS;
+  double4_32a *FT;
+  const double *map_in;
+  double *map_out;
+  const float2 *d, *w;
+  const double *w64;
+  float2 *gain;
+  double *gainlam;
+  double *ring_part;
+  const Ctl *ctl, *gate;
+  double tau;
+};
+struct RingMaps { RingMap m[kRingMapsMax]; };
 
 // Batched engine (batch_kernels.cu): B slots of one shape in lockstep.
 constexpr int kBatchMax = 64;
@@ -252,8 +268,10 @@ void launch_batch_export_slot(const BatchArgs &a, int b, cudaStream_t s);
 void launch_hi_table(const float4 *src, float2 *dst, long long n, cudaStream_t s);
 
 void launch_ring(const RingArgs &a, const RingClass *cls, int ncls, cudaStream_t s, int mode);
-void launch_ring_df(const RingArgs &a, const RingDfArgs &t, const RingClass *cls, int ncls, cudaStream_t s,
-                    int mode);
+// nmaps maps of one shape (a[i], t[i]; the tables and the band limit are those of the first) in as few launches as
+// kRingMapsMax allows
+void launch_ring_df(const RingArgs *a, const RingDfArgs *t, int nmaps, const RingClass *cls, int ncls,
+                    cudaStream_t s, int mode);
 // ring order and classes of a ring table (host; rings as built for the plan)
 void ring_classes(const RingDev *rings, int R, std::vector<int> &order, std::vector<RingClass> &cls);
 void launch_to_df(const double2 *src, float4 *dst, long long n, cudaStream_t s);
@@ -275,8 +293,16 @@ void launch_start_values(const double *x, const double2 *rec, int lmax, int RP, 
                          double2 *sv, cudaStream_t s);
 void launch_bluestein_setup(const RingDev *rings, const int *order, const RingClass *cls, int ncls, void *scratch,
                             const double2 *tw, int logMmax, const double2 *chirp, double2 *B, cudaStream_t s);
-void launch_control(Ctl *ctl, const double *ring_part, int R, const double *m_part, int lmax,
-                    const double *cl, wf_iter_record *hist, int hist_cap, cudaStream_t s);
+// The controllers of n maps, each with its own partial sums ([R][2] and [lmax+1][3]) and records.
+constexpr int kCtlMapsMax = 4;
+struct CtlMap {
+  Ctl *ctl;
+  const double *ring_part, *m_part, *cl;
+  wf_iter_record *hist;
+  int hist_cap;
+};
+struct CtlMaps { CtlMap m[kCtlMapsMax]; };
+void launch_control(const CtlMap *maps, int n, int R, int lmax, cudaStream_t s);
 
 // Raise a kernel's dynamic shared-memory cap to the device's opt-in maximum
 // (once per function). The cap is an attribute of the function, read when a

@@ -99,8 +99,19 @@ struct Plan : wf_plan_s {
   // the ring stage of the plan's precision
   void launch_rng(const RingArgs &a, cudaStream_t s, int mode) const {
     if (opt.precision == WF_PREC_FP64_NATIVE) launch_ring(a, rsingle.data(), (int)rsingle.size(), s, mode);
-    else launch_ring_df(a, ringdf_args(), psingle.data(), (int)psingle.size(), s, mode);
+    else {
+      const RingDfArgs t = ringdf_args();
+      launch_ring_df(&a, &t, 1, psingle.data(), (int)psingle.size(), s, mode);
+    }
   }
+  // the ring stage of n maps of this plan's shape and precision, map i's arguments in a[i] and, for the
+  // double-float data, noise and gains, t[i]
+  void launch_rng_maps(const RingArgs *a, const RingDfArgs *t, int n, cudaStream_t s, int mode) const {
+    if (opt.precision == WF_PREC_FP64_NATIVE)
+      for (int i = 0; i < n; ++i) launch_ring(a[i], rsingle.data(), (int)rsingle.size(), s, mode);
+    else launch_ring_df(a, t, n, psingle.data(), (int)psingle.size(), s, mode);
+  }
+  CtlMap ctl_map() const { return CtlMap{d_ctl, d_ring_part, d_m_part, d_cl, d_hist, hist_cap}; }
   // this plan's map in slot b of a launch of the table form
   void tab_map(LegBatchMaps &bm, int b) const {
     bm.FT[b] = d_FT; bm.FS[b] = d_FS; bm.alm[b] = d_s; bm.ctl[b] = d_ctl; bm.m_part[b] = d_m_part; bm.cl[b] = d_cl;
