@@ -91,7 +91,7 @@ Engine::~Engine() {
 BatchArgs Engine::args() const {
   BatchArgs a{};
   a.rings = geo->d_rings;
-  a.order = geo->d_order;
+  a.porder = geo->d_porder;
   a.first = 0;
   a.twf = geo->d_twf; a.hsf = geo->d_hsf; a.chf = geo->d_chf; a.Bf = geo->d_Bf;
   a.tw2 = tw2; a.Bf2 = Bf2;
@@ -198,7 +198,7 @@ wf_status Engine::create(Plan *shape_plan, int nslots, cudaStream_t s_, int max_
       (st = dalloc((void **)&tstiles, sizeof(int2) * syn.size())) ||
       (st = dalloc((void **)&offTc, sizeof(int) * off.size())) || (st = dalloc((void **)&err, sizeof(int))) ||
       (st = dalloc((void **)&alm_of_row, sizeof(int) * nalm)) ||
-      (st = dalloc((void **)&tw2, sizeof(float2) * std::max<long long>(geo->n_tw, 1))) ||
+      (st = dalloc((void **)&tw2, sizeof(float2) * twiddles_f32(geo->logMmax))) ||
       (st = dalloc((void **)&Bf2, sizeof(float2) * std::max<long long>(geo->n_B, 1))) ||
       (st = dalloc((void **)&FS, sizeof(float4) * nF * B)) || (st = dalloc((void **)&FT, sizeof(float4) * nF * B)) ||
       (st = dalloc((void **)&d, sizeof(double) * npix)) || (st = dalloc((void **)&w, sizeof(double) * npix)) ||
@@ -240,7 +240,7 @@ wf_status Engine::create(Plan *shape_plan, int nslots, cudaStream_t s_, int max_
     ENG_CUDA(cudaMemcpyAsync(alm_of_row, a_of_r.data(), sizeof(int) * nalm, cudaMemcpyHostToDevice, stream));
     ENG_CUDA(cudaStreamSynchronize(stream));   // a_of_r and cinfo are released by then
   }
-  launch_hi_table(geo->d_twf, tw2, geo->n_tw, stream);
+  launch_pack_twiddles(geo->d_tw, geo->logMmax, nullptr, tw2, stream);
   launch_hi_table(geo->d_Bf, Bf2, geo->n_B, stream);
   ENG_CUDA(cudaMemsetAsync(SPT, 0, sizeof(float) * nSPT, stream));
   ENG_CUDA(cudaMemsetAsync(dw32, 0, sizeof(float2) * npix * B, stream));
@@ -263,7 +263,7 @@ wf_status Engine::create(Plan *shape_plan, int nslots, cudaStream_t s_, int max_
 }
 
 wf_status Engine::autotune() {
-  const int ncls = (int)geo->rclass.size();
+  const int ncls = (int)geo->pclass.size();
   ring_groups.assign(ncls, 0);
   // every slot active on a full-band step (the data are zero)
   const Ctl c = geo->make_ctl(1, 1.0, geo->lmax, 0);
@@ -276,7 +276,7 @@ wf_status Engine::autotune() {
   ENG_CUDA(cudaEventCreate(&e1));
   const BatchArgs a = args();
   for (int k = 0; k < ncls; ++k) {
-    const RingClass &rc = geo->rclass[k];
+    const RingClass &rc = geo->pclass[k];
     float best = 0.f;
     for (int G = 2; G <= 8; G *= 2) {
       if (!batch_ring_group_ok(rc.logM, G)) continue;
@@ -362,7 +362,7 @@ wf_status Engine::step() {
     cudaGraph_t g;
     ENG_CUDA(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
     for (int i = 0; i < graph_iters; ++i)
-      launch_batch_iteration(args(), tc_args(), maps, geo->rclass.data(), (int)geo->rclass.size(),
+      launch_batch_iteration(args(), tc_args(), maps, geo->pclass.data(), (int)geo->pclass.size(),
                              ring_groups.empty() ? nullptr : ring_groups.data(), bstate, stream, bands.data(),
                              (int)bands.size());
     ENG_CUDA(cudaStreamEndCapture(stream, &g));

@@ -38,45 +38,58 @@ __device__ __forceinline__ void prefetch_l2(const void *p) {
 }  // namespace
 
 // ---------------------------------------------------------------- ring stage
-// One CTA per (ring, group of G slots). The ring values of every slot are
-// real, so two slots a, b share one complex FFT: the inverse transform of
-// Z = G_a + i G_b gives f_a + i f_b, and the forward transform of u_a + i u_b
+// One CTA per (ring pair, group of G slots), ND = 2. The ring values of every
+// slot are real, so two slots a, b share one complex FFT: the inverse transform
+// of Z = G_a + i G_b gives f_a + i f_b, and the forward transform of u_a + i u_b
 // gives Z with U_a = (Z_q + conj Z_{n-q}) / 2 and U_b = (Z_q - conj Z_{n-q}) / 2i.
-// The G / 2 packed arrays share every twiddle load, the pixel pass updates
-// them in place (the inverse transform's output order is the forward
-// transform's input order), and the G slots read their Fourier coefficients
-// as one contiguous run of G float4. Four CTAs of 256 threads per SM (64
-// registers), so that the FFT passes of one CTA overlap the global loads and
-// stores of the others.
+// The two rings of a pair have the same length, half-pixel shift and tables and
+// lie side by side in every Fourier record (north re, im, south re, im), so a
+// CTA takes both: each record is read and written whole. (A CTA per ring read
+// every record twice and wrote it in 8-byte halves: 3.65 ms an iteration at
+// Nside 512 / 64 slots, now 2.83 with the twiddles laid out by stage, fft.cuh;
+// the load and store pipe, 77 % busy at Nside 256, bounds the long rings.) The arrays share every twiddle load, the pixel
+// pass updates them in place (the inverse transform's output order is the
+// forward transform's input order), and the G slots read their Fourier
+// coefficients as one contiguous run of G float4. Four CTAs of 256 threads per
+// SM (64 registers), so that the FFT passes of one CTA overlap the global loads
+// and stores of the others. ND = 1, a CTA per ring, serves the rings whose two
+// FFT buffers do not fit shared memory (Nside 2048).
 constexpr int kBringThreads = 256;
-template <int G>
+template <int G, int ND>
 __global__ void __launch_bounds__(kBringThreads, 4) bring_kernel(const BatchArgs A) {
   static_assert(G % 2 == 0, "slots are packed in pairs");
   constexpr int P = G / 2;
   extern __shared__ float2 bsm[];
-  const int r = A.order[A.first + blockIdx.x], b0 = blockIdx.y * G;
+  const int2 pr = A.porder[A.first + (ND == 2 ? blockIdx.x : blockIdx.x >> 1)];   // (north ring, south ring or -1)
+  const int side0 = ND == 2 ? 0 : blockIdx.x & 1;   // the first side (ND = 1: the only one)
+  if (ND == 1 && side0 && pr.y < 0) return;
+  const int b0 = blockIdx.y * G;
   const int B = A.B;
   // slots of this group that iterate (the group's live mask is uniform per CTA)
   bool on[G];
-  bool any = false;
+  unsigned onm = 0;                                 // the same as a mask, for indexes known at run time only
 #pragma unroll
   for (int g = 0; g < G; ++g) {
     const int b = b0 + g;
     on[g] = b < B && A.active[b] && !A.ctl[b].done;
-    any |= on[g];
+    onm |= on[g] ? 1u << g : 0u;
   }
-  if (!any) return;
-  const RingDev rg = A.rings[r];
+  if (!onm) return;
+  const RingDev rg = A.rings[side0 ? pr.y : pr.x];
+  const int nd = ND == 2 && pr.y < 0 ? 1 : ND;      // sides with a ring (the equator pair has one)
+  long long off[ND];
+  off[0] = rg.off;
+  if (ND == 2) off[ND - 1] = nd == 2 ? A.rings[pr.y].off : 0;
   const int n = rg.n, M = 1 << rg.logM;
-  float2 *buf = bsm;                                          // [P][M] (swizzled, px)
-  // alias partial sums of rings shorter than the block: [kBringThreads][G] after
+  float2 *buf = bsm;                                          // [ND][P][M] (swizzled, px)
+  // alias partial sums of rings shorter than the block: [kBringThreads][ND][G] after
   // the FFT buffers (present in the classes whose rings can be that short)
-  float2(*fpart)[G] = reinterpret_cast<float2(*)[G]>(bsm + P * M);
-  __shared__ double red[kBringThreads / 32][2 * G];
+  float2(*fpart)[ND][G] = reinterpret_cast<float2(*)[ND][G]>(bsm + ND * P * M);
+  __shared__ double red[kBringThreads / 32][2 * ND * G];
   const float4 *hs = A.hsf + rg.hs_off;
   const float4 *ch = A.chf + rg.ch_off;
   const float2 *Bf = A.Bf2 + rg.B_off;
-  const int k = rg.pair, slot = rg.side;
+  const int k = rg.pair;
   int Lg[G];
   float lt[G], l1t[G];
 #pragma unroll
@@ -95,33 +108,41 @@ __global__ void __launch_bounds__(kBringThreads, 4) bring_kernel(const BatchArgs
   for (int g = 0; g < G; ++g) Lmax = max(Lmax, Lg[g]);
   // Every global line this CTA reads goes to L2 first, all requests at once:
   // the Fourier coefficients of the G slots (one run of G float4 per m) and
-  // the slots' (d, w) on the ring. The fold's and the pixel pass's loads then
+  // the slots' (d, w) on the rings. The fold's and the pixel pass's loads then
   // wait on L2, not on HBM, one after another.
   for (int m = threadIdx.x; m <= Lmax; m += blockDim.x) prefetch_l2(A.FS + ((size_t)m * A.RP + k) * B + b0);
   {
     constexpr int kLine = 128 / sizeof(float2);   // pixels per line
     const int nl = (n + kLine - 1) / kLine + 1;     // the ring's run may straddle one more line
-    for (int e = threadIdx.x; e < G * nl; e += blockDim.x) {
-      const int g = e / nl, li = e % nl;
-      if (on[g]) prefetch_l2(A.dw32 + (size_t)(b0 + g) * A.npix + rg.off + min(li * kLine, n - 1));
+    for (int e = threadIdx.x; e < nd * G * nl; e += blockDim.x) {
+      const int h = e / (G * nl), g = (e / nl) % G, li = e % nl;
+      if (onm >> g & 1) prefetch_l2(A.dw32 + (size_t)(b0 + g) * A.npix + (h ? off[ND - 1] : off[0]) + min(li * kLine, n - 1));
     }
   }
 
   // fold F_m onto residues q for the G slots (m-aliasing), packed in pairs;
   // on rings shorter than the block each residue's alias series is split over
   // several threads (partial sums added in a fixed order)
-  auto alias_sum = [&](int q, int j0, int dj, float2 (&acc)[G]) {
+  auto side_of = [&](const float4 &f4, int h) {
+    return (ND == 2 ? h : side0) ? make_float2(f4.z, f4.w) : make_float2(f4.x, f4.y);
+  };
+  auto alias_sum = [&](int q, int j0, int dj, float2 (&acc)[ND][G]) {
 #pragma unroll
-    for (int g = 0; g < G; ++g) acc[g] = make_float2(0.f, 0.f);
+    for (int h = 0; h < ND; ++h)
+#pragma unroll
+      for (int g = 0; g < G; ++g) acc[h][g] = make_float2(0.f, 0.f);
     for (int j = j0, m = q + n * j0; m <= Lmax; j += dj, m += n * dj) {
       const float4 *src = A.FS + ((size_t)m * A.RP + k) * B + b0;
 #pragma unroll
       for (int g = 0; g < G; ++g) {
         if (m > Lg[g]) continue;
         const float4 f4 = __ldg(src + g);
-        float2 f = slot ? make_float2(f4.z, f4.w) : make_float2(f4.x, f4.y);
-        if (rg.shifted && (j & 1)) { f.x = -f.x; f.y = -f.y; }
-        acc[g] = f2add(acc[g], f);
+#pragma unroll
+        for (int h = 0; h < ND; ++h) {
+          float2 f = side_of(f4, h);
+          if (rg.shifted && (j & 1)) { f.x = -f.x; f.y = -f.y; }
+          acc[h][g] = f2add(acc[h][g], f);
+        }
       }
     }
     for (int j = 1 + j0, m = n * (1 + j0) - q; m <= Lmax; j += dj, m += n * dj) {
@@ -130,71 +151,88 @@ __global__ void __launch_bounds__(kBringThreads, 4) bring_kernel(const BatchArgs
       for (int g = 0; g < G; ++g) {
         if (m > Lg[g]) continue;
         const float4 f4 = __ldg(src + g);
-        float2 f = slot ? make_float2(f4.z, -f4.w) : make_float2(f4.x, -f4.y);
-        if (rg.shifted && (j & 1)) { f.x = -f.x; f.y = -f.y; }
-        acc[g] = f2add(acc[g], f);
+#pragma unroll
+        for (int h = 0; h < ND; ++h) {
+          float2 f = f2conj(side_of(f4, h));
+          if (rg.shifted && (j & 1)) { f.x = -f.x; f.y = -f.y; }
+          acc[h][g] = f2add(acc[h][g], f);
+        }
       }
     }
   };
-  auto store_residue = [&](int q, const float2 (&acc)[G]) {
+  auto store_residue = [&](int q, const float2 (&acc)[ND][G]) {
     const float2 h = rg.shifted ? hi2(hs[q]) : make_float2(0.f, 0.f), cq = rg.blue ? hi2(ch[q]) : make_float2(0.f, 0.f);
+    const int at = px<OpsF32>(q);
 #pragma unroll
-    for (int pp = 0; pp < P; ++pp) {
-      float2 va = acc[2 * pp], vb = acc[2 * pp + 1];
-      if (rg.shifted) { va = f2mul(va, h); vb = f2mul(vb, h); }
-      const float2 z = make_float2(va.x - vb.y, va.y + vb.x);    // G_a + i G_b
-      buf[pp * M + px<OpsF32>(q)] = rg.blue ? f2mul(f2conj(z), cq) : z;
-    }
+    for (int sd = 0; sd < ND; ++sd)
+#pragma unroll
+      for (int pp = 0; pp < P; ++pp) {
+        float2 va = acc[sd][2 * pp], vb = acc[sd][2 * pp + 1];
+        if (rg.shifted) { va = f2mul(va, h); vb = f2mul(vb, h); }
+        const float2 z = make_float2(va.x - vb.y, va.y + vb.x);    // G_a + i G_b
+        buf[(sd * P + pp) * M + at] = rg.blue ? f2mul(f2conj(z), cq) : z;
+      }
   };
   if (n >= kBringThreads) {
     for (int q = threadIdx.x; q < n; q += blockDim.x) {
-      float2 acc[G];
+      float2 acc[ND][G];
       alias_sum(q, 0, 1, acc);
       store_residue(q, acc);
     }
   } else {
     const int nj = kBringThreads / n, t = threadIdx.x;
     if (t < n * nj) {
-      float2 acc[G];
+      float2 acc[ND][G];
       alias_sum(t % n, t / n, nj, acc);
 #pragma unroll
-      for (int g = 0; g < G; ++g) fpart[t][g] = acc[g];
+      for (int h = 0; h < ND; ++h)
+#pragma unroll
+        for (int g = 0; g < G; ++g) fpart[t][h][g] = acc[h][g];
     }
     __syncthreads();
     if (t < n) {
-      float2 acc[G];
+      float2 acc[ND][G];
 #pragma unroll
-      for (int g = 0; g < G; ++g) acc[g] = make_float2(0.f, 0.f);
+      for (int h = 0; h < ND; ++h)
+#pragma unroll
+        for (int g = 0; g < G; ++g) acc[h][g] = make_float2(0.f, 0.f);
       for (int jg = 0; jg < nj; ++jg)
 #pragma unroll
-        for (int g = 0; g < G; ++g) acc[g] = f2add(acc[g], fpart[jg * n + t][g]);
+        for (int h = 0; h < ND; ++h)
+#pragma unroll
+          for (int g = 0; g < G; ++g) acc[h][g] = f2add(acc[h][g], fpart[jg * n + t][h][g]);
       store_residue(t, acc);
     }
   }
   if (rg.blue)
     for (int q = n + threadIdx.x; q < M; q += blockDim.x)
 #pragma unroll
-      for (int pp = 0; pp < P; ++pp) buf[pp * M + px<OpsF32>(q)] = make_float2(0.f, 0.f);
+      for (int pp = 0; pp < ND * P; ++pp) buf[pp * M + px<OpsF32>(q)] = make_float2(0.f, 0.f);
   __syncthreads();
-  if (rg.blue) bluestein4<OpsF32, P>(buf, M, M, rg.logM, Bf, A.tw2, A.logMmax);
-  else fft_dif4<OpsF32, P>(buf, M, M, rg.logM, +1, A.tw2, A.logMmax);
+  if (rg.blue) bluestein4<OpsF32, ND * P>(buf, M, M, rg.logM, Bf, A.tw2, A.logMmax);
+  else fft_dif4<OpsF32, ND * P>(buf, M, M, rg.logM, +1, A.tw2, A.logMmax);
 
   // Eq. 3 per pixel (in place: s_a + i s_b -> u_a + i u_b) and the chi^2
   // partials in FP32 (per-thread sums, warp sums by shuffles), the sum over
   // warps in double
-  float c2n[G], c2l[G];
+  float c2n[ND][G], c2l[ND][G];
 #pragma unroll
-  for (int g = 0; g < G; ++g) { c2n[g] = 0.f; c2l[g] = 0.f; }
+  for (int h = 0; h < ND; ++h)
+#pragma unroll
+    for (int g = 0; g < G; ++g) { c2n[h][g] = 0.f; c2l[h][g] = 0.f; }
   // kPix pixels per thread at a time: their (d, w) loads are issued together
-  constexpr int kPix = G <= 2 ? 8 : 16 / G;
+  constexpr int kPix = ND * G <= 2 ? 8 : ND * G >= 16 ? 1 : 16 / (ND * G);
   for (int p0 = threadIdx.x; p0 < n; p0 += kPix * blockDim.x) {
-    float2 dw[kPix][G];
+    float2 dw[kPix][ND][G];
 #pragma unroll
     for (int k = 0; k < kPix; ++k) {
       const int p = p0 + k * blockDim.x;
 #pragma unroll
-      for (int g = 0; g < G; ++g)
-        dw[k][g] = (p < n && on[g]) ? __ldg(A.dw32 + (size_t)(b0 + g) * A.npix + rg.off + p) : make_float2(0.f, 0.f);
+      for (int h = 0; h < ND; ++h)
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+          dw[k][h][g] = (p < n && on[g] && h < nd) ? __ldg(A.dw32 + (size_t)(b0 + g) * A.npix + off[h] + p)
+                                                   : make_float2(0.f, 0.f);
     }
 #pragma unroll
     for (int k = 0; k < kPix; ++k) {
@@ -203,60 +241,70 @@ __global__ void __launch_bounds__(kBringThreads, 4) bring_kernel(const BatchArgs
       const float2 cp = rg.blue ? hi2(ch[p]) : make_float2(0.f, 0.f);
       const int br = px<OpsF32>(rg.blue ? p : digitrev(p, rg.logM));
 #pragma unroll
-      for (int pp = 0; pp < P; ++pp) {
-        const float2 z = buf[pp * M + br];
-        float sv[2];
-        if (rg.blue) {   // the inverse DFT came out conjugated (conj of the DFT of conj Z)
-          const float2 R = f2mul(cp, z);
-          sv[0] = R.x; sv[1] = -R.y;
-        } else {
-          sv[0] = z.x; sv[1] = z.y;
-        }
-        float u[2];
+      for (int h = 0; h < ND; ++h)
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const int g = 2 * pp + e;
-          u[e] = 0.f;
-          if (!on[g]) continue;
-          const float wp = dw[k][g].y;
-          const float res = dw[k][g].x - sv[e];
-          const float gg = __fdividef(wp, fmaf(l1t[g], wp, 1.f));
-          c2n[g] = fmaf(wp * res, res, c2n[g]);
-          c2l[g] = fmaf(gg * res, res, c2l[g]);
-          u[e] = lt[g] * gg * res;
+        for (int pp = 0; pp < P; ++pp) {
+          const float2 z = buf[(h * P + pp) * M + br];
+          float sv[2];
+          if (rg.blue) {   // the inverse DFT came out conjugated (conj of the DFT of conj Z)
+            const float2 R = f2mul(cp, z);
+            sv[0] = R.x; sv[1] = -R.y;
+          } else {
+            sv[0] = z.x; sv[1] = z.y;
+          }
+          float u[2];
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const int g = 2 * pp + e;
+            u[e] = 0.f;
+            if (!on[g]) continue;
+            const float wp = dw[k][h][g].y;
+            const float res = dw[k][h][g].x - sv[e];
+            const float gg = __fdividef(wp, fmaf(l1t[g], wp, 1.f));
+            c2n[h][g] = fmaf(wp * res, res, c2n[h][g]);
+            c2l[h][g] = fmaf(gg * res, res, c2l[h][g]);
+            u[e] = lt[g] * gg * res;
+          }
+          const float2 uz = make_float2(u[0], u[1]);
+          buf[(h * P + pp) * M + br] = rg.blue ? f2mul(uz, cp) : uz;
         }
-        const float2 uz = make_float2(u[0], u[1]);
-        buf[pp * M + br] = rg.blue ? f2mul(uz, cp) : uz;
-      }
     }
   }
   if (rg.blue)
     for (int p = n + threadIdx.x; p < M; p += blockDim.x)
 #pragma unroll
-      for (int pp = 0; pp < P; ++pp) buf[pp * M + px<OpsF32>(p)] = make_float2(0.f, 0.f);
+      for (int pp = 0; pp < ND * P; ++pp) buf[pp * M + px<OpsF32>(p)] = make_float2(0.f, 0.f);
   {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-      float a = c2n[g], bsum = c2l[g];   // warp sums in FP32, the per-warp partials in double
-      for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        bsum += __shfl_xor_sync(0xffffffffu, bsum, o);
+    for (int h = 0; h < ND; ++h)
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        float a = c2n[h][g], bsum = c2l[h][g];   // warp sums in FP32, the per-warp partials in double
+        for (int o = 16; o > 0; o >>= 1) {
+          a += __shfl_xor_sync(0xffffffffu, a, o);
+          bsum += __shfl_xor_sync(0xffffffffu, bsum, o);
+        }
+        if (lane == 0) { red[warp][2 * (h * G + g)] = a; red[warp][2 * (h * G + g) + 1] = bsum; }
       }
-      if (lane == 0) { red[warp][2 * g] = a; red[warp][2 * g + 1] = bsum; }
-    }
     __syncthreads();   // also orders the pixel pass before the forward transform
-    if (threadIdx.x < G && on[threadIdx.x]) {
-      const int g = threadIdx.x;
-      double sa = 0.0, sb = 0.0;
-      for (int w2 = 0; w2 < kBringThreads / 32; ++w2) { sa += red[w2][2 * g]; sb += red[w2][2 * g + 1]; }
-      A.ring_part[((size_t)(b0 + g) * A.R + r) * 2] = sa;
-      A.ring_part[((size_t)(b0 + g) * A.R + r) * 2 + 1] = sb;
+    if (threadIdx.x < nd * G) {
+      const int h = threadIdx.x / G, g = threadIdx.x % G;
+      if (onm >> g & 1) {
+        double sa = 0.0, sb = 0.0;
+        for (int w2 = 0; w2 < kBringThreads / 32; ++w2) {
+          sa += red[w2][2 * threadIdx.x];
+          sb += red[w2][2 * threadIdx.x + 1];
+        }
+        const int r = (ND == 2 ? h : side0) ? pr.y : pr.x;
+        A.ring_part[((size_t)(b0 + g) * A.R + r) * 2] = sa;
+        A.ring_part[((size_t)(b0 + g) * A.R + r) * 2 + 1] = sb;
+      }
     }
   }
   // forward DFT of u_a + i u_b
-  if (rg.blue) bluestein4<OpsF32, P>(buf, M, M, rg.logM, Bf, A.tw2, A.logMmax);
-  else fft_dit4<OpsF32, P>(buf, M, M, rg.logM, -1, A.tw2, A.logMmax);
+  if (rg.blue) bluestein4<OpsF32, ND * P>(buf, M, M, rg.logM, Bf, A.tw2, A.logMmax);
+  else fft_dit4<OpsF32, ND * P>(buf, M, M, rg.logM, -1, A.tw2, A.logMmax);
   // unpack U_a, U_b and unfold to m = 0 .. Lmax
   const float om = (float)A.omega;
   for (int m = threadIdx.x; m <= Lmax; m += blockDim.x) {
@@ -265,23 +313,33 @@ __global__ void __launch_bounds__(kBringThreads, 4) bring_kernel(const BatchArgs
     const float2 cq2 = rg.blue ? hi2(ch[q2]) : make_float2(0.f, 0.f);
     const float2 hq = f2conj(hi2(hs[q]));
     float4 *dst4 = A.FT + ((size_t)m * A.RP + k) * B + b0;
+    const int at1 = px<OpsF32>(q), at2 = px<OpsF32>(q2);
 #pragma unroll
     for (int pp = 0; pp < P; ++pp) {
-      float2 Z1 = buf[pp * M + px<OpsF32>(q)], Z2 = buf[pp * M + px<OpsF32>(q2)];
-      if (rg.blue) { Z1 = f2mul(cq, Z1); Z2 = f2mul(cq2, Z2); }
-      float2 U[2];
-      U[0] = make_float2(0.5f * (Z1.x + Z2.x), 0.5f * (Z1.y - Z2.y));   // (Z_q + conj Z_{n-q}) / 2
-      U[1] = make_float2(0.5f * (Z1.y + Z2.y), 0.5f * (Z2.x - Z1.x));   // (Z_q - conj Z_{n-q}) / 2i
+      float2 out[ND][2];
+#pragma unroll
+      for (int h = 0; h < ND; ++h) {
+        float2 Z1 = buf[(h * P + pp) * M + at1], Z2 = buf[(h * P + pp) * M + at2];
+        if (rg.blue) { Z1 = f2mul(cq, Z1); Z2 = f2mul(cq2, Z2); }
+        float2 U[2];
+        U[0] = make_float2(0.5f * (Z1.x + Z2.x), 0.5f * (Z1.y - Z2.y));   // (Z_q + conj Z_{n-q}) / 2
+        U[1] = make_float2(0.5f * (Z1.y + Z2.y), 0.5f * (Z2.x - Z1.x));   // (Z_q - conj Z_{n-q}) / 2i
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          float2 V = U[e];
+          if (rg.shifted) {
+            V = f2mul(V, hq);
+            if (j & 1) { V.x = -V.x; V.y = -V.y; }
+          }
+          out[h][e] = h < nd ? make_float2(om * V.x, om * V.y) : make_float2(0.f, 0.f);
+        }
+      }
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         const int g = 2 * pp + e;
         if (m > Lg[g]) continue;
-        float2 V = U[e];
-        if (rg.shifted) {
-          V = f2mul(V, hq);
-          if (j & 1) { V.x = -V.x; V.y = -V.y; }
-        }
-        reinterpret_cast<float2 *>(dst4 + g)[slot] = make_float2(om * V.x, om * V.y);
+        if (ND == 2) dst4[g] = make_float4(out[0][e].x, out[0][e].y, out[ND - 1][e].x, out[ND - 1][e].y);
+        else reinterpret_cast<float2 *>(dst4 + g)[side0] = out[0][e];
       }
     }
   }
@@ -398,49 +456,53 @@ void launch_batch_convert_slot(const BatchArgs &a, int b, cudaStream_t s) {
   bconvert_slot_kernel<<<512, 256, 0, s>>>(a, b);
 }
 
-// shared memory of one packed pair of slots of a class
-static size_t bring_smem_per_pair(int logM) { return ((size_t)1 << logM) * sizeof(float2); }
-
-// shared memory of a CTA of G slots: the packed FFT buffers, plus the alias
-// partial sums when the class can hold rings shorter than the block
-static size_t bring_smem(int logM, int G) {
-  const size_t part = ((size_t)1 << logM) <= 2 * kBringThreads ? (size_t)kBringThreads * G * sizeof(float2) : 0;
-  return (size_t)(G / 2) * bring_smem_per_pair(logM) + part;
+// shared memory of a CTA of G slots: the packed FFT buffers of the CTA's one or
+// two rings, plus the alias partial sums when the class can hold rings shorter
+// than the block
+static size_t bring_smem(int logM, int G, int nd) {
+  const size_t part = ((size_t)1 << logM) <= 2 * kBringThreads ? (size_t)kBringThreads * nd * G * sizeof(float2) : 0;
+  return (size_t)nd * (G / 2) * (sizeof(float2) << logM) + part;
 }
 
+constexpr size_t kBringSmemMax = 200 * 1024;
+
+// both rings of a pair in a CTA where two slots of them fit
+static int bring_sides(int logM) { return bring_smem(logM, 2, 2) <= kBringSmemMax ? 2 : 1; }
 
 // default slots per ring-stage CTA of a class (before autotuning): 8, 4 or 2
 // (pairs share one FFT), within a quarter of an SM's shared memory so that four
 // CTAs share each SM
 static int batch_ring_group(int logM, int B) {
   int G = 8;
-  while (G > 2 && (bring_smem(logM, G) > 54 * 1024 || G >= 2 * B)) G >>= 1;
+  while (G > 2 && (bring_smem(logM, G, bring_sides(logM)) > 54 * 1024 || G >= 2 * B)) G >>= 1;
   return G;
 }
 
-template <int G>
+template <int G, int ND>
 static void launch_bring(const BatchArgs &a, const RingClass &c, cudaStream_t s) {
-  const size_t sm = bring_smem(c.logM, G);
+  raise_smem_cap(reinterpret_cast<const void *>(bring_kernel<G, ND>));
   BatchArgs ac = a;
   ac.first = c.first;
-  bring_kernel<G><<<dim3(c.count, (a.B + G - 1) / G), kBringThreads, sm, s>>>(ac);
+  bring_kernel<G, ND><<<dim3(c.count * (ND == 2 ? 1 : 2), (a.B + G - 1) / G), kBringThreads, bring_smem(c.logM, G, ND),
+                        s>>>(ac);
 }
 
 // slots per CTA that a ring class may use: even, at most 8, the packed FFT
 // buffers within the shared memory of one CTA
 bool batch_ring_group_ok(int logM, int G) {
-  return (G == 2 || G == 4 || G == 8) && bring_smem(logM, G) <= 200 * 1024;
+  return (G == 2 || G == 4 || G == 8) && bring_smem(logM, G, bring_sides(logM)) <= kBringSmemMax;
 }
 
 void launch_batch_ring_class(const BatchArgs &a, const RingClass &c, int G, cudaStream_t s) {
-  raise_smem_cap(reinterpret_cast<const void *>(bring_kernel<2>));
-  raise_smem_cap(reinterpret_cast<const void *>(bring_kernel<4>));
-  raise_smem_cap(reinterpret_cast<const void *>(bring_kernel<8>));
   if (c.count <= 0) return;
   if (G <= 0 || !batch_ring_group_ok(c.logM, G)) G = batch_ring_group(c.logM, a.B);
-  if (G == 8) launch_bring<8>(a, c, s);
-  else if (G == 4) launch_bring<4>(a, c, s);
-  else launch_bring<2>(a, c, s);
+  if (bring_sides(c.logM) == 2) {
+    if (G == 8) launch_bring<8, 2>(a, c, s);
+    else if (G == 4) launch_bring<4, 2>(a, c, s);
+    else launch_bring<2, 2>(a, c, s);
+  } else {
+    launch_bring<2, 1>(a, c, s);   // buffers over 100 KB a side: two slots at most
+  }
 }
 
 void launch_batch_iteration(const BatchArgs &a, const TcArgs &t, const TcMaps &maps, const RingClass *cls, int ncls,

@@ -219,6 +219,16 @@ static wf_status build_geometry(Plan *P) {
     g.count = (int)porder.size() - g.first;
     P->psingle.push_back(g);
   }
+  // and every class in pairs: porder follows the classes' order, and the rings of a pair are of one class
+  P->pclass.clear();
+  for (int c = 0, at = 0; c < (int)P->rclass.size(); ++c) {
+    RingClass g = P->rclass[c];
+    g.first = at;
+    const int end = P->rclass[c].first + P->rclass[c].count;
+    for (int rings_in = P->rclass[c].first; rings_in < end; ++at) rings_in += porder[at].y >= 0 ? 2 : 1;
+    g.count = at - g.first;
+    P->pclass.push_back(g);
+  }
   if ((st = P->dalloc((void **)&P->d_rings, sizeof(RingDev) * R))) return st;
   if ((st = P->dalloc((void **)&P->d_order, sizeof(int) * R))) return st;
   if ((st = P->dalloc((void **)&P->d_porder, sizeof(int2) * porder.size()))) return st;
@@ -240,7 +250,7 @@ static wf_status build_geometry(Plan *P) {
     launch_bluestein_setup(P->d_rings, P->d_order, P->rsingle.data(), (int)P->rsingle.size(), P->d_ring_scratch,
                            P->d_tw, P->logMmax, P->d_chirp, P->d_B, s);
   // double-float copies for the ring_df kernels
-  P->n_tw = (long long)tw.size();
+  P->n_tw = twiddles_df(P->logMmax);
   P->n_hs = (long long)hs.size();
   P->n_ch = (long long)ch.size();
   P->n_B = B_tot > 0 ? B_tot : 1;
@@ -248,7 +258,7 @@ static wf_status build_geometry(Plan *P) {
   if ((st = P->dalloc((void **)&P->d_hsf, sizeof(float4) * P->n_hs))) return st;
   if ((st = P->dalloc((void **)&P->d_chf, sizeof(float4) * P->n_ch))) return st;
   if ((st = P->dalloc((void **)&P->d_Bf, sizeof(float4) * P->n_B))) return st;
-  launch_to_df(P->d_tw, P->d_twf, P->n_tw, s);
+  launch_pack_twiddles(P->d_tw, P->logMmax, P->d_twf, nullptr, s);
   launch_to_df(P->d_hs, P->d_hsf, P->n_hs, s);
   launch_to_df(P->d_chirp, P->d_chf, P->n_ch, s);
   launch_to_df(P->d_B, P->d_Bf, P->n_B, s);

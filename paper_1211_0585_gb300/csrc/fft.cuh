@@ -21,7 +21,15 @@
 // where a thread owns consecutive elements) and the digit-reversed accesses
 // of the pixel pass over distinct banks. G arrays of length M lie one after
 // another (stride Mp) and share every twiddle load.
-// tw[k] = e^{-2 pi i k / Mmax}, k < Mmax.
+// Twiddles: the FP64 policy reads tw[k] = e^{-2 pi i k / Mmax}, k < Mmax. There
+// the lanes of a stage below the longest stride over up to 32 lines a load, as
+// many wavefronts of the load pipe as the stage's data; the float policies
+// read the same values laid out by stage, consecutive for consecutive lanes
+// (FP32 ring stage at Nside 512 / 64 slots 3.25 -> 2.83 ms an iteration,
+// double-float 203 -> 184 us):
+//   double-float  stage 2^s: W_{2^s}^{i c}, c = 1 .. 3, i < 2^(s-2), at 3 (2^(s-2) - 1) + (c - 1) 2^(s-2) + i
+//   FP32          pass 2^s:  W_{2^s}^{i c} and W_{2^(s-2)}^{i c}, i < Q = 2^(s-4), at 6 (Q - 1) + (c - 1) Q + i and + 3 Q
+// (pack_twiddles_df / _f32; s = 4 .. max(4, log2 Mmax) for the latter).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -59,6 +67,10 @@ struct OpsF64 {
     if (sign > 0) w.y = -w.y;
     return w;
   }
+  // twiddle c = 1 .. 3 of position i of the radix-4 stage at size 2^s
+  static __device__ __forceinline__ T tw4(const W *t, int s, int i, int c, int logMmax, int sign) {
+    return tw(t, (c * i) << (logMmax - s), sign);
+  }
 };
 
 struct OpsF32 {  // float complex; twiddles from a float table
@@ -77,6 +89,13 @@ struct OpsF32 {  // float complex; twiddles from a float table
   static __device__ __forceinline__ T tw(const W *t, int idx, int sign) {
     const float2 w = t[idx];
     return make_float2(w.x, sign > 0 ? -w.y : w.y);
+  }
+  // the radix-4 stages left to this policy have size 4: i = 0, W = 1
+  static __device__ __forceinline__ T tw4(const W *t, int, int, int, int, int sign) { return tw(t, 0, sign); }
+  // twiddles c = 1 .. 3 of the two stages of the radix-16 pass at size 2^s (second = 0, 1)
+  static __device__ __forceinline__ T tw16(const W *t, int s, int i, int c, int second, int sign) {
+    const int Q = 1 << (s - 4);
+    return tw(t, 6 * (Q - 1) + (3 * second + c - 1) * Q + i, sign);
   }
   // e^{sign 2 pi i m / 16}, m = 0 .. 15 (m a compile-time constant after unrolling)
   static __device__ __forceinline__ T w16(int m, int sign) {
@@ -145,6 +164,10 @@ struct OpsDF {  // double-float complex: float4 (re hi, re lo, im hi, im lo)
     const float4 w = t[idx];
     return sign > 0 ? make_float4(w.x, w.y, -w.z, -w.w) : w;
   }
+  static __device__ __forceinline__ T tw4(const W *t, int s, int i, int c, int, int sign) {
+    const int Q = 1 << (s - 2);
+    return tw(t, 3 * (Q - 1) + (c - 1) * Q + i, sign);
+  }
 };
 
 // swizzled position of element e (e < 2^15)
@@ -174,13 +197,12 @@ template <class O, int G, bool DIT>
 __device__ void stage4(typename O::T *buf, int Mp, int M, int s, int sign, const typename O::W *tw, int logMmax) {
   using T = typename O::T;
   const int qsh = s - 2, Q = 1 << qsh;
-  const int tsh = logMmax - s;
   for (int t = threadIdx.x; t < (M >> 2); t += blockDim.x) {
     const int i = t & (Q - 1);
     const int base = ((t >> qsh) << s) + i;
-    const T w1 = O::tw(tw, i << tsh, sign);
-    const T w2 = O::tw(tw, (2 * i) << tsh, sign);
-    const T w3 = O::tw(tw, (3 * i) << tsh, sign);
+    const T w1 = O::tw4(tw, s, i, 1, logMmax, sign);
+    const T w2 = O::tw4(tw, s, i, 2, logMmax, sign);
+    const T w3 = O::tw4(tw, s, i, 3, logMmax, sign);
     // base and j Q have disjoint bits, so px(base + j Q) = px(base) ^ px(j Q)
     const int p0 = px<O>(base), q1 = px<O>(Q), q2 = px<O>(2 * Q);
     const int p1 = p0 ^ q1, p2 = p0 ^ q2, p3 = p0 ^ q1 ^ q2;
@@ -221,15 +243,14 @@ __device__ void stage2(typename O::T *buf, int Mp, int M) {
 // v[4c + j] (j = 0..3) at position i, with twiddles W_{4Q}^{i j}. DIF runs A
 // then B (twiddles after the butterflies), DIT runs B then A (before).
 template <class O, bool DIT>
-__device__ __forceinline__ void pass16_body(typename O::T (&v)[16], int i, int s, int sign, const typename O::W *tw,
-                                            int logMmax) {
+__device__ __forceinline__ void pass16_body(typename O::T (&v)[16], int i, int s, int sign,
+                                            const typename O::W *tw) {
   using T = typename O::T;
-  const int tshA = logMmax - s, tshB = tshA + 2;
   T a[4], b[4];
 #pragma unroll
   for (int c = 1; c < 4; ++c) {
-    a[c] = O::tw(tw, (i * c) << tshA, sign);
-    b[c] = O::tw(tw, (i * c) << tshB, sign);
+    a[c] = O::tw16(tw, s, i, c, 0, sign);
+    b[c] = O::tw16(tw, s, i, c, 1, sign);
   }
   auto stageA = [&](bool pre) {
 #pragma unroll
@@ -267,8 +288,7 @@ __device__ __forceinline__ void pass16_body(typename O::T (&v)[16], int i, int s
 }
 
 template <class O, int G, bool DIT>
-__device__ void pass16(typename O::T *buf, int Mp, int M, int logM, int s, int sign, const typename O::W *tw,
-                       int logMmax) {
+__device__ void pass16(typename O::T *buf, int Mp, int M, int logM, int s, int sign, const typename O::W *tw) {
   using T = typename O::T;
   const int qsh = s - 4, Q = 1 << qsh;
   const int ngrp = M >> 4;
@@ -289,7 +309,7 @@ __device__ void pass16(typename O::T *buf, int Mp, int M, int logM, int s, int s
     T v[16];
 #pragma unroll
     for (int j = 0; j < 16; ++j) v[j] = x[pj[j]];
-    pass16_body<O, DIT>(v, i, s, sign, tw, logMmax);
+    pass16_body<O, DIT>(v, i, s, sign, tw);
 #pragma unroll
     for (int j = 0; j < 16; ++j) x[pj[j]] = v[j];
   }
@@ -348,7 +368,7 @@ __device__ void fft_dif4(typename O::T *buf, int Mp, int M, int logM, int sign, 
                          int logMmax) {
   int s = logM;
   if constexpr (O::kR16) {
-    for (; s >= 4; s -= 4) pass16<O, G, false>(buf, Mp, M, logM, s, sign, tw, logMmax);
+    for (; s >= 4; s -= 4) pass16<O, G, false>(buf, Mp, M, logM, s, sign, tw);
     if (s == 3) { pass8<O, G, false>(buf, Mp, M, logM, sign); return; }
   }
   for (; s >= 2; s -= 2) stage4<O, G, false>(buf, Mp, M, s, sign, tw, logMmax);
@@ -364,7 +384,7 @@ __device__ void fft_dit4(typename O::T *buf, int Mp, int M, int logM, int sign, 
     if (s == 3) pass8<O, G, true>(buf, Mp, M, logM, sign);
     else if (s == 2) stage4<O, G, true>(buf, Mp, M, 2, sign, tw, logMmax);
     else if (s == 1) stage2<O, G>(buf, Mp, M);
-    for (s += 4; s <= logM; s += 4) pass16<O, G, true>(buf, Mp, M, logM, s, sign, tw, logMmax);
+    for (s += 4; s <= logM; s += 4) pass16<O, G, true>(buf, Mp, M, logM, s, sign, tw);
   } else {
     int s = 0;
     if (logM & 1) { stage2<O, G>(buf, Mp, M); s = 1; }

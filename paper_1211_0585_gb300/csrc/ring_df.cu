@@ -58,7 +58,8 @@ __device__ __forceinline__ void warp_sum_df(float &S, float &C) {
 // 512), so that one pair's barriers and global loads overlap another's work.
 // With the records, the fold and the sums in double, the FP64 pipe was as busy
 // as the FP32 one (37 %) and the kernel took 250 us at Nside 512, 65 us at 256;
-// in double-float throughout 203 and 52 us.
+// in double-float throughout 203 and 52 us, with the twiddles by stage
+// (fft.cuh) 184 us at Nside 512.
 constexpr int kRingDfThreads = 256;
 template <int MODE>
 __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingArgs A, const RingDfArgs T,
@@ -235,6 +236,31 @@ void launch_to_df(const double2 *src, float4 *dst, long long n, cudaStream_t s) 
   long long blocks = (n + 255) / 256;
   if (blocks > 4096) blocks = 4096;
   to_df_kernel<<<(int)blocks, 256, 0, s>>>(src, dst, n);
+}
+
+__global__ void pack_twiddles_kernel(const double2 *tw, int logMmax, float4 *df, float2 *f32) {
+  const int id = blockIdx.x * blockDim.x + threadIdx.x;
+  auto get = [&](int s, int i, int c) {   // e^{-2 pi i (i c) / 2^s}; sizes above the longest only at i = 0
+    const double2 v = tw[s <= logMmax ? (i * c) << (logMmax - s) : 0];
+    return df_pair(df_from(v.x), df_from(v.y));
+  };
+  if (df && id < (1 << logMmax) / 2 - 1) {            // (s, i) at 2^(s-2) - 1 + i
+    const int qsh = 31 - __clz(id + 1), Q = 1 << qsh, i = id + 1 - Q;
+    for (int c = 1; c < 4; ++c) df[3 * (Q - 1) + (c - 1) * Q + i] = get(qsh + 2, i, c);
+  }
+  if (f32 && id < (1 << (logMmax < 4 ? 4 : logMmax)) / 8 - 1) {
+    const int qsh = 31 - __clz(id + 1), Q = 1 << qsh, i = id + 1 - Q;
+    for (int c = 1; c < 4; ++c) {
+      const float4 a = get(qsh + 4, i, c), b = get(qsh + 2, i, c);
+      f32[6 * (Q - 1) + (c - 1) * Q + i] = make_float2(a.x, a.z);
+      f32[6 * (Q - 1) + (2 + c) * Q + i] = make_float2(b.x, b.z);
+    }
+  }
+}
+
+void launch_pack_twiddles(const double2 *tw, int logMmax, float4 *df, float2 *f32, cudaStream_t s) {
+  const int n = 1 << (logMmax < 4 ? 4 : logMmax);
+  pack_twiddles_kernel<<<(n + 255) / 256, 256, 0, s>>>(tw, logMmax, df, f32);
 }
 
 template <int MODE>

@@ -176,6 +176,11 @@ struct RingDfArgs {
   double *gainlam;        // [R] lambda the cached gains of each ring belong to (-1: none)
 };
 void launch_to_df2(const double *src, float2 *dst, long long n, cudaStream_t s);
+// The twiddles laid out by stage (fft.cuh) for FFTs up to 2^logMmax, from tw[k] = e^{-2 pi i k / 2^logMmax}:
+// entries, and the kernels that place them (double-float and, from its high parts, FP32)
+inline long long twiddles_df(int logMmax) { return logMmax < 2 ? 1 : 3 * ((1LL << (logMmax - 1)) - 1); }
+inline long long twiddles_f32(int logMmax) { return 6 * ((1LL << ((logMmax < 4 ? 4 : logMmax) - 3)) - 1); }
+void launch_pack_twiddles(const double2 *tw, int logMmax, float4 *df, float2 *f32, cudaStream_t s);
 // One map of a double-float ring-stage launch: what a RingArgs and RingDfArgs hold beside the shape's tables.
 constexpr int kRingMapsMax = 4;
 struct RingMap {
@@ -198,10 +203,10 @@ constexpr int kBatchMax = 64;
 
 struct BatchArgs {
   const RingDev *rings;
-  const int *order;          // ring of ring-stage CTA i is order[first + i]
+  const int2 *porder;        // ring pair of ring-stage CTA i: porder[first + i] = (north ring, south ring or -1)
   int first;
   const float4 *twf, *hsf, *chf, *Bf;
-  const float2 *tw2, *Bf2;   // FP32 twiddle and Bluestein filter tables (hi parts of twf, Bf)
+  const float2 *tw2, *Bf2;   // FP32 twiddles by stage and Bluestein filter tables (hi parts)
   int logMmax;
   int lmax, RP, R, B;
   long long npix, nalm;

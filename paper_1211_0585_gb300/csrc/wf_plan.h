@@ -35,7 +35,8 @@ struct Plan : wf_plan_s {
   // geometry and tables
   RingDev *d_rings = nullptr;
   int *d_order = nullptr;               // rings sorted by FFT class (RingClass), largest first
-  std::vector<RingClass> rclass;        // the classes (batched ring stage: one launch each)
+  std::vector<RingClass> rclass;        // the classes
+  std::vector<RingClass> pclass;        // the classes in ring pairs (batched ring stage: one launch each)
   std::vector<RingClass> rsingle;       // single-solve ring stage: the classes whose 16-byte FFT buffers
                                         // do not fit shared memory (global scratch), then every other ring
   std::vector<RingClass> psingle;       // the same classes in ring pairs (double-float ring stage)
