@@ -35,53 +35,57 @@
 namespace wfk {
 
 constexpr int kNoStartD = 1 << 30;
-constexpr int kAnaChunk = 1024;   // ring pairs whose analysis state is held in shared memory at once
+// ring pairs whose analysis state is held in shared memory at once: four a thread
+template <int NT> constexpr int kAnaChunk = 4 * NT;
 
 __device__ __forceinline__ size_t alm_idx_d(int lmax, int l, int m) {
   return (size_t)m * (2 * lmax + 1 - m) / 2 + l;
 }
 
-// Lane q ends with the double-float sum over the warp's lanes of (S[q], C[q]).
-__device__ __forceinline__ double warp_transpose_sum_df(float (&S)[32], float (&C)[32]) {
+// Sixteen compensated sums over the warp's lanes by exchanging halves: lanes 2 q and 2 q + 1 end with sum q
+__device__ __forceinline__ void warp_sums16(float (&S)[16], float (&C)[16]) {
   const int lane = threadIdx.x & 31;
+  auto add = [](float &s0, float &c0, float s1, float c1) {
+    const float s = s0 + s1;
+    const float bb = s - s0;
+    c0 = c0 + c1 + ((s0 - (s - bb)) + (s1 - bb));
+    s0 = s;
+  };
 #pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
+  for (int off = 16, n = 8; n >= 1; off >>= 1, n >>= 1) {
     const bool up = (lane & off) != 0;
 #pragma unroll
-    for (int j = 0; j < off; ++j) {
-      const float sS = up ? S[j] : S[j + off], sC = up ? C[j] : C[j + off];
-      const float kS = up ? S[j + off] : S[j], kC = up ? C[j + off] : C[j];
-      const float rS = __shfl_xor_sync(0xffffffffu, sS, off);
-      const float rC = __shfl_xor_sync(0xffffffffu, sC, off);
-      const float s = kS + rS;
-      const float bb = s - kS;
-      const float e = (kS - (s - bb)) + (rS - bb);
-      S[j] = s;
-      C[j] = kC + rC + e;
+    for (int j = 0; j < n; ++j) {
+      const float oS = up ? S[j] : S[j + n], oC = up ? C[j] : C[j + n];
+      S[j] = up ? S[j + n] : S[j];
+      C[j] = up ? C[j + n] : C[j];
+      add(S[j], C[j], __shfl_xor_sync(0xffffffffu, oS, off), __shfl_xor_sync(0xffffffffu, oC, off));
     }
   }
-  return (double)S[0] + (double)C[0];
+  add(S[0], C[0], __shfl_xor_sync(0xffffffffu, S[0], 1), __shfl_xor_sync(0xffffffffu, C[0], 1));
 }
 
-// 16 recurrence steps of one ring pair from l0, accumulating mu * (E or O)
-// into the 32 compensated sums; INJECT places the table start values.
+constexpr int kDB = 8;   // l per block of the analysis
+
+// kDB recurrence steps of one ring pair from l0, accumulating mu * (E or O)
+// into the 2 kDB compensated sums; INJECT places the table start values.
 template <bool INJECT>
-__device__ __forceinline__ void analysis_block(int l0, int m, const float2 *sA, dfl x, dfl &p1, dfl &p2, int ls,
-                                               dfl v0, dfl v1, dfl Er, dfl Ei, dfl Or, dfl Oi, float (&S)[32],
-                                               float (&C)[32]) {
+__device__ __forceinline__ void analysis_block(int l0, const float2 *sA, dfl x, dfl &p1, dfl &p2, int ls, float4 v,
+                                               float4 e, float4 o, float (&S)[16], float (&C)[16]) {
 #pragma unroll
-  for (int j = 0; j < kLB; ++j) {
+  for (int j = 0; j < kDB; ++j) {
     const int l = l0 + j;
-    const float2 a2 = sA[l - m];
+    const float2 a2 = sA[j];
     dfl mu = df_step(dfl{a2.x, a2.y}, x, p1, p2);
     if (INJECT) {
-      if (l == ls) mu = v0;
-      if (l == ls + 1) mu = v1;
+      if (l == ls) mu = dfl{v.x, v.y};
+      if (l == ls + 1) mu = dfl{v.z, v.w};
     }
     p2 = p1;
     p1 = mu;
-    dot2_acc(S[2 * j], C[2 * j], mu, (j & 1) ? Or : Er);
-    dot2_acc(S[2 * j + 1], C[2 * j + 1], mu, (j & 1) ? Oi : Ei);
+    const float4 f = (j & 1) ? o : e;
+    dot2_acc(S[2 * j], C[2 * j], mu, dfl{f.x, f.y});
+    dot2_acc(S[2 * j + 1], C[2 * j + 1], mu, dfl{f.z, f.w});
   }
 }
 
@@ -196,11 +200,19 @@ __global__ void lam_table_kernel(const double *xk, const double2 *rec, const int
   }
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(kThreads, 2) legendre_df_kernel(const LegArgs A, const LegDfArgs D) {
+// NT threads a CTA. At Nside 2048 / lmax 4096 the sums, coefficients and ring-pair
+// state of one m take most of an SM's shared memory, so that one CTA fits however
+// small it is: 256 threads there left 8 warps an SM to hide the recurrences'
+// chains. With 512 threads, 1024 for the synthesis alone, an iteration's launch
+// went from 102 to 94 ms and a synthesis from 36 to 31; blocks of 8 l with one
+// barrier each (16 l, two barriers and sums in double before) and one form of the
+// recurrence block a warp took the iteration to 78 ms. FP32 issue bounds both
+// (37 instructions a term: 25 ms a pass).
+template <int MODE, int NT>
+__global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) legendre_df_kernel(const LegArgs A, const LegDfArgs D) {
   extern __shared__ double2 dsm[];
-  __shared__ double red[kThreads / 32][32];
-  __shared__ double mred[kThreads / 32][3];
+  __shared__ float2 red[2][NT / 32][16];
+  __shared__ double mred[NT / 32][3];
   const int m = blockIdx.x;
   const int lmax = A.lmax, RP = A.RP;
   int L = A.lsht;
@@ -234,7 +246,7 @@ __global__ void __launch_bounds__(kThreads, 2) legendre_df_kernel(const LegArgs 
         __syncthreads();
         if (threadIdx.x == 0) {
           double a = 0.0, b = 0.0;
-          for (int w = 0; w < kThreads / 32; ++w) { a += mred[w][0]; b += mred[w][1]; }
+          for (int w = 0; w < NT / 32; ++w) { a += mred[w][0]; b += mred[w][1]; }
           A.m_part[3 * m] = a;
           A.m_part[3 * m + 1] = b;
           A.m_part[3 * m + 2] = 0.0;
@@ -262,11 +274,11 @@ __global__ void __launch_bounds__(kThreads, 2) legendre_df_kernel(const LegArgs 
 
   if (MODE == LEG_ANALYSIS || MODE == LEG_ITER) {
     // per ring pair state in shared memory: the thread's sums then cover all of
-    // its ring pairs of a chunk before one reduction per block of kLB values of
-    // l; chunks of kAnaChunk ring pairs run one after another (one chunk up to
-    // Nside 512), each adding its share to t_l
-    for (int k0 = 0; k0 < RP; k0 += kAnaChunk) {
-      const int nk = min(kAnaChunk, RP - k0);
+    // its ring pairs of a chunk before one reduction per block of kDB values of
+    // l; chunks of kAnaChunk ring pairs run one after another, each adding its
+    // share to t_l
+    for (int k0 = 0; k0 < RP; k0 += kAnaChunk<NT>) {
+      const int nk = min(kAnaChunk<NT>, RP - k0);
       float4 *stE = ss;                            // (Er, Ei) as hi/lo
       float4 *stO = stE + nk;                      // (Or, Oi)
       float4 *stP = stO + nk;                      // (p1, p2)
@@ -280,40 +292,52 @@ __global__ void __launch_bounds__(kThreads, 2) legendre_df_kernel(const LegArgs 
         stX[kk] = make_float2(xk.h, xk.l);
       }
       __syncthreads();
-      for (int l0 = m; l0 <= L; l0 += kLB) {
-        float S[32], C[32];
+      int lsr[4];                                  // first l of the thread's ring pairs
 #pragma unroll
-        for (int j = 0; j < 32; ++j) { S[j] = 0.f; C[j] = 0.f; }
-        for (int kk = threadIdx.x; kk < nk; kk += blockDim.x) {
-          const size_t mk = (size_t)m * RP + k0 + kk;
-          const int ls = D.ls[mk];
-          if (ls >= l0 + kLB) continue;            // no evaluated term yet in this block
-          const float2 x2 = stX[kk];
-          const dfl x = dfl{x2.x, x2.y};
-          const float4 e4 = stE[kk], o4 = stO[kk], q4 = stP[kk];
-          dfl p1 = dfl{q4.x, q4.y}, p2 = dfl{q4.z, q4.w};
-          if (ls + 1 >= l0) {                      // a start value falls in this block
-            const float4 s4 = D.sv[mk];
-            analysis_block<true>(l0, m, sA, x, p1, p2, ls, dfl{s4.x, s4.y}, dfl{s4.z, s4.w}, dfl{e4.x, e4.y},
-                                 dfl{e4.z, e4.w}, dfl{o4.x, o4.y}, dfl{o4.z, o4.w}, S, C);
-          } else {
-            analysis_block<false>(l0, m, sA, x, p1, p2, ls, dfl{0.f, 0.f}, dfl{0.f, 0.f}, dfl{e4.x, e4.y},
-                                  dfl{e4.z, e4.w}, dfl{o4.x, o4.y}, dfl{o4.z, o4.w}, S, C);
-          }
-          stP[kk] = make_float4(p1.h, p1.l, p2.h, p2.l);
-        }
-        const double s = warp_transpose_sum_df(S, C);
-        red[warp][lane] = s;
-        __syncthreads();
-        if (threadIdx.x < 32) {
-          double t = 0.0;
-#pragma unroll
-          for (int w = 0; w < kThreads / 32; ++w) t += red[w][threadIdx.x];
-          double *dst = reinterpret_cast<double *>(&tl[l0 - m + (threadIdx.x >> 1)]);
-          dst[threadIdx.x & 1] += t;
-        }
-        __syncthreads();
+      for (int i = 0; i < 4; ++i) {
+        const int kk = threadIdx.x + i * NT;
+        lsr[i] = kk < nk ? D.ls[(size_t)m * RP + k0 + kk] : kNoStartD;
       }
+      int buf = 0;
+      for (int l0 = m; l0 <= L; l0 += kDB, buf ^= 1) {
+        float S[16], C[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) { S[j] = 0.f; C[j] = 0.f; }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          // the whole warp runs the same block: lanes without a term yet carry zeros, and one with a start value in
+          // it takes the others through the injecting form (as per-lane branches the two forms ran one after the other)
+          const int ls = lsr[i], kk = min((int)threadIdx.x + i * NT, nk - 1);
+          const bool begun = ls < l0 + kDB;
+          if (!__any_sync(0xffffffffu, begun)) continue;
+          const bool starts = begun && ls + 1 >= l0;
+          const float2 x2 = stX[kk];
+          const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+          const float4 e4 = begun ? stE[kk] : z, o4 = begun ? stO[kk] : z, q4 = stP[kk];
+          dfl p1 = dfl{q4.x, q4.y}, p2 = dfl{q4.z, q4.w};
+          if (__any_sync(0xffffffffu, starts))
+            analysis_block<true>(l0, sA + (l0 - m), dfl{x2.x, x2.y}, p1, p2, ls,
+                                 starts ? D.sv[(size_t)m * RP + k0 + kk] : z, e4, o4, S, C);
+          else
+            analysis_block<false>(l0, sA + (l0 - m), dfl{x2.x, x2.y}, p1, p2, ls, z, e4, o4, S, C);
+          if (begun) stP[kk] = make_float4(p1.h, p1.l, p2.h, p2.l);
+        }
+        warp_sums16(S, C);
+        if (!(lane & 1)) red[buf][warp][lane >> 1] = make_float2(S[0], C[0]);
+        __syncthreads();                           // one a block: the other buffer is the next one's
+        if (threadIdx.x < 16) {
+          float tS = 0.f, tC = 0.f;
+          for (int w = 0; w < NT / 32; ++w) {
+            const float2 v = red[buf][w][threadIdx.x];
+            const float n = tS + v.x, bb = n - tS;
+            tC += v.y + ((tS - (n - bb)) + (v.x - bb));
+            tS = n;
+          }
+          double *dst = reinterpret_cast<double *>(&tl[l0 - m + (threadIdx.x >> 1)]);
+          dst[threadIdx.x & 1] += (double)tS + (double)tC;
+        }
+      }
+      __syncthreads();
     }
     // undo the rescaling: lambda = g mu
     for (int l = m + threadIdx.x; l <= L; l += blockDim.x) {
@@ -363,7 +387,7 @@ __global__ void __launch_bounds__(kThreads, 2) legendre_df_kernel(const LegArgs 
     __syncthreads();
     if (threadIdx.x == 0) {
       double a = 0.0, b = 0.0, c = 0.0;
-      for (int w = 0; w < kThreads / 32; ++w) { a += mred[w][0]; b += mred[w][1]; c += mred[w][2]; }
+      for (int w = 0; w < NT / 32; ++w) { a += mred[w][0]; b += mred[w][1]; c += mred[w][2]; }
       A.m_part[3 * m] = a;
       A.m_part[3 * m + 1] = b;
       A.m_part[3 * m + 2] = c;
@@ -434,12 +458,20 @@ __global__ void __launch_bounds__(kThreads, 2) legendre_df_kernel(const LegArgs 
 
 // tl [Lp] double2 | sA [Lp (+1)] float2 | max(Lp, 3.5 chunk) float4 (synthesis
 // coefficients, or the per-ring-pair analysis state of one chunk)
-static size_t leg_df_smem(int lmax, int RP) {
+static size_t leg_df_smem(int lmax, int RP, int chunk) {
   const size_t Lp = (size_t)lmax + 1 + kLB;
-  const size_t nk = RP < kAnaChunk ? (size_t)RP : (size_t)kAnaChunk;
+  const size_t nk = RP < chunk ? (size_t)RP : (size_t)chunk;
   const size_t st = 3 * nk + (nk + 1) / 2;
   const size_t q = Lp > st ? Lp : st;
   return Lp * sizeof(double2) + (Lp + 1) * sizeof(float2) + q * sizeof(float4) + 16;
+}
+
+template <int MODE, int NT>
+static void launch_df(const LegArgs &a, const LegDfArgs &d, cudaStream_t s) {
+  raise_smem_cap(reinterpret_cast<const void *>(legendre_df_kernel<MODE, NT>));
+  // the synthesis alone holds no ring-pair state
+  const size_t sm = leg_df_smem(a.lmax, a.RP, MODE == LEG_SYNTH ? 0 : kAnaChunk<NT>);
+  legendre_df_kernel<MODE, NT><<<a.lmax + 1, NT, sm, s>>>(a, d);
 }
 
 void launch_legendre_df(const LegArgs &a, const LegDfArgs &d, cudaStream_t s, int mode) {
@@ -458,20 +490,20 @@ void launch_legendre_df(const LegArgs &a, const LegDfArgs &d, cudaStream_t s, in
     launch_legendre_tab(a, d, bm, 1, s, mode);
     return;
   }
-  const int grid = a.lmax + 1;
-  const size_t sm = leg_df_smem(a.lmax, a.RP);
+  // four ring pairs a thread keep the larger CTAs' sums over lanes as cheap a term as the smaller ones'
+  const bool wide = a.RP >= 2048;
   switch (mode) {
     case LEG_SYNTH:
-      raise_smem_cap(reinterpret_cast<const void *>(legendre_df_kernel<LEG_SYNTH>));
-      legendre_df_kernel<LEG_SYNTH><<<grid, kThreads, sm, s>>>(a, d);
+      if (wide) launch_df<LEG_SYNTH, 1024>(a, d, s);
+      else launch_df<LEG_SYNTH, 256>(a, d, s);
       break;
     case LEG_ANALYSIS:
-      raise_smem_cap(reinterpret_cast<const void *>(legendre_df_kernel<LEG_ANALYSIS>));
-      legendre_df_kernel<LEG_ANALYSIS><<<grid, kThreads, sm, s>>>(a, d);
+      if (wide) launch_df<LEG_ANALYSIS, 512>(a, d, s);
+      else launch_df<LEG_ANALYSIS, 256>(a, d, s);
       break;
     default:
-      raise_smem_cap(reinterpret_cast<const void *>(legendre_df_kernel<LEG_ITER>));
-      legendre_df_kernel<LEG_ITER><<<grid, kThreads, sm, s>>>(a, d);
+      if (wide) launch_df<LEG_ITER, 512>(a, d, s);
+      else launch_df<LEG_ITER, 256>(a, d, s);
       break;
   }
 }
