@@ -57,8 +57,9 @@ __device__ __forceinline__ double warp_transpose_sum(double (&v)[32]) {
 // binary exponent so that sin^m(theta) cannot underflow. Bound by the FP64
 // pipe: the factors sqrt((2i + 1) / 2i) of lambda_mm are the same for every
 // column, so the CTA forms them once (a division and a square root each), and
-// exponents are compared as integers; with both in every thread's own loop the
-// kernel took 199 us at Nside 64 / lmax 128.
+// exponents are compared as integers (199 -> 44 us at Nside 64 / lmax 128; with
+// the recurrence's coefficients loaded ahead 39, with CTAs of 64 threads for a
+// small problem, start_values.cuh, 36).
 __global__ void __launch_bounds__(256) start_values_kernel(const double *xk, const double2 *rec, int lmax, int RP,
                                                            int *ls_out, double2 *sv_out) {
   extern __shared__ double croot[];   // [m + 1] sqrt((2i + 1) / 2i)
@@ -74,27 +75,7 @@ __global__ void __launch_bounds__(256) start_values_kernel(const double *xk, con
   if (m == 0 || st > 0.0) {
     int e = 0;
     const double v = lambda_mm_scaled(croot, m, st, e);
-    // walk up in l until the true value reaches 2^kStartExp
-    double p2 = v;                               // lambda_l (scaled)
-    double p1 = x * sqrt(2.0 * m + 3.0) * v;     // lambda_{l+1} (scaled)
-    for (int l = m; l <= lmax; ++l) {
-      if (p2 != 0.0 && exponent_of(p2) + e >= kStartExp) {
-        ls = l;
-        v0 = ldexp(p2, e);
-        v1 = (l + 1 <= lmax) ? ldexp(p1, e) : 0.0;
-        break;
-      }
-      if (l + 2 <= lmax) {
-        const double2 ab = rec[alm_idx(lmax, l + 2, m)];
-        const double nx = ab.x * x * p1 - ab.y * p2;
-        p2 = p1;
-        p1 = nx;
-        if (exponent_of(p2) >= 400 || exponent_of(p1) >= 400) { p1 *= 0x1p-400; p2 *= 0x1p-400; e += 400; }
-      } else {
-        p2 = p1;
-        p1 = 0.0;
-      }
-    }
+    ls = walk_to_cut(rec + alm_idx(lmax, m, m), x, v, e, m, lmax, kStartExp, kNoStart, v0, v1);
   }
   ls_out[id] = ls;
   sv_out[id] = make_double2(v0, v1);
@@ -347,8 +328,8 @@ void launch_legendre(const LegArgs &a, cudaStream_t s, int mode) {
 void launch_start_values(const double *x, const double2 *rec, int lmax, int RP, int *ls, double2 *sv,
                          cudaStream_t s) {
   const long long n = (long long)(lmax + 1) * RP;
-  const int blocks = (int)((n + 255) / 256);
-  start_values_kernel<<<blocks, 256, (size_t)(lmax + 1) * sizeof(double), s>>>(x, rec, lmax, RP, ls, sv);
+  const int nt = start_value_threads(n);
+  start_values_kernel<<<(int)((n + nt - 1) / nt), nt, (size_t)(lmax + 1) * sizeof(double), s>>>(x, rec, lmax, RP, ls, sv);
 }
 
 }  // namespace wfk

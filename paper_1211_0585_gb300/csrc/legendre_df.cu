@@ -106,25 +106,7 @@ __global__ void __launch_bounds__(256) start_values_df_kernel(const double *xk, 
   if (m == 0 || st > 0.0) {
     int e = 0;
     const double v = lambda_mm_scaled(croot, m, st, e);
-    double p2 = v, p1 = x * sqrt(2.0 * m + 3.0) * v;
-    for (int l = m; l <= lmax; ++l) {
-      if (p2 != 0.0 && exponent_of(p2) + e >= -60) {
-        ls = l;
-        v0 = ldexp(p2, e);
-        v1 = (l + 1 <= lmax) ? ldexp(p1, e) : 0.0;
-        break;
-      }
-      if (l + 2 <= lmax) {
-        const double2 ab = rec[alm_idx_d(lmax, l + 2, m)];
-        const double nx = ab.x * x * p1 - ab.y * p2;
-        p2 = p1;
-        p1 = nx;
-        if (exponent_of(p2) >= 400 || exponent_of(p1) >= 400) { p1 *= 0x1p-400; p2 *= 0x1p-400; e += 400; }
-      } else {
-        p2 = p1;
-        p1 = 0.0;
-      }
-    }
+    ls = walk_to_cut(rec + alm_idx_d(lmax, m, m), x, v, e, m, lmax, -60, kNoStartD, v0, v1);
   }
   float4 out = make_float4(0.f, 0.f, 0.f, 0.f);
   if (ls != kNoStartD) {
@@ -524,7 +506,8 @@ void launch_df_tables(const double *x, const double2 *rec, int lmax, int RP, dou
                       float4 *sv, cudaStream_t s) {
   rescale_coeffs_kernel<<<lmax + 1, 32, 0, s>>>(rec, lmax, g, A);
   const long long n = (long long)(lmax + 1) * RP;
-  start_values_df_kernel<<<(int)((n + 255) / 256), 256, (size_t)(lmax + 1) * sizeof(double), s>>>(x, rec, g, lmax, RP, ls, sv);
+  const int nt = start_value_threads(n);
+  start_values_df_kernel<<<(int)((n + nt - 1) / nt), nt, (size_t)(lmax + 1) * sizeof(double), s>>>(x, rec, g, lmax, RP, ls, sv);
 }
 
 }  // namespace wfk

@@ -227,7 +227,8 @@ __device__ __forceinline__ dfl warp_sum8_df(float (&S)[8], float (&C)[8]) {
 // tiles of 32 ring pairs are in flight while one is summed. Chunks of l instead
 // of a CTA per m keep every SM busy at any lmax. A CTA per m, FP64 sums over the
 // warp and one step of loads ahead: 2.28 ms a launch at Nside 512 / lmax 1024 and
-// 156 us at Nside 128 / lmax 256; now 1.80 ms and 54 us.
+// 156 us at Nside 128 / lmax 256; now 1.51 ms and 47 us (1.80 and 54 before the
+// loop over tiles was counted, without a search and moves a step).
 __global__ void __launch_bounds__(kPolThreads, 3) spin2_analysis_df_kernel(const Ctl *gate, const float4 *tab,
                                                                             const int *ls, const double4_32a *FTQ,
                                                                             const double4_32a *FTU, int lmax, int RP,
@@ -244,10 +245,13 @@ __global__ void __launch_bounds__(kPolThreads, 3) spin2_analysis_df_kernel(const
     const int k = 32 * t + lane;
     const int mn = __reduce_min_sync(0xffffffffu, k < RP ? ls[(size_t)m * RP + k] : 1 << 30);
     if (lane == 0) tmin[t] = mn;
-    if (k < RP && mn <= lend) {
-      f_parities(FTQ[(size_t)m * RP + k], pol_dsm[k], pol_dsm[RP + k]);
-      f_parities(FTU[(size_t)m * RP + k], pol_dsm[2 * RP + k], pol_dsm[3 * RP + k]);
-    }
+  }
+  __syncthreads();
+  int tf = 0;                           // the tiles any row of the chunk reads
+  while (tf < ntile && tmin[tf] > lend + 1) ++tf;
+  for (int k = 32 * tf + threadIdx.x; k < RP; k += blockDim.x) {
+    f_parities(FTQ[(size_t)m * RP + k], pol_dsm[k], pol_dsm[RP + k]);
+    f_parities(FTU[(size_t)m * RP + k], pol_dsm[2 * RP + k], pol_dsm[3 * RP + k]);
   }
   __syncthreads();
   const size_t base = idx_lm(lmax, m, m);
@@ -257,10 +261,8 @@ __global__ void __launch_bounds__(kPolThreads, 3) spin2_analysis_df_kernel(const
 #pragma unroll
     for (int j = 0; j < 8; ++j) { S[j] = 0.f; C[j] = 0.f; }
     const float4 *row0 = tab + (base + (l - m)) * RP, *row1 = row0 + RP;
-    auto next_tile = [&](int t) {   // the next tile with a term of l or l + 1 (F+- = 0 below a ring pair's first l)
-      while (t < ntile && tmin[t] > l + 1) ++t;
-      return t;
-    };
+    int t0 = 0;                       // the first tile with a term of l or l + 1 (F+- = 0 below a ring pair's first l;
+    while (t0 < ntile && tmin[t0] > l + 1) ++t0;   // towards the equator the first l falls)
     auto load = [&](int t, float4 &f0, float4 &f1) {
       const int k = 32 * t + lane;
       f0 = k < RP ? row0[k] : zero4();
@@ -293,20 +295,17 @@ __global__ void __launch_bounds__(kPolThreads, 3) spin2_analysis_df_kernel(const
         dot2_acc(S[7], C[7], fn, dfl{A.x, A.y});
       }
     };
-    float4 a0 = zero4(), a1 = zero4(), b0 = zero4(), b1 = zero4();
-    int ta = next_tile(0), tb = next_tile(ta + 1);
-    if (ta < ntile) load(ta, a0, a1);
-    if (tb < ntile) load(tb, b0, b1);
-    while (ta < ntile) {
-      const int t0 = ta;
-      const float4 f0 = a0, f1 = a1;
-      const int tc = next_tile(tb + 1);
-      ta = tb;
-      tb = tc;
-      a0 = b0;
-      a1 = b1;
-      if (tc < ntile) load(tc, b0, b1);
-      term(t0, f0, f1);
+    float4 f[2][2];
+    if (t0 < ntile) load(t0, f[0][0], f[0][1]);
+    if (t0 + 1 < ntile) load(t0 + 1, f[1][0], f[1][1]);
+    for (int tb = t0; tb < ntile; tb += 2) {
+#pragma unroll
+      for (int d = 0; d < 2; ++d) {   // compile-time buffer indices
+        const int t = tb + d;
+        if (t >= ntile) break;
+        term(t, f[d][0], f[d][1]);
+        if (t + 2 < ntile) load(t + 2, f[d][0], f[d][1]);
+      }
     }
     const dfl v = warp_sum8_df(S, C);
     if ((lane & 3) == 0) {   // sum lane / 4: E re, im, B re, im of l, then of l + 1
@@ -329,7 +328,7 @@ __global__ void __launch_bounds__(kPolThreads, 3) spin2_analysis_df_kernel(const
 // nobody else reads it), which holds the loads of a DRAM latency without the
 // registers that a third CTA per SM needs. Four rows loaded at a time, a CTA per
 // m: 1.65 ms a launch at Nside 512 / lmax 1024, 78 us at Nside 128 / lmax 256; now
-// 1.48 ms and 48 us.
+// 1.41 ms and 46 us.
 constexpr int kSynDepth = 8;   // rows in flight, even
 __device__ __forceinline__ void cp_async16(float4 *dst, const float4 *src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
@@ -355,13 +354,13 @@ __global__ void __launch_bounds__(kPolThreads, 3) spin2_synthesis_df_kernel(cons
   const int lw = __reduce_min_sync(0xffffffffu, k < RP ? ls[(size_t)m * RP + k] : 1 << 30);
   const int i0 = max(m < 2 ? 2 - m : 0, lw - m) & ~1;
   const float4 *col = tab + base * RP + min(k, RP - 1);
-  auto fetch = [&](int i) {   // rows i and i + 1 into the ring (one group, also when there is none left)
-    if (i < Lm) cp_async16(ring + (size_t)(i & (kSynDepth - 1)) * nt, col + (size_t)i * RP);
-    if (i + 1 < Lm) cp_async16(ring + (size_t)((i + 1) & (kSynDepth - 1)) * nt, col + (size_t)(i + 1) * RP);
+  auto fetch = [&](int i, int j) {   // rows i and i + 1 into places j, j + 1 (one group, also when there is none left)
+    if (i < Lm) cp_async16(ring + (size_t)j * nt, col + (size_t)i * RP);
+    if (i + 1 < Lm) cp_async16(ring + (size_t)(j + 1) * nt, col + (size_t)(i + 1) * RP);
     cp_commit();
   };
 #pragma unroll
-  for (int j = 0; j < kSynDepth; j += 2) fetch(i0 + j);
+  for (int j = 0; j < kSynDepth; j += 2) fetch(i0 + j, j);
   for (int i = threadIdx.x; i < Lm; i += nt) {
     coef[2 * i] = cdf(aE[base + i].x, aE[base + i].y);
     coef[2 * i + 1] = cdf(aB[base + i].x, aB[base + i].y);
@@ -384,13 +383,17 @@ __global__ void __launch_bounds__(kPolThreads, 3) spin2_synthesis_df_kernel(cons
     dot2_acc(Sa[7], Ca[7], fm, er);
   };
   const int istart = m < 2 ? 2 - m : 0;   // rows of l < 2 hold zeros; their coefficients may be anything
-  for (int i = i0; i < Lm; i += 2) {
-    cp_wait<kSynDepth / 2 - 1>();
-    const float4 f0 = ring[(size_t)(i & (kSynDepth - 1)) * nt];
-    const float4 f1 = ring[(size_t)((i + 1) & (kSynDepth - 1)) * nt];
-    if (i >= istart) accum(i, f0, S0, C0);
-    if (i + 1 < Lm && i + 1 >= istart) accum(i + 1, f1, S1, C1);
-    fetch(i + kSynDepth);   // into the slots just used
+  for (int ib = i0; ib < Lm; ib += kSynDepth) {
+#pragma unroll
+    for (int j = 0; j < kSynDepth; j += 2) {   // compile-time places in the ring
+      const int i = ib + j;
+      if (i >= Lm) break;
+      cp_wait<kSynDepth / 2 - 1>();
+      const float4 f0 = ring[(size_t)j * nt], f1 = ring[(size_t)(j + 1) * nt];
+      if (i >= istart) accum(i, f0, S0, C0);
+      if (i + 1 < Lm && i + 1 >= istart) accum(i + 1, f1, S1, C1);
+      fetch(i + kSynDepth, j);          // into the places just used
+    }
   }
   cp_wait<0>();
   if (k >= RP) return;
