@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 
 #include "ctl.cuh"
+#include "pdl.cuh"
 #include "wf_internal.h"
 
 namespace wfk {
@@ -36,6 +37,8 @@ __global__ void __launch_bounds__(kCtlThreads) control_kernel(const __grid_const
   const CtlMap &M = Maps.m[blockIdx.x];
   static_assert(sizeof(Ctl) % 4 == 0 && sizeof(Ctl) / 4 <= kCtlThreads, "copied a word a thread");
   constexpr int kWords = sizeof(Ctl) / 4;
+  pdl_wait();
+  pdl_next();
   if (threadIdx.x < kWords) reinterpret_cast<int *>(&live)[threadIdx.x] = reinterpret_cast<const int *>(M.ctl)[threadIdx.x];
   double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};   // chi2_N, chi2_lambda_N, chi2_S, increment, norm
   const double2 *rp = reinterpret_cast<const double2 *>(M.ring_part);
@@ -75,7 +78,7 @@ void launch_control(const CtlMap *maps, int n, int R, int lmax, cudaStream_t s) 
     CtlMaps q{};
     const int k = n - i0 < kCtlMapsMax ? n - i0 : kCtlMapsMax;
     for (int i = 0; i < k; ++i) q.m[i] = maps[i0 + i];
-    control_kernel<<<k, kCtlThreads, 0, s>>>(q, R, lmax);
+    launch_pdl(control_kernel, k, kCtlThreads, 0, s, q, R, lmax);
   }
 }
 

@@ -28,6 +28,7 @@
 #include <algorithm>
 
 #include "df.cuh"
+#include "pdl.cuh"
 #include "wf_internal.h"
 
 namespace wfk {
@@ -86,6 +87,8 @@ __global__ void __launch_bounds__(kThreads, NB == 1 ? 3 : 2) tab_analysis_kernel
   __shared__ double mred[kWarpsT][3];
   const int m = blockIdx.x, r0 = blockIdx.y * kTabRows;
   const int lmax = A.lmax, RP = A.RP;
+  pdl_wait();
+  pdl_next();
   if (m + 2 * r0 > lmax) return;
   const MapSet<NB, ITER> S(A, Bm);
   if (S.L < 0) return;
@@ -251,6 +254,8 @@ __global__ void __launch_bounds__(kThreads, 3) tab_synthesis_kernel(const LegArg
   extern __shared__ float4 csm[];   // [NB][nc] coefficients (re hi, re lo, im hi, im lo)
   const int m = blockIdx.x;
   const int lmax = A.lmax, RP = A.RP;
+  pdl_wait();
+  pdl_next();
   const MapSet<NB, ITER> S(A, Bm);
   if (S.L < 0) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -367,11 +372,11 @@ void launch_tab(const LegArgs &a, const LegDfArgs &d, const LegBatchMaps &bm, cu
   const size_t sa = ana_smem(NB, a.RP), ss = syn_smem(NB, a.lmax);
   auto ana = [&](auto kernel) {
     raise_smem_cap(reinterpret_cast<const void *>(kernel));
-    kernel<<<ga, kThreads, sa, s>>>(a, d, bm);
+    launch_pdl(kernel, ga, kThreads, sa, s, a, d, bm);
   };
   auto syn = [&](auto kernel) {
     raise_smem_cap(reinterpret_cast<const void *>(kernel));
-    kernel<<<gs, 32 * nw, ss, s>>>(a, d, bm, nchunk);
+    launch_pdl(kernel, gs, 32 * nw, ss, s, a, d, bm, nchunk);
   };
   if (mode == LEG_SYNTH) syn(tab_synthesis_kernel<NB, false>);
   else if (mode == LEG_ANALYSIS) ana(tab_analysis_kernel<NB, false>);
