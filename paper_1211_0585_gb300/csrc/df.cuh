@@ -44,6 +44,19 @@ __device__ __forceinline__ dfl df_add(dfl a, dfl b) {
   return {r, e - (r - s)};
 }
 
+// a + b with the low parts' sum error-free too (accurate double-word addition, Joldes, Muller and Popescu, ACM TOMS 44,
+// 2017): where a few sums stand between long chains of products, as the Fourier records' do
+__device__ __forceinline__ dfl df_add2(dfl a, dfl b) {
+  const float s = a.h + b.h, bb = s - a.h;
+  const float e = (a.h - (s - bb)) + (b.h - bb);
+  const float t = a.l + b.l, bt = t - a.l;
+  const float f = (a.l - (t - bt)) + (b.l - bt);
+  const float c = e + t;
+  const float v = s + c, w = f + (c - (v - s));
+  const float r = v + w;
+  return {r, w - (r - v)};
+}
+
 // a * b (two_prod of the high parts plus the cross terms, renormalised)
 __device__ __forceinline__ dfl df_mul(dfl a, dfl b) {
   const float p = a.h * b.h;
@@ -53,25 +66,52 @@ __device__ __forceinline__ dfl df_mul(dfl a, dfl b) {
   return {r, e - (r - p)};
 }
 
+// a * b with the product of the low parts
+__device__ __forceinline__ dfl df_mul2(dfl a, dfl b) {
+  const float p = a.h * b.h;
+  float e = fmaf(a.l, b.l, fmaf(a.h, b.h, -p));
+  e = fmaf(a.h, b.l, fmaf(a.l, b.h, e));
+  const float r = p + e;
+  return {r, e - (r - p)};
+}
+
 // S + C += a * b: compensated dot-product step (Ogita, Rump and Oishi,
-// "Accurate sum and dot product", SIAM J. Sci. Comput. 26, 2005), ten FP32
-// instructions. two_sum(S, p) splits into the parts of S and of p that the
-// rounded sum lost; the part of p, p - bb, is formed from the exact product
-// (one fma instead of two_prod's error term and a subtraction), and the cross
-// terms are added to it, at its own magnitude, by two more. The loops over
+// "Accurate sum and dot product", SIAM J. Sci. Comput. 26, 2005). The loops over
 // l and over ring pairs are made of this step, and FP32 issue bounds them once
-// their table reads are hidden: 13.7 instructions a product measured 2.8e12
-// products/s.
+// their table reads are hidden: in 13 instructions 2.8e12 products/s measured.
+// FINE, 12 instructions: every error term exact but for the two cross terms,
+// as in the sum of Ogita et al. Else 10: two_sum(S, p) splits into the parts of S
+// and of p that the rounded sum lost, the part of p is formed from the exact
+// product (one fma instead of two_prod's error term and a subtraction) and the
+// cross terms are added to it. Those three round at the sum's own ulp, which
+// short sums feel (7 % more error over 16 terms, 1 % over 128); long ones are
+// bound by the rounding of C, which dot2_tidy keeps small.
+template <bool FINE = false>
 __device__ __forceinline__ void dot2_acc(float &S, float &C, dfl a, dfl b) {
   const float p = __fmul_rn(a.h, b.h);
   const float s = __fadd_rn(S, p);
   const float bb = s - S;
   const float d = S - (s - bb);
-  float v = fmaf(a.h, b.h, -bb);
-  v = fmaf(a.l, b.h, v);
-  v = fmaf(a.h, b.l, v);
+  if (FINE) {
+    float v = fmaf(a.h, b.h, -p);
+    v = fmaf(a.l, b.h, v);
+    v = fmaf(a.h, b.l, v);
+    C += (d + (p - bb)) + v;
+  } else {
+    float v = fmaf(a.h, b.h, -bb);
+    v = fmaf(a.l, b.h, v);
+    v = fmaf(a.h, b.l, v);
+    C += d + v;
+  }
   S = s;
-  C += d + v;
+}
+
+// The collected errors of a long compensated sum moved into its leading part: the next ones round at a small C's ulp
+// again (every 32 terms or so the error of a sum of 512 falls by two)
+__device__ __forceinline__ void dot2_tidy(float &S, float &C) {
+  const float s = S + C;
+  C -= s - S;
+  S = s;
 }
 
 // mu_l = (A x) mu1 - mu2 in double-float: one step of the rescaled Legendre
@@ -95,12 +135,12 @@ __device__ __forceinline__ dfl df_step(dfl A, dfl x, dfl mu1, dfl mu2) {
 // and for odd, O = N - S, each (re hi, re lo, im hi, im lo); and the record of E and O.
 __device__ __forceinline__ void f_parities(const double4_32a &t, float4 &E, float4 &O) {
   const dfl nr = df_unpack(t.x), ni = df_unpack(t.y), sr = df_unpack(t.z), si = df_unpack(t.w);
-  E = df_pair(df_add(nr, sr), df_add(ni, si));
-  O = df_pair(df_add(nr, df_neg(sr)), df_add(ni, df_neg(si)));
+  E = df_pair(df_add2(nr, sr), df_add2(ni, si));
+  O = df_pair(df_add2(nr, df_neg(sr)), df_add2(ni, df_neg(si)));
 }
 __device__ __forceinline__ double4_32a f_rings(dfl er, dfl ei, dfl orr, dfl oi) {
-  return make_double4_32a(df_pack(df_add(er, orr)), df_pack(df_add(ei, oi)), df_pack(df_add(er, df_neg(orr))),
-                          df_pack(df_add(ei, df_neg(oi))));
+  return make_double4_32a(df_pack(df_add2(er, orr)), df_pack(df_add2(ei, oi)), df_pack(df_add2(er, df_neg(orr))),
+                          df_pack(df_add2(ei, df_neg(oi))));
 }
 
 }  // namespace wfk

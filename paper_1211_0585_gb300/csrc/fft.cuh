@@ -136,21 +136,21 @@ struct OpsDF {  // double-float complex: float4 (re hi, re lo, im hi, im lo)
     const float2 re = dadd(a.x, a.y, -b.x, -b.y), im = dadd(a.z, a.w, -b.z, -b.w);
     return make_float4(re.x, re.y, im.x, im.y);
   }
-  // p q - r s (real double-floats): two_sum of the rounded high products, and
-  // what it lost of each product formed from the exact one by fma, the cross
-  // terms added to it; 15 FP32 instructions against 25 of two products and a sum
+  // p q - r s (real double-floats): two_prod of both, two_sum of the high
+  // products, the error and cross terms added up and renormalised once; 19 FP32
+  // instructions against 25 of two products and a sum
   static __device__ __forceinline__ float2 pqrs(float ph, float pl, float qh, float ql, float rh, float rl, float sh,
                                                 float sl) {
     const float a = __fmul_rn(ph, qh), b = __fmul_rn(rh, sh);
+    float u = fmaf(ph, qh, -a), v = fmaf(rh, sh, -b);
     const float s = __fadd_rn(a, -b);
-    const float bb = __fadd_rn(s, -a);       // the part of -b in s
-    const float t = __fadd_rn(s, -bb);       // the part of a in s
-    float u = fmaf(ph, qh, -t), v = fmaf(-rh, sh, -bb);
+    const float bb = __fadd_rn(s, -a);
+    const float e = (a - (s - bb)) + (-b - bb);
     u = fmaf(ph, ql, fmaf(pl, qh, u));
-    v = fmaf(-rh, sl, fmaf(-rl, sh, v));
-    const float e = u + v;
-    const float h = s + e;
-    return make_float2(h, e - (h - s));
+    v = fmaf(rh, sl, fmaf(rl, sh, v));
+    const float w = e + (u - v);
+    const float h = s + w;
+    return make_float2(h, w - (h - s));
   }
   static __device__ __forceinline__ T mul(T a, T b) {
     const float2 re = pqrs(a.x, a.y, b.x, b.y, a.z, a.w, b.z, b.w);

@@ -45,7 +45,7 @@ __device__ __forceinline__ FoldPair fold_record(const double4_32a *FS, size_t at
           make_float4(sg * sr.h, sg * sr.l, ci * si.h, ci * si.l)};
 }
 __device__ __forceinline__ float4 fold_add(float4 a, float4 b) {
-  return df_pair(df_add(dfl{a.x, a.y}, dfl{b.x, b.y}), df_add(dfl{a.z, a.w}, dfl{b.z, b.w}));
+  return df_pair(df_add2(dfl{a.x, a.y}, dfl{b.x, b.y}), df_add2(dfl{a.z, a.w}, dfl{b.z, b.w}));
 }
 __device__ __forceinline__ FoldPair fold_alias_sum2(const double4_32a *FS, int RP, int k, int shifted, int n, int q,
                                                     int L, int j0, int dj) {

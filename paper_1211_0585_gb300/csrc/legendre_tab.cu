@@ -78,7 +78,7 @@ struct MapSet {
 // registers leave two CTAs per SM), by FP32 issue with two maps (833 us for
 // both) and below Nside 512. 96 rows a CTA: 91 us at Nside 256 / lmax 512 and 816
 // at Nside 512 for two maps, against 97 and 855 with 64 and 98 and 968 with 32.
-template <int NB, bool ITER>
+template <int NB, bool ITER, bool FINE>
 __global__ void __launch_bounds__(kThreads, NB == 1 ? 3 : 2) tab_analysis_kernel(const LegArgs A, const LegDfArgs D,
                                                                                  const LegBatchMaps Bm) {
   extern __shared__ float4 fsm[];   // [NB][parity][chunk] Fourier sums E = N + S, O = N - S
@@ -159,13 +159,19 @@ __global__ void __launch_bounds__(kThreads, NB == 1 ? 3 : 2) tab_analysis_kernel
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
               const float4 f = fsm[(size_t)(2 * b + p) * nkc + kk];
-              dot2_acc(aS[b][0], aC[b][0], la, dfl{f.x, f.y});
-              dot2_acc(aS[b][1], aC[b][1], la, dfl{f.z, f.w});
-              dot2_acc(aS[b][2], aC[b][2], lb, dfl{f.x, f.y});
-              dot2_acc(aS[b][3], aC[b][3], lb, dfl{f.z, f.w});
+              dot2_acc<FINE>(aS[b][0], aC[b][0], la, dfl{f.x, f.y});
+              dot2_acc<FINE>(aS[b][1], aC[b][1], la, dfl{f.z, f.w});
+              dot2_acc<FINE>(aS[b][2], aC[b][2], lb, dfl{f.x, f.y});
+              dot2_acc<FINE>(aS[b][3], aC[b][3], lb, dfl{f.z, f.w});
             }
           }
           if (t + kAhead < ntile) load(t + kAhead, v[d]);
+        }
+        if (((tb - t0) & 7) == 6) {                    // 32 terms a sum
+#pragma unroll
+          for (int b = 0; b < NB; ++b)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) dot2_tidy(aS[b][q], aC[b][q]);
         }
       }
       // lane bits 1, 2 keep the row, re or im; bit 3 is summed over
@@ -248,7 +254,7 @@ __global__ void __launch_bounds__(kThreads, NB == 1 ? 3 : 2) tab_analysis_kernel
 // the rows from the first any of them needs, two batches of kSynRows in flight
 // in registers. Bound by HBM at Nside 512 (489 us a launch at lmax 1024, 0.96 of
 // the copy rate; 624 us for two maps), 69 us at Nside 256 / lmax 512.
-template <int NB, bool ITER>
+template <int NB, bool ITER, bool FINE>
 __global__ void __launch_bounds__(kThreads, 3) tab_synthesis_kernel(const LegArgs A, const LegDfArgs D,
                                                                                   const LegBatchMaps Bm, int nchunk) {
   extern __shared__ float4 csm[];   // [NB][nc] coefficients (re hi, re lo, im hi, im lo)
@@ -328,16 +334,22 @@ __global__ void __launch_bounds__(kThreads, 3) tab_synthesis_kernel(const LegArg
 #pragma unroll
           for (int b = 0; b < NB; ++b) {
             const float4 *c = csm + (size_t)b * nc + 2 * (r + i);
-            dot2_acc(acc[b][0], acc[b][1], dfl{e.x, e.y}, dfl{c[0].x, c[0].y});
-            dot2_acc(acc[b][2], acc[b][3], dfl{e.x, e.y}, dfl{c[0].z, c[0].w});
-            dot2_acc(acc[b][4], acc[b][5], dfl{o.x, o.y}, dfl{c[1].x, c[1].y});
-            dot2_acc(acc[b][6], acc[b][7], dfl{o.x, o.y}, dfl{c[1].z, c[1].w});
-            dot2_acc(acc[b][0], acc[b][1], dfl{e.z, e.w}, dfl{c[2].x, c[2].y});
-            dot2_acc(acc[b][2], acc[b][3], dfl{e.z, e.w}, dfl{c[2].z, c[2].w});
-            dot2_acc(acc[b][4], acc[b][5], dfl{o.z, o.w}, dfl{c[3].x, c[3].y});
-            dot2_acc(acc[b][6], acc[b][7], dfl{o.z, o.w}, dfl{c[3].z, c[3].w});
+            dot2_acc<FINE>(acc[b][0], acc[b][1], dfl{e.x, e.y}, dfl{c[0].x, c[0].y});
+            dot2_acc<FINE>(acc[b][2], acc[b][3], dfl{e.x, e.y}, dfl{c[0].z, c[0].w});
+            dot2_acc<FINE>(acc[b][4], acc[b][5], dfl{o.x, o.y}, dfl{c[1].x, c[1].y});
+            dot2_acc<FINE>(acc[b][6], acc[b][7], dfl{o.x, o.y}, dfl{c[1].z, c[1].w});
+            dot2_acc<FINE>(acc[b][0], acc[b][1], dfl{e.z, e.w}, dfl{c[2].x, c[2].y});
+            dot2_acc<FINE>(acc[b][2], acc[b][3], dfl{e.z, e.w}, dfl{c[2].z, c[2].w});
+            dot2_acc<FINE>(acc[b][4], acc[b][5], dfl{o.z, o.w}, dfl{c[3].x, c[3].y});
+            dot2_acc<FINE>(acc[b][6], acc[b][7], dfl{o.z, o.w}, dfl{c[3].z, c[3].w});
           }
         }
+      }
+      if ((r0 - rfirst) % (2 * (kAhead + 1) * kSynRows)) {   // every 24 rows
+#pragma unroll
+        for (int b = 0; b < NB; ++b)
+#pragma unroll
+          for (int q = 0; q < 8; q += 2) dot2_tidy(acc[b][q], acc[b][q + 1]);
       }
     }
   }
@@ -346,10 +358,10 @@ __global__ void __launch_bounds__(kThreads, 3) tab_synthesis_kernel(const LegArg
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
       const float4 *c = csm + (size_t)b * nc + 2 * (npr - 1);
-      dot2_acc(acc[b][0], acc[b][1], dfl{x.x, x.y}, dfl{c[0].x, c[0].y});
-      dot2_acc(acc[b][2], acc[b][3], dfl{x.x, x.y}, dfl{c[0].z, c[0].w});
-      dot2_acc(acc[b][4], acc[b][5], dfl{x.z, x.w}, dfl{c[1].x, c[1].y});
-      dot2_acc(acc[b][6], acc[b][7], dfl{x.z, x.w}, dfl{c[1].z, c[1].w});
+      dot2_acc<FINE>(acc[b][0], acc[b][1], dfl{x.x, x.y}, dfl{c[0].x, c[0].y});
+      dot2_acc<FINE>(acc[b][2], acc[b][3], dfl{x.x, x.y}, dfl{c[0].z, c[0].w});
+      dot2_acc<FINE>(acc[b][4], acc[b][5], dfl{x.z, x.w}, dfl{c[1].x, c[1].y});
+      dot2_acc<FINE>(acc[b][6], acc[b][7], dfl{x.z, x.w}, dfl{c[1].z, c[1].w});
     }
   }
   if (k < RP) {
@@ -364,7 +376,7 @@ __global__ void __launch_bounds__(kThreads, 3) tab_synthesis_kernel(const LegArg
 size_t ana_smem(int nb, int RP) { return (size_t)nb * 2 * std::min(RP, kTabChunk) * sizeof(float4); }
 size_t syn_smem(int nb, int lmax) { return (size_t)nb * 2 * (tab_rows(lmax, 0) + 1) * sizeof(float4); }
 
-template <int NB>
+template <int NB, bool FINE>
 void launch_tab(const LegArgs &a, const LegDfArgs &d, const LegBatchMaps &bm, cudaStream_t s, int mode) {
   const int nchunk = tab_chunks(a.lmax), ntile = (a.RP + 31) / 32;
   const int nw = std::min(8, ntile);
@@ -378,11 +390,11 @@ void launch_tab(const LegArgs &a, const LegDfArgs &d, const LegBatchMaps &bm, cu
     raise_smem_cap(reinterpret_cast<const void *>(kernel));
     launch_pdl(kernel, gs, 32 * nw, ss, s, a, d, bm, nchunk);
   };
-  if (mode == LEG_SYNTH) syn(tab_synthesis_kernel<NB, false>);
-  else if (mode == LEG_ANALYSIS) ana(tab_analysis_kernel<NB, false>);
+  if (mode == LEG_SYNTH) syn(tab_synthesis_kernel<NB, false, FINE>);
+  else if (mode == LEG_ANALYSIS) ana(tab_analysis_kernel<NB, false, FINE>);
   else {
-    ana(tab_analysis_kernel<NB, true>);
-    syn(tab_synthesis_kernel<NB, true>);
+    ana(tab_analysis_kernel<NB, true, FINE>);
+    syn(tab_synthesis_kernel<NB, true, FINE>);
   }
 }
 
@@ -394,8 +406,10 @@ size_t leg_tab_smem(int lmax, int RP) { return std::max(ana_smem(1, RP), syn_sme
 
 void launch_legendre_tab(const LegArgs &a, const LegDfArgs &d, const LegBatchMaps &bm, int nb, cudaStream_t s,
                          int mode) {
-  if (nb == 1) launch_tab<1>(a, d, bm, s, mode);
-  else launch_tab<2>(a, d, bm, s, mode);
+  // sums of few terms in the finer steps (dot2_acc): up to Nside 64 latency, not FP32 issue, bounds these kernels
+  const bool fine = a.RP <= 128;
+  if (nb == 1) fine ? launch_tab<1, true>(a, d, bm, s, mode) : launch_tab<1, false>(a, d, bm, s, mode);
+  else fine ? launch_tab<2, true>(a, d, bm, s, mode) : launch_tab<2, false>(a, d, bm, s, mode);
 }
 
 }  // namespace wfk

@@ -229,6 +229,7 @@ __device__ __forceinline__ dfl warp_sum8_df(float (&S)[8], float (&C)[8]) {
 // warp and one step of loads ahead: 2.28 ms a launch at Nside 512 / lmax 1024 and
 // 156 us at Nside 128 / lmax 256; now 1.51 ms and 47 us (1.80 and 54 before the
 // loop over tiles was counted, without a search and moves a step).
+template <bool FINE>
 __global__ void __launch_bounds__(kPolThreads, 3) spin2_analysis_df_kernel(const Ctl *gate, const float4 *tab,
                                                                             const int *ls, const double4_32a *FTQ,
                                                                             const double4_32a *FTU, int lmax, int RP,
@@ -274,25 +275,25 @@ __global__ void __launch_bounds__(kPolThreads, 3) spin2_analysis_df_kernel(const
       // -a^E = F+ Q+ + i F- U-,  -a^B = F+ U+ - i F- Q-
       {   // l: Q+ = A, Q- = Bq, U+ = Cu, U- = Du
         const dfl fp = {f0.x, f0.y}, fm = {f0.z, f0.w}, fn = df_neg(fm);
-        dot2_acc(S[0], C[0], fp, dfl{A.x, A.y});
-        dot2_acc(S[0], C[0], fn, dfl{Du.z, Du.w});
-        dot2_acc(S[1], C[1], fp, dfl{A.z, A.w});
-        dot2_acc(S[1], C[1], fm, dfl{Du.x, Du.y});
-        dot2_acc(S[2], C[2], fp, dfl{Cu.x, Cu.y});
-        dot2_acc(S[2], C[2], fm, dfl{Bq.z, Bq.w});
-        dot2_acc(S[3], C[3], fp, dfl{Cu.z, Cu.w});
-        dot2_acc(S[3], C[3], fn, dfl{Bq.x, Bq.y});
+        dot2_acc<FINE>(S[0], C[0], fp, dfl{A.x, A.y});
+        dot2_acc<FINE>(S[0], C[0], fn, dfl{Du.z, Du.w});
+        dot2_acc<FINE>(S[1], C[1], fp, dfl{A.z, A.w});
+        dot2_acc<FINE>(S[1], C[1], fm, dfl{Du.x, Du.y});
+        dot2_acc<FINE>(S[2], C[2], fp, dfl{Cu.x, Cu.y});
+        dot2_acc<FINE>(S[2], C[2], fm, dfl{Bq.z, Bq.w});
+        dot2_acc<FINE>(S[3], C[3], fp, dfl{Cu.z, Cu.w});
+        dot2_acc<FINE>(S[3], C[3], fn, dfl{Bq.x, Bq.y});
       }
       {   // l + 1: Q+ = Bq, Q- = A, U+ = Du, U- = Cu
         const dfl fp = {f1.x, f1.y}, fm = {f1.z, f1.w}, fn = df_neg(fm);
-        dot2_acc(S[4], C[4], fp, dfl{Bq.x, Bq.y});
-        dot2_acc(S[4], C[4], fn, dfl{Cu.z, Cu.w});
-        dot2_acc(S[5], C[5], fp, dfl{Bq.z, Bq.w});
-        dot2_acc(S[5], C[5], fm, dfl{Cu.x, Cu.y});
-        dot2_acc(S[6], C[6], fp, dfl{Du.x, Du.y});
-        dot2_acc(S[6], C[6], fm, dfl{A.z, A.w});
-        dot2_acc(S[7], C[7], fp, dfl{Du.z, Du.w});
-        dot2_acc(S[7], C[7], fn, dfl{A.x, A.y});
+        dot2_acc<FINE>(S[4], C[4], fp, dfl{Bq.x, Bq.y});
+        dot2_acc<FINE>(S[4], C[4], fn, dfl{Cu.z, Cu.w});
+        dot2_acc<FINE>(S[5], C[5], fp, dfl{Bq.z, Bq.w});
+        dot2_acc<FINE>(S[5], C[5], fm, dfl{Cu.x, Cu.y});
+        dot2_acc<FINE>(S[6], C[6], fp, dfl{Du.x, Du.y});
+        dot2_acc<FINE>(S[6], C[6], fm, dfl{A.z, A.w});
+        dot2_acc<FINE>(S[7], C[7], fp, dfl{Du.z, Du.w});
+        dot2_acc<FINE>(S[7], C[7], fn, dfl{A.x, A.y});
       }
     };
     float4 f[2][2];
@@ -305,6 +306,10 @@ __global__ void __launch_bounds__(kPolThreads, 3) spin2_analysis_df_kernel(const
         if (t >= ntile) break;
         term(t, f[d][0], f[d][1]);
         if (t + 2 < ntile) load(t + 2, f[d][0], f[d][1]);
+      }
+      if (((tb - t0) & 15) == 14) {   // 32 terms a sum (two a tile)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) dot2_tidy(S[j], C[j]);
       }
     }
     const dfl v = warp_sum8_df(S, C);
@@ -338,6 +343,7 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+template <bool FINE>
 __global__ void __launch_bounds__(kPolThreads, 3) spin2_synthesis_df_kernel(const Ctl *gate, const float4 *tab,
                                                                              const int *ls, const double2 *aE,
                                                                              const double2 *aB, int lmax, int RP,
@@ -373,14 +379,14 @@ __global__ void __launch_bounds__(kPolThreads, 3) spin2_synthesis_df_kernel(cons
     const dfl fp = {f.x, f.y}, fm = {f.z, f.w};
     const float4 E = coef[2 * i], Bv = coef[2 * i + 1];
     const dfl er = {E.x, E.y}, ei = {E.z, E.w}, br = {Bv.x, Bv.y}, bi = {Bv.z, Bv.w};
-    dot2_acc(Sa[0], Ca[0], fp, er);
-    dot2_acc(Sa[1], Ca[1], fm, bi);
-    dot2_acc(Sa[2], Ca[2], fp, ei);
-    dot2_acc(Sa[3], Ca[3], fm, br);
-    dot2_acc(Sa[4], Ca[4], fp, br);
-    dot2_acc(Sa[5], Ca[5], fm, ei);
-    dot2_acc(Sa[6], Ca[6], fp, bi);
-    dot2_acc(Sa[7], Ca[7], fm, er);
+    dot2_acc<FINE>(Sa[0], Ca[0], fp, er);
+    dot2_acc<FINE>(Sa[1], Ca[1], fm, bi);
+    dot2_acc<FINE>(Sa[2], Ca[2], fp, ei);
+    dot2_acc<FINE>(Sa[3], Ca[3], fm, br);
+    dot2_acc<FINE>(Sa[4], Ca[4], fp, br);
+    dot2_acc<FINE>(Sa[5], Ca[5], fm, ei);
+    dot2_acc<FINE>(Sa[6], Ca[6], fp, bi);
+    dot2_acc<FINE>(Sa[7], Ca[7], fm, er);
   };
   const int istart = m < 2 ? 2 - m : 0;   // rows of l < 2 hold zeros; their coefficients may be anything
   for (int ib = i0; ib < Lm; ib += kSynDepth) {
@@ -394,6 +400,10 @@ __global__ void __launch_bounds__(kPolThreads, 3) spin2_synthesis_df_kernel(cons
       if (i + 1 < Lm && i + 1 >= istart) accum(i + 1, f1, S1, C1);
       fetch(i + kSynDepth, j);          // into the places just used
     }
+    if (((ib - i0) & 31) == 24) {   // 16 terms a sum
+#pragma unroll
+      for (int j = 0; j < 8; ++j) { dot2_tidy(S0[j], C0[j]); dot2_tidy(S1[j], C1[j]); }
+    }
   }
   cp_wait<0>();
   if (k >= RP) return;
@@ -404,9 +414,9 @@ __global__ void __launch_bounds__(kPolThreads, 3) spin2_synthesis_df_kernel(cons
     o[j] = df_norm(S1[j], C1[j]);
   }
   // sums over both parities (p) and their difference (d)
-  auto p = [&](int j) { return df_add(e[j], o[j]); };
-  auto d = [&](int j) { return df_add(e[j], df_neg(o[j])); };
-  auto put = [](dfl x, dfl y) { return df_pack(df_neg(df_add(x, y))); };
+  auto p = [&](int j) { return df_add2(e[j], o[j]); };
+  auto d = [&](int j) { return df_add2(e[j], df_neg(o[j])); };
+  auto put = [](dfl x, dfl y) { return df_pack(df_neg(df_add2(x, y))); };
   // north: Q = -(F+ E + i F- B), U = -(F+ B - i F- E); south: F+ -> p F+, F- -> -p F-
   FSQ[(size_t)m * RP + k] = make_double4_32a(put(p(0), df_neg(p(1))), put(p(2), p(3)), put(d(0), d(1)),
                                              put(d(2), df_neg(d(3))));
@@ -585,12 +595,13 @@ void Pol::synth(cudaStream_t s, const double2 *alm, double *map, const Ctl *gate
   la.gate = gate;
   P->launch_leg(la, s, LEG_SYNTH);                                    // T -> the plan's FS
   if (df) {
-    raise_smem_cap(reinterpret_cast<const void *>(spin2_synthesis_df_kernel));
+    auto kernel = RP <= 128 ? spin2_synthesis_df_kernel<true> : spin2_synthesis_df_kernel<false>;   // short sums in the finer steps
+    raise_smem_cap(reinterpret_cast<const void *>(kernel));
     // half of the ring pairs a CTA up to 256 of them: enough CTAs where few values of m do not fill the chip,
     // and the coefficients (whose conversion is FP64 work) read by few
     const int nt = std::min(kPolThreads, std::max(32, (RP / 2 + 31) / 32 * 32));
     const dim3 grid(lmax + 1, (RP + nt - 1) / nt);
-    spin2_synthesis_df_kernel<<<grid, nt, sizeof(float4) * (kSynDepth * nt + 2 * (size_t)(lmax + 1)), s>>>(
+    kernel<<<grid, nt, sizeof(float4) * (kSynDepth * nt + 2 * (size_t)(lmax + 1)), s>>>(
         gate, reinterpret_cast<const float4 *>(d_tab), P->d_ls, alm + nalm, alm + 2 * nalm, lmax, RP, d_FSQ, d_FSU);
   } else {
     raise_smem_cap(reinterpret_cast<const void *>(spin2_synthesis_kernel));
@@ -630,11 +641,12 @@ void Pol::analysis(cudaStream_t s, const double *map, double2 *alm, const Ctl *g
   la.gate = gate;
   P->launch_leg(la, s, LEG_ANALYSIS);                                 // T
   if (df) {
-    raise_smem_cap(reinterpret_cast<const void *>(spin2_analysis_df_kernel));
+    auto kernel = RP <= 128 ? spin2_analysis_df_kernel<true> : spin2_analysis_df_kernel<false>;   // short sums in the finer steps
+    raise_smem_cap(reinterpret_cast<const void *>(kernel));
     // 64 values of l a CTA (four row pairs a warp), 16 where lmax leaves few chunks
     const int lchunk = lmax >= 256 ? 64 : 16;
     const dim3 grid(lmax + 1, (lmax + lchunk) / lchunk);
-    spin2_analysis_df_kernel<<<grid, kPolThreads, sizeof(float4) * 4 * RP + sizeof(int) * ((RP + 31) / 32), s>>>(
+    kernel<<<grid, kPolThreads, sizeof(float4) * 4 * RP + sizeof(int) * ((RP + 31) / 32), s>>>(
         gate, reinterpret_cast<const float4 *>(d_tab), P->d_ls, d_FTQ, d_FTU, lmax, RP, lchunk, alm + nalm,
         alm + 2 * nalm);
   } else {

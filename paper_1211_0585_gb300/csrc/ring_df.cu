@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingAr
   if (MODE == RING_SYNTH || MODE == RING_ITER) {
     // Z = G_N + i G_S
     fold_ring2(Q.FS, A.RP, k, rg.shifted, n, L, fold_part, [&](int q, float4 gN, float4 gS) {
-      float4 acc = df_pair(df_add(RE(gN), df_neg(IM(gS))), df_add(IM(gN), RE(gS)));
+      float4 acc = df_pair(df_add2(RE(gN), df_neg(IM(gS))), df_add2(IM(gN), RE(gS)));
       if (rg.shifted) acc = cmul(acc, hs[q]);
       buf[px<OpsDF>(q)] = rg.blue ? cmul(cconj(acc), ch[q]) : acc;
     });
@@ -157,8 +157,8 @@ __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingAr
       }
       const dfl res = df_add(dv, df_neg(s));
       const dfl r2 = df_mul(res, res);
-      dot2_acc(cs[2 * half], cc[2 * half], wv, r2);
-      dot2_acc(cs[2 * half + 1], cc[2 * half + 1], g, r2);
+      dot2_acc<true>(cs[2 * half], cc[2 * half], wv, r2);
+      dot2_acc<true>(cs[2 * half + 1], cc[2 * half + 1], g, r2);
       return df_mul(df_mul(ltd, g), res);
     };
     for (int p = threadIdx.x; p < n; p += blockDim.x) {
@@ -220,8 +220,8 @@ __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingAr
       if (j & 1) { UN = cneg(UN); US = cneg(US); }
     }
     Q.FT[(size_t)m * A.RP + k] = make_double4_32a(
-        df_pack(df_mul(RE(UN), om)), df_pack(df_mul(IM(UN), om)), two ? df_pack(df_mul(RE(US), om)) : 0.0,
-        two ? df_pack(df_mul(IM(US), om)) : 0.0);
+        df_pack(df_mul2(RE(UN), om)), df_pack(df_mul2(IM(UN), om)), two ? df_pack(df_mul2(RE(US), om)) : 0.0,
+        two ? df_pack(df_mul2(IM(US), om)) : 0.0);
   }
 }
 
