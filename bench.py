@@ -158,11 +158,11 @@ def make_problem(seed):
     return I.wmap_problem(seed=seed, nside=NSIDE, lmax=LMAX)
 
 
-LEGENDRE_DF_INSTR = 90    # FP32 instructions per evaluated (l, m, ring pair) term, both passes
-# DRAM bytes (read + write) per algorithmic byte of legendre_df_kernel<LEG_ITER, table>: 885.0 MB
-# measured by ncu for one launch of `bench.py --profile-fp64 256 512 4` against 864.0 MB algorithmic;
-# the full-size launch is scaled by it
-TABLE_TRAFFIC_RATIO = 885.04e6 / 864049664
+LEGENDRE_DF_INSTR = 74    # FP32 instructions per evaluated (l, m, ring pair) term, both passes
+# DRAM bytes (read + write) per algorithmic byte of an iteration's tab_analysis_kernel and
+# tab_synthesis_kernel launches: 892.1 MB measured by ncu at Nside 256 / lmax 512 against 864.0 MB
+# algorithmic; the full-size launches are scaled by it
+TABLE_TRAFFIC_RATIO = 892.1e6 / 864049664
 
 
 def run_ours(args):
@@ -218,8 +218,10 @@ def run_ours(args):
     graph_iters = opts.graph_iters
     per_iter = P.kernels_per_iteration()
     # the iterations' graphs (controller-stopped launches return at once but count), then the posterior
-    # gradient: one synthesis, the pixel kernel, two analyses, the norms (r = ring-stage launches)
-    r = per_iter - 2
+    # gradient: one synthesis, the pixel kernel, two analyses, the norms (r = ring-stage launches; the
+    # Legendre stage is two launches an iteration with the table, one without, the controller one)
+    held, per_pass = P.legendre_table(LMAX)
+    r = per_iter - (3 if held else 2)
     posterior = (5 + 3 * r) if opts.posterior_grad else 0
     launches_per_solve = [math.ceil(i / graph_iters) * graph_iters * per_iter + posterior for i in iters]
 
@@ -243,12 +245,11 @@ def run_ours(args):
     s_prof = out.clone()
     prof = P.profile(dmap.data_ptr(), s_prof.data_ptr(), 1.0, LMAX, 10)
     evaluated, full = P.legendre_terms(LMAX)
-    held, per_pass = P.legendre_table(LMAX)
     alu = {} if held else measure_alu_peaks()   # the ALU-bound forms' denominators
     fp32_peak = alu.get("fp32_tflops") or 75.3
     # the double-float Legendre kernel: per evaluated (l, m, ring pair) term, one
-    # recurrence step (19 FP32 instructions) and two compensated multiply-adds
-    # (13 each) in each of the analysis and synthesis passes = 90 FP32
+    # recurrence step (17 FP32 instructions) and two compensated multiply-adds
+    # (10 each) in each of the analysis and synthesis passes = 74 FP32
     # instructions; each counted as 2 flops against the FP32 FMA peak
     t_leg = prof["legendre"] * 1e-3
     if held:
@@ -260,7 +261,7 @@ def run_ours(args):
         nbytes = (2 * per_pass + (LMAX + 1) * rp * 32 * 2 + (LMAX + 1) * rp * 4 * 2 + P.nalm * 16 * 2)
         hbm_peak, src = hbm_peak_gbs()
         achieved = nbytes / t_leg / 1e9
-        roofline = {"bound": "hbm", "kernel": "legendre_df_kernel<LEG_ITER, table> (double-float lambda table)",
+        roofline = {"bound": "hbm", "kernel": "tab_analysis_kernel + tab_synthesis_kernel (double-float lambda table)",
                     "achieved": round(achieved, 1), "peak": hbm_peak, "unit": "GB/s",
                     "frac": round(achieved / hbm_peak, 4), "traffic": int(TABLE_TRAFFIC_RATIO * nbytes),
                     "traffic_source": "ncu DRAM bytes of the same kernel at Nside 256 / lmax 512, scaled by "

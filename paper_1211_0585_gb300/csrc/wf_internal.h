@@ -7,7 +7,7 @@
 //              m = 0 .. lmax, the azimuthal coefficients of ring pair k.
 //              FS: synthesis side (from a_lm), FT: analysis side (to a_lm).
 //              Native FP64 stages hold doubles; the double-float stages (ring_df,
-//              legendre_df, legendre_batch, spin-2) hold each value as its (hi, lo)
+//              legendre_df, legendre_tab, spin-2) hold each value as its (hi, lo)
 //              floats in the same 8 bytes (df_pack).
 //   a_lm       m-major complex doubles, index(l, m) = m (2 lmax + 1 - m) / 2 + l.
 //   maps       RING order doubles.
