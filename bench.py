@@ -264,7 +264,7 @@ def run_ours(args):
         roofline = {"bound": "hbm", "kernel": "tab_analysis_kernel + tab_synthesis_kernel (double-float lambda table)",
                     "achieved": round(achieved, 1), "peak": hbm_peak, "unit": "GB/s",
                     "frac": round(achieved / hbm_peak, 4), "traffic": int(TABLE_TRAFFIC_RATIO * nbytes),
-                    "traffic_source": "ncu DRAM bytes of the same kernel at Nside 256 / lmax 512, scaled by "
+                    "traffic_source": "ncu DRAM bytes of the same kernels at Nside 256 / lmax 512, scaled by "
                                       "the algorithmic bytes",
                     "per_launch_ms": round(prof["legendre"], 4), "algorithmic_bytes_per_launch": nbytes,
                     "table_bytes_held": held, "table_bytes_per_pass": per_pass,
