@@ -407,7 +407,8 @@ size_t leg_tab_smem(int lmax, int RP) { return std::max(ana_smem(1, RP), syn_sme
 void launch_legendre_tab(const LegArgs &a, const LegDfArgs &d, const LegBatchMaps &bm, int nb, cudaStream_t s,
                          int mode) {
   // Sums of few terms in the finer steps (dot2_acc). Up to Nside 64 latency bounds these kernels and the two more
-  // instructions are free (Nside 16: 21 us an iteration either way, error 4.9 instead of 5.5e-15); with the line at
+  // instructions cost little (an Nside 16 solve 1 to 2 %, the FFT's longer product included; error 4.9 instead
+  // of 5.5e-15); with the line at
   // Nside 128 a T + P solve there, bound by FP32 issue in the same sums (pol.cu), takes 68 instead of 62 ms, and
   // dot2_tidy does as much for its error (7.3e-15 against 9.9e-15)
   const bool fine = a.RP <= 128;
