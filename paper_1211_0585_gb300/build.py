@@ -38,7 +38,8 @@ def _stale() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(INCLUDE, "*.h"))
+    deps = sources() + [p for d, pat in ((CSRC, "*.h"), (CSRC, "*.cuh"), (INCLUDE, "*.h"))
+                        for p in glob.glob(os.path.join(d, pat))]
     return any(os.path.getmtime(p) > t for p in deps)
 
 
