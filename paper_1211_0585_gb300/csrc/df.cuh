@@ -107,10 +107,11 @@ __device__ __forceinline__ void dot2_acc(float &S, float &C, dfl a, dfl b) {
 }
 
 // The collected errors of a long compensated sum moved into its leading part: the next ones round at a small C's ulp
-// again (every 32 terms or so the error of a sum of 512 falls by two)
+// again (every 32 terms or so the error of a sum of 512 falls by two). two_sum, exact also where the terms cancelled
+// and |C| > |S|: folding a sum that has ended once more, as a launch for a longer one beside it does, changes nothing.
 __device__ __forceinline__ void dot2_tidy(float &S, float &C) {
-  const float s = S + C;
-  C -= s - S;
+  const float s = S + C, bb = s - S;
+  C = (S - (s - bb)) + (C - bb);
   S = s;
 }
 

@@ -118,7 +118,10 @@ __global__ void __launch_bounds__(kThreads, NB == 1 ? 3 : 2) tab_analysis_kernel
       while (t < ntile && tmin[t] > l) ++t;
       return t;
     };
-    for (int kk = 32 * first_tile(m + 2 * rend + 1) + threadIdx.x; kk < nk; kk += kThreads) {
+    // a group of rows is taken from the tile of its own last l, whatever band limits share the launch: where its sums are
+    // folded back (dot2_tidy) then depends on the map alone
+    auto first_of_group = [&](int rg) { return first_tile(m + 2 * (r0 + 4 * rg) + 7); };
+    for (int kk = 32 * first_of_group((rend - r0) >> 2) + threadIdx.x; kk < nk; kk += kThreads) {
 #pragma unroll
       for (int b = 0; b < NB; ++b) {
         float4 e = make_float4(0.f, 0.f, 0.f, 0.f), o = e;
@@ -143,7 +146,7 @@ __global__ void __launch_bounds__(kThreads, NB == 1 ? 3 : 2) tab_analysis_kernel
 #pragma unroll
         for (int q = 0; q < 4; ++q) { aS[b][q] = 0.f; aC[b][q] = 0.f; }
       float4 v[kAhead][4];                             // tiles in flight
-      const int t0 = first_tile(min(m + 2 * (r0 + 4 * rg) + 7, m + 2 * rend + 1));
+      const int t0 = first_of_group(rg);
 #pragma unroll
       for (int d = 0; d < kAhead; ++d)
         if (t0 + d < ntile) load(t0 + d, v[d]);
