@@ -261,16 +261,20 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) legendre_df_kernel(cons
     // share to t_l
     for (int k0 = 0; k0 < RP; k0 += kAnaChunk<NT>) {
       const int nk = min(kAnaChunk<NT>, RP - k0);
+      const int np = (nk + 31) & ~31;              // whole warps: a lane past the last ring pair has a state of its own
       float4 *stE = ss;                            // (Er, Ei) as hi/lo
-      float4 *stO = stE + nk;                      // (Or, Oi)
-      float4 *stP = stO + nk;                      // (p1, p2)
-      float2 *stX = reinterpret_cast<float2 *>(stP + nk);  // x as double-float
-      for (int kk = threadIdx.x; kk < nk; kk += blockDim.x) {
-        const int k = k0 + kk;
-        const double4_32a t = A.FT[(size_t)m * RP + k];
+      float4 *stO = stE + np;                      // (Or, Oi)
+      float4 *stP = stO + np;                      // (p1, p2)
+      float2 *stX = reinterpret_cast<float2 *>(stP + np);  // x as double-float
+      for (int kk = threadIdx.x; kk < np; kk += blockDim.x) {
+        double4_32a t = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+        dfl xk{0.f, 0.f};
+        if (kk < nk) {
+          t = A.FT[(size_t)m * RP + k0 + kk];
+          xk = df_from(A.x[k0 + kk]);
+        }
         f_parities(t, stE[kk], stO[kk]);
         stP[kk] = make_float4(0.f, 0.f, 0.f, 0.f);
-        const dfl xk = df_from(A.x[k]);
         stX[kk] = make_float2(xk.h, xk.l);
       }
       __syncthreads();
@@ -289,7 +293,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) legendre_df_kernel(cons
         for (int i = 0; i < 4; ++i) {
           // the whole warp runs the same block: lanes without a term yet carry zeros, and one with a start value in
           // it takes the others through the injecting form (as per-lane branches the two forms ran one after the other)
-          const int ls = lsr[i], kk = min((int)threadIdx.x + i * NT, nk - 1);
+          const int ls = lsr[i], kk = threadIdx.x + i * NT;
           const bool begun = ls < l0 + kDB;
           if (!__any_sync(0xffffffffu, begun)) continue;
           const bool starts = begun && ls + 1 >= l0;
@@ -442,8 +446,8 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) legendre_df_kernel(cons
 // coefficients, or the per-ring-pair analysis state of one chunk)
 static size_t leg_df_smem(int lmax, int RP, int chunk) {
   const size_t Lp = (size_t)lmax + 1 + kLB;
-  const size_t nk = RP < chunk ? (size_t)RP : (size_t)chunk;
-  const size_t st = 3 * nk + (nk + 1) / 2;
+  const size_t np = ((RP < chunk ? (size_t)RP : (size_t)chunk) + 31) / 32 * 32;
+  const size_t st = 3 * np + np / 2;
   const size_t q = Lp > st ? Lp : st;
   return Lp * sizeof(double2) + (Lp + 1) * sizeof(float2) + q * sizeof(float4) + 16;
 }
