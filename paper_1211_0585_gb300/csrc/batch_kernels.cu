@@ -52,8 +52,8 @@ __device__ __forceinline__ void prefetch_l2(const void *p) {
 // forward transform's input order), and the G slots read their Fourier
 // coefficients as one contiguous run of G float4. Four CTAs of 256 threads per
 // SM (64 registers), so that the FFT passes of one CTA overlap the global loads
-// and stores of the others. ND = 1, a CTA per ring, serves the rings whose two
-// FFT buffers do not fit shared memory (Nside 2048).
+// and stores of the others. ND = 1, a CTA per ring, serves the longest rings of Nside 1024
+// and 2048, whose two buffers leave an SM one CTA or none (bring_sides).
 constexpr int kBringThreads = 256;
 template <int G, int ND>
 __global__ void __launch_bounds__(kBringThreads, 4) bring_kernel(const BatchArgs A) {
@@ -466,8 +466,9 @@ static size_t bring_smem(int logM, int G, int nd) {
 
 constexpr size_t kBringSmemMax = 200 * 1024;
 
-// both rings of a pair in a CTA where two slots of them fit
-static int bring_sides(int logM) { return bring_smem(logM, 2, 2) <= kBringSmemMax ? 2 : 1; }
+// both rings of a pair in a CTA where two slots of them leave room for a second CTA on the SM: with 128 KB a CTA (the
+// 8192-point rings of Nside 1024) 8 iterations of 16 slots at lmax 2048 took 36.7 ms, a CTA per ring 30.9
+static int bring_sides(int logM) { return bring_smem(logM, 2, 2) <= 100 * 1024 ? 2 : 1; }
 
 // default slots per ring-stage CTA of a class (before autotuning): 8, 4 or 2
 // (pairs share one FFT), within a quarter of an SM's shared memory so that four
@@ -501,7 +502,8 @@ void launch_batch_ring_class(const BatchArgs &a, const RingClass &c, int G, cuda
     else if (G == 4) launch_bring<4, 2>(a, c, s);
     else launch_bring<2, 2>(a, c, s);
   } else {
-    launch_bring<2, 1>(a, c, s);   // buffers over 100 KB a side: two slots at most
+    if (G == 4) launch_bring<4, 1>(a, c, s);
+    else launch_bring<2, 1>(a, c, s);
   }
 }
 
