@@ -1,10 +1,17 @@
 // One step of the Sect. 3 schedule on a controller state, shared by the
-// single-map controller (control.cu) and the per-slot batched controller.
+// single-map controller (control.cu) and the per-slot batched controller; and
+// what the joint Eq. 4 kernels share.
 #pragma once
 
 #include "wf_internal.h"
 
 namespace wfk {
+
+// whether 1 / x is a normal number, a safe way in from the ends of the range (by the exponent bits: no work for the FP64
+// pipe): a product with it may then stand for a quotient
+__device__ __forceinline__ bool has_reciprocal(double x) {
+  return (((unsigned)__double2hiint(x) >> 20) & 0x7ff) - 64u < 1920u;
+}
 
 __device__ __forceinline__ double ctl_lambda_for(const Ctl *c, const double *cl, int l_iter) {
   if (l_iter > c->lmax) return 1.0;

@@ -125,9 +125,15 @@ __global__ void multi_eq4_kernel(const Ctl *ctl, int K, int lmax, long long nalm
         ny = fma(gb, fma(b, so.y, t.y), ny);
         den = fma(gb, b, den);
       }
-      const double r = 1.0 / den;
-      sn = make_double2(nx * r, ny * r);
-      c2 += wgt * (so.x * so.x + so.y * so.y) * ic;
+      const double a2 = wgt * (so.x * so.x + so.y * so.y);
+      if (has_reciprocal(c) && has_reciprocal(den)) {
+        const double r = 1.0 / den;
+        sn = make_double2(nx * r, ny * r);
+        c2 += a2 * ic;
+      } else {                       // a subnormal C_l: 1 / C_l is infinite, the quotient is not
+        sn = make_double2(nx / den, ny / den);
+        c2 += a2 / c;
+      }
     }
     const double dx = sn.x - so.x, dy = sn.y - so.y;
     inc += wgt * (dx * dx + dy * dy);
