@@ -38,6 +38,7 @@
 #include <string>
 #include <vector>
 
+#include "ctl.cuh"
 #include "df.cuh"
 #include "wf_internal.h"
 #include "wf_plan.h"
@@ -480,8 +481,8 @@ __global__ void __launch_bounds__(kPolThreads) pol_pixel_kernel(const Ctl *ctl, 
 }
 
 // Eq. 4 with the (T, E) block and B, the prior chi^2 of the input state, increment and norm per m. Bound by the FP64
-// pipe: a reciprocal each of the block's determinant, of S's and of C_BB + k and C_BB, and products with them (a
-// division an element: 22 us at Nside 128 / lmax 256; now 17)
+// pipe: the block's four elements are products with the reciprocal of its determinant, where that is a normal number
+// (a division each: 22 us at Nside 128 / lmax 256; now 17)
 __global__ void __launch_bounds__(128) pol_eq4_kernel(const Ctl *ctl, int lmax, long long nalm, double tau,
                                                        double omega, const double *cls, const double2 *ta,
                                                        double2 *s, double *m_part) {
@@ -501,9 +502,14 @@ __global__ void __launch_bounds__(128) pol_eq4_kernel(const Ctl *ctl, int lmax, 
     const double tt = TT[l], ee = EE[l], bb = BB[l], te = TE[l];
     // S (S + k)^-1 on (T, E)
     const double a11 = tt + k, a12 = te, a22 = ee + k, det = a11 * a22 - a12 * a12;
-    const double rd = 1.0 / det;
-    const double m11 = (tt * a22 - te * a12) * rd, m12 = (-tt * a12 + te * a11) * rd;
-    const double m21 = (te * a22 - ee * a12) * rd, m22 = (-te * a12 + ee * a11) * rd;
+    double m11 = tt * a22 - te * a12, m12 = -tt * a12 + te * a11;
+    double m21 = te * a22 - ee * a12, m22 = -te * a12 + ee * a11;
+    if (has_reciprocal(det)) {
+      const double rd = 1.0 / det;
+      m11 *= rd; m12 *= rd; m21 *= rd; m22 *= rd;
+    } else {
+      m11 /= det; m12 /= det; m21 /= det; m22 /= det;
+    }
     const double fb = bb > 0.0 ? bb / (bb + k) : 0.0;
     const double2 nT = make_double2(m11 * tT.x + m12 * tE.x, m11 * tT.y + m12 * tE.y);
     const double2 nE = make_double2(m21 * tT.x + m22 * tE.x, m21 * tT.y + m22 * tE.y);

@@ -34,3 +34,25 @@ def test_joint_filter_of_a_spectrum_that_fades_through_the_subnormals(precision)
     assert np.linalg.norm(got[0][0] - got[1][0]) <= 1e-12 * np.linalg.norm(got[1][0])
     # chi^2 of 14 faint modes with s = C_l x: C_l x^2, nothing
     np.testing.assert_allclose(got[0][1], got[1][1], rtol=1e-12)
+
+
+def test_polarised_filter_far_below_unit_scale():
+    """Spectra and noise times 2^-514, data times 2^-257: the same filter scaled by 2^-257, although the determinants of
+    Eq. 4 (about 2^-1028) are subnormal. Bar 1e-11: their last bit is 2^-46 of them (1.4e-14), met a few times in each of
+    five iterations."""
+    nside, lmax = 4, 9
+    npix = 12 * nside * nside
+    rng = np.random.default_rng(6)
+    tt = 1.0 / (1.0 + 0.1 * np.arange(lmax + 1))
+    cls = np.stack([tt, 0.8 * tt, 0.7 * tt, 0.3 * tt])
+    cov = np.tile([1.0, 1.2, 0.1, 1.1], (npix, 1)) * (1.0 + rng.random((npix, 1)))
+    d = rng.standard_normal((3, npix))
+    out = []
+    for e in (0, -257):
+        P = wf.Pol(nside, lmax, list(cls * 2.0 ** (2 * e)), cov * 2.0 ** (2 * e),
+                   opts=wf.options(precision=wf.WF_PREC_FP64_NATIVE, tol=0.0, max_iter=5, cooling=0))
+        alm, st, _, _ = P.solve(d * 2.0 ** e)
+        assert st["iters"] == 5
+        out.append(alm * 2.0 ** -e)
+        P.close()
+    assert np.linalg.norm(out[1] - out[0]) <= 1e-11 * np.linalg.norm(out[0])
