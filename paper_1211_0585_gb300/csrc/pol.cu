@@ -98,16 +98,22 @@ __global__ void spin2_table_kernel(const double *xk, const double2 *rec, const i
   }
 }
 
+// A launch of the spin-2 analyses takes nk <= kSpin2Pairs ring pairs (64 bytes of shared memory each; 128 KB), from the
+// one that tab, ls and the Fourier records point at; RP stays their stride. The launches after the first (Nside 2048) add
+// to a^E and a^B.
+constexpr int kSpin2Pairs = 2048;
+
 // spin-2 analysis: (a^E, a^B)_lm = - sum over ring pairs of the F+- terms; one CTA per m,
 // a warp per l, lanes over ring pairs
 __global__ void __launch_bounds__(kPolThreads) spin2_analysis_kernel(const Ctl *gate, const double2 *tab,
                                                                       const double4_32a *FTQ, const double4_32a *FTU,
-                                                                      int lmax, int RP, double2 *aE, double2 *aB) {
+                                                                      int lmax, int RP, int nk, int add, double2 *aE,
+                                                                      double2 *aB) {
   if (gate && gate->done) return;
   extern __shared__ double4_32a pol_sm[];
-  double4_32a *q = pol_sm, *u = pol_sm + RP;
+  double4_32a *q = pol_sm, *u = pol_sm + nk;
   const int m = blockIdx.x;
-  for (int k = threadIdx.x; k < RP; k += blockDim.x) {
+  for (int k = threadIdx.x; k < nk; k += blockDim.x) {
     q[k] = FTQ[(size_t)m * RP + k];
     u[k] = FTU[(size_t)m * RP + k];
   }
@@ -118,7 +124,7 @@ __global__ void __launch_bounds__(kPolThreads) spin2_analysis_kernel(const Ctl *
     const double p = ((l - m) & 1) ? -1.0 : 1.0;
     double er = 0.0, ei = 0.0, br = 0.0, bi = 0.0;
     const double2 *row = tab + (base + (l - m)) * RP;
-    for (int k = lane; k < RP; k += 32) {
+    for (int k = lane; k < nk; k += 32) {
       const double2 f = row[k];
       const double4_32a Q = q[k], U = u[k];
       // F+ sees Q_N + p Q_S, U_N + p U_S; F- sees Q_N - p Q_S, U_N - p U_S
@@ -137,8 +143,10 @@ __global__ void __launch_bounds__(kPolThreads) spin2_analysis_kernel(const Ctl *
       bi += __shfl_xor_sync(0xffffffffu, bi, o);
     }
     if (lane == 0) {
-      aE[base + (l - m)] = l >= 2 ? make_double2(er, ei) : make_double2(0.0, 0.0);
-      aB[base + (l - m)] = l >= 2 ? make_double2(br, bi) : make_double2(0.0, 0.0);
+      double2 &E = aE[base + (l - m)], &B = aB[base + (l - m)];
+      if (add) { er += E.x; ei += E.y; br += B.x; bi += B.y; }
+      E = l >= 2 ? make_double2(er, ei) : make_double2(0.0, 0.0);
+      B = l >= 2 ? make_double2(br, bi) : make_double2(0.0, 0.0);
     }
   }
 }
@@ -234,26 +242,27 @@ template <bool FINE>
 __global__ void __launch_bounds__(kPolThreads, 3) spin2_analysis_df_kernel(const Ctl *gate, const float4 *tab,
                                                                             const int *ls, const double4_32a *FTQ,
                                                                             const double4_32a *FTU, int lmax, int RP,
-                                                                            int lchunk, double2 *aE, double2 *aB) {
+                                                                            int nk, int add, int lchunk, double2 *aE,
+                                                                            double2 *aB) {
   if (gate && gate->done) return;
-  extern __shared__ float4 pol_dsm[];   // [4][RP] combinations, then [RP / 32] first l of each tile
+  extern __shared__ float4 pol_dsm[];   // [4][nk] combinations, then [nk / 32] first l of each tile
   const int m = blockIdx.x;
   const int lbeg = m + blockIdx.y * lchunk, lend = min(lmax, lbeg + lchunk - 1);
   if (lbeg > lmax) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const int ntile = (RP + 31) >> 5;
-  int *tmin = reinterpret_cast<int *>(pol_dsm + 4 * RP);
+  const int ntile = (nk + 31) >> 5;
+  int *tmin = reinterpret_cast<int *>(pol_dsm + 4 * nk);
   for (int t = warp; t < ntile; t += nw) {
     const int k = 32 * t + lane;
-    const int mn = __reduce_min_sync(0xffffffffu, k < RP ? ls[(size_t)m * RP + k] : 1 << 30);
+    const int mn = __reduce_min_sync(0xffffffffu, k < nk ? ls[(size_t)m * RP + k] : 1 << 30);
     if (lane == 0) tmin[t] = mn;
   }
   __syncthreads();
   int tf = 0;                           // the tiles any row of the chunk reads
   while (tf < ntile && tmin[tf] > lend + 1) ++tf;
-  for (int k = 32 * tf + threadIdx.x; k < RP; k += blockDim.x) {
-    f_parities(FTQ[(size_t)m * RP + k], pol_dsm[k], pol_dsm[RP + k]);
-    f_parities(FTU[(size_t)m * RP + k], pol_dsm[2 * RP + k], pol_dsm[3 * RP + k]);
+  for (int k = 32 * tf + threadIdx.x; k < nk; k += blockDim.x) {
+    f_parities(FTQ[(size_t)m * RP + k], pol_dsm[k], pol_dsm[nk + k]);
+    f_parities(FTU[(size_t)m * RP + k], pol_dsm[2 * nk + k], pol_dsm[3 * nk + k]);
   }
   __syncthreads();
   const size_t base = idx_lm(lmax, m, m);
@@ -267,12 +276,12 @@ __global__ void __launch_bounds__(kPolThreads, 3) spin2_analysis_df_kernel(const
     while (t0 < ntile && tmin[t0] > l + 1) ++t0;   // towards the equator the first l falls)
     auto load = [&](int t, float4 &f0, float4 &f1) {
       const int k = 32 * t + lane;
-      f0 = k < RP ? row0[k] : zero4();
-      f1 = k < RP && has1 ? row1[k] : zero4();
+      f0 = k < nk ? row0[k] : zero4();
+      f1 = k < nk && has1 ? row1[k] : zero4();
     };
     auto term = [&](int t, float4 f0, float4 f1) {
-      const int k = min(32 * t + lane, RP - 1);   // lanes past RP: zero table values
-      const float4 A = pol_dsm[k], Bq = pol_dsm[RP + k], Cu = pol_dsm[2 * RP + k], Du = pol_dsm[3 * RP + k];
+      const int k = min(32 * t + lane, nk - 1);   // lanes past nk: zero table values
+      const float4 A = pol_dsm[k], Bq = pol_dsm[nk + k], Cu = pol_dsm[2 * nk + k], Du = pol_dsm[3 * nk + k];
       // -a^E = F+ Q+ + i F- U-,  -a^B = F+ U+ - i F- Q-
       {   // l: Q+ = A, Q- = Bq, U+ = Cu, U- = Du
         const dfl fp = {f0.x, f0.y}, fm = {f0.z, f0.w}, fn = df_neg(fm);
@@ -317,8 +326,9 @@ __global__ void __launch_bounds__(kPolThreads, 3) spin2_analysis_df_kernel(const
     if ((lane & 3) == 0) {   // sum lane / 4: E re, im, B re, im of l, then of l + 1
       const int q = lane >> 2, lq = l + (q >> 2);
       if (lq <= lend) {
-        double2 *dst = ((q >> 1) & 1) ? aB : aE;
-        reinterpret_cast<double *>(dst + base + (lq - m))[q & 1] = lq >= 2 ? -df_to(v) : 0.0;
+        double &dst = reinterpret_cast<double *>((((q >> 1) & 1) ? aB : aE) + base + (lq - m))[q & 1];
+        const double a = -df_to(v);
+        dst = lq >= 2 ? (add ? dst + a : a) : 0.0;
       }
     }
   }
@@ -646,19 +656,22 @@ void Pol::analysis(cudaStream_t s, const double *map, double2 *alm, const Ctl *g
   la.alm = alm;
   la.gate = gate;
   P->launch_leg(la, s, LEG_ANALYSIS);                                 // T
-  if (df) {
-    auto kernel = RP <= 128 ? spin2_analysis_df_kernel<true> : spin2_analysis_df_kernel<false>;   // short sums in the finer steps
-    raise_smem_cap(reinterpret_cast<const void *>(kernel));
-    // 64 values of l a CTA (four row pairs a warp), 16 where lmax leaves few chunks
-    const int lchunk = lmax >= 256 ? 64 : 16;
-    const dim3 grid(lmax + 1, (lmax + lchunk) / lchunk);
-    kernel<<<grid, kPolThreads, sizeof(float4) * 4 * RP + sizeof(int) * ((RP + 31) / 32), s>>>(
-        gate, reinterpret_cast<const float4 *>(d_tab), P->d_ls, d_FTQ, d_FTU, lmax, RP, lchunk, alm + nalm,
-        alm + 2 * nalm);
-  } else {
-    raise_smem_cap(reinterpret_cast<const void *>(spin2_analysis_kernel));
-    spin2_analysis_kernel<<<lmax + 1, kPolThreads, sizeof(double4_32a) * 2 * RP, s>>>(
-        gate, d_tab, d_FTQ, d_FTU, lmax, RP, alm + nalm, alm + 2 * nalm);
+  for (int k0 = 0; k0 < RP; k0 += kSpin2Pairs) {
+    const int nk = std::min(kSpin2Pairs, RP - k0), add = k0 > 0;
+    if (df) {
+      auto kernel = RP <= 128 ? spin2_analysis_df_kernel<true> : spin2_analysis_df_kernel<false>;   // short sums in the finer steps
+      raise_smem_cap(reinterpret_cast<const void *>(kernel));
+      // 64 values of l a CTA (four row pairs a warp), 16 where lmax leaves few chunks
+      const int lchunk = lmax >= 256 ? 64 : 16;
+      const dim3 grid(lmax + 1, (lmax + lchunk) / lchunk);
+      kernel<<<grid, kPolThreads, sizeof(float4) * 4 * nk + sizeof(int) * ((nk + 31) / 32), s>>>(
+          gate, reinterpret_cast<const float4 *>(d_tab) + k0, P->d_ls + k0, d_FTQ + k0, d_FTU + k0, lmax, RP, nk, add,
+          lchunk, alm + nalm, alm + 2 * nalm);
+    } else {
+      raise_smem_cap(reinterpret_cast<const void *>(spin2_analysis_kernel));
+      spin2_analysis_kernel<<<lmax + 1, kPolThreads, sizeof(double4_32a) * 2 * nk, s>>>(
+          gate, d_tab + k0, d_FTQ + k0, d_FTU + k0, lmax, RP, nk, add, alm + nalm, alm + 2 * nalm);
+    }
   }
 }
 
