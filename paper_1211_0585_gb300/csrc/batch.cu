@@ -359,16 +359,12 @@ wf_status Engine::refresh_state() {
 
 wf_status Engine::step() {
   if (!graph) {
-    cudaGraph_t g;
-    ENG_CUDA(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
-    for (int i = 0; i < graph_iters; ++i)
+    const wf_status st = capture_graph(stream, graph_iters, &graph, "graph of the batched engine", [&] {
       launch_batch_iteration(args(), tc_args(), maps, geo->pclass.data(), (int)geo->pclass.size(),
                              ring_groups.empty() ? nullptr : ring_groups.data(), bstate, stream, bands.data(),
                              (int)bands.size());
-    ENG_CUDA(cudaStreamEndCapture(stream, &g));
-    cudaError_t e = cudaGraphInstantiate(&graph, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return cuda_status(e, "cudaGraphInstantiate (batched engine)");
+    });
+    if (st) return st;
   }
   ENG_CUDA(cudaGraphLaunch(graph, stream));
   ENG_CUDA(cudaMemcpyAsync(h_ctl, ctl, sizeof(Ctl) * B, cudaMemcpyDeviceToHost, stream));

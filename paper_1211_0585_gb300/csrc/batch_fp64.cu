@@ -116,17 +116,12 @@ wf_status solve_fp64_batch(Plan *P, int nrhs, const double *d, int d_on_device, 
       ra.push_back(M[b]->ring_args());
       rd.push_back(M[b]->ringdf_args());
     }
-    cudaGraph_t g;
-    FB_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-    for (int i = 0; i < gi; ++i) {
+    st = capture_graph(s, gi, &F->graph, "graph of the batched FP64 solve", [&] {
       P->launch_rng_maps(ra.data(), rd.data(), nb, s, RING_ITER);
       launch_legendre_tab(P->leg_args(), P->legdf_args(), bm, nb, s, LEG_ITER);
       launch_control(rc.data(), nb, P->R, P->lmax, s);
-    }
-    FB_CUDA(cudaStreamEndCapture(s, &g));
-    cudaError_t e = cudaGraphInstantiate(&F->graph, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return cuda_status(e, "cudaGraphInstantiate (batched FP64)");
+    });
+    if (st) return st;
     F->graph_iters = gi;
     F->graph_hist = hist;
   }

@@ -886,13 +886,9 @@ static wf_status solve_impl(Plan *P, const double *d, int d_on_device, double *a
   WF_CUDA(cudaMemcpyAsync(P->d_ctl, P->h_ctl, sizeof(Ctl), cudaMemcpyHostToDevice, s));
   // one CUDA graph holds graph_iters iterations; the controller stops the rest early
   if (!P->graph_exec) {
-    cudaGraph_t g;
-    WF_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-    for (int i = 0; i < P->opt.graph_iters; ++i) P->enqueue_iteration(s);
-    WF_CUDA(cudaStreamEndCapture(s, &g));
-    cudaError_t e = cudaGraphInstantiate(&P->graph_exec, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return cuda_status(e, "cudaGraphInstantiate");
+    const wf_status gs = capture_graph(s, P->opt.graph_iters, &P->graph_exec, "graph of the solve",
+                                       [&] { P->enqueue_iteration(s); });
+    if (gs) return gs;
     P->graph_prec = P->opt.precision;
   }
   const int max_launch = (P->opt.max_iter + P->opt.graph_iters - 1) / P->opt.graph_iters + 1;

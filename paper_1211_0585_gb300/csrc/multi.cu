@@ -329,13 +329,9 @@ wf_status wf_multi_solve(wf_multi_t multi, const double *d, int d_on_device, dou
   MU_CUDA(cudaMemcpyAsync(M->d_ctl, M->h_ctl, sizeof(Ctl), cudaMemcpyHostToDevice, s));
   const int gi = M->opt.graph_iters;
   if (!M->graph) {
-    cudaGraph_t g;
-    MU_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-    for (int i = 0; i < gi; ++i) M->enqueue_iteration(s);
-    MU_CUDA(cudaStreamEndCapture(s, &g));
-    cudaError_t e = cudaGraphInstantiate(&M->graph, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return cuda_status(e, "cudaGraphInstantiate (several messenger fields)");
+    const wf_status gs = capture_graph(s, gi, &M->graph, "graph of the several messenger fields",
+                                       [&] { M->enqueue_iteration(s); });
+    if (gs) return gs;
   }
   const int max_launch = (M->opt.max_iter + gi - 1) / gi + 1;
   for (int it = 0; it < max_launch; ++it) {

@@ -868,13 +868,9 @@ wf_status wf_pol_solve(wf_pol_t pol, const double *d, int d_on_device, double *a
   PO_CUDA(cudaMemcpyAsync(Q->d_ctl, Q->h_ctl, sizeof(Ctl), cudaMemcpyHostToDevice, s));
   const int gi = Q->opt.graph_iters;
   if (!Q->graph) {
-    cudaGraph_t g;
-    PO_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-    for (int i = 0; i < gi; ++i) Q->enqueue_iteration(s);
-    PO_CUDA(cudaStreamEndCapture(s, &g));
-    cudaError_t e = cudaGraphInstantiate(&Q->graph, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return cuda_status(e, "cudaGraphInstantiate (polarisation)");
+    const wf_status gs = capture_graph(s, gi, &Q->graph, "graph of the polarised solve",
+                                       [&] { Q->enqueue_iteration(s); });
+    if (gs) return gs;
   }
   const int max_launch = (Q->opt.max_iter + gi - 1) / gi + 1;
   for (int it = 0; it < max_launch; ++it) {

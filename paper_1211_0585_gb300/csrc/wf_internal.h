@@ -320,4 +320,21 @@ void raise_smem_cap(const void *func);
 void set_error(const std::string &msg);
 wf_status cuda_status(cudaError_t e, const char *where);
 
+// iters times one() on s as an executable graph. A launch that is refused while a stream is being captured ends neither
+// the capture nor the graph, which would then leave that kernel out: its error is looked at here.
+template <class F>
+wf_status capture_graph(cudaStream_t s, int iters, cudaGraphExec_t *exec, const char *what, F one) {
+  cudaGetLastError();   // an error of before is not this graph's
+  cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
+  if (e != cudaSuccess) return cuda_status(e, what);
+  for (int i = 0; i < iters; ++i) one();
+  const cudaError_t launched = cudaGetLastError();
+  cudaGraph_t g = nullptr;
+  e = cudaStreamEndCapture(s, &g);
+  if (e == cudaSuccess) e = launched;
+  if (e == cudaSuccess) e = cudaGraphInstantiate(exec, g, 0);
+  if (g) cudaGraphDestroy(g);
+  return e == cudaSuccess ? WF_OK : cuda_status(e, what);
+}
+
 }  // namespace wfk
