@@ -79,8 +79,8 @@ __device__ __forceinline__ dfl df_mul2(dfl a, dfl b) {
 // "Accurate sum and dot product", SIAM J. Sci. Comput. 26, 2005). The loops over
 // l and over ring pairs are made of this step, and FP32 issue bounds them once
 // their table reads are hidden: in 13 instructions 2.8e12 products/s measured.
-// FINE, 12 instructions: every error term exact but for the two cross terms,
-// as in the sum of Ogita et al. Else 10: two_sum(S, p) splits into the parts of S
+// FINE, 13 instructions: every error term exact but for the two cross terms,
+// as in the sum of Ogita et al., and the product of the low parts. Else 10: two_sum(S, p) splits into the parts of S
 // and of p that the rounded sum lost, the part of p is formed from the exact
 // product (one fma instead of two_prod's error term and a subtraction) and the
 // cross terms are added to it. Those three round at the sum's own ulp, which
@@ -94,6 +94,7 @@ __device__ __forceinline__ void dot2_acc(float &S, float &C, dfl a, dfl b) {
   const float d = S - (s - bb);
   if (FINE) {
     float v = fmaf(a.h, b.h, -p);
+    v = fmaf(a.l, b.l, v);
     v = fmaf(a.l, b.h, v);
     v = fmaf(a.h, b.l, v);
     C += (d + (p - bb)) + v;
@@ -116,18 +117,30 @@ __device__ __forceinline__ void dot2_tidy(float &S, float &C) {
 }
 
 // mu_l = (A x) mu1 - mu2 in double-float: one step of the rescaled Legendre
-// recurrence mu_l = A_l x mu_{l-1} - mu_{l-2}, 17 FP32 instructions (the sum's
-// error from the exact product, as in dot2_acc)
+// recurrence mu_l = A_l x mu_{l-1} - mu_{l-2}. 17 FP32 instructions, the sum's
+// error from the exact product as in dot2_acc; FINE, 19: the product's error by
+// itself, which rounds at the product's ulp and not at the sum's
+template <bool FINE = false>
 __device__ __forceinline__ dfl df_step(dfl A, dfl x, dfl mu1, dfl mu2) {
-  const float ch = A.h * x.h;
+  const float ch = __fmul_rn(A.h, x.h);
   float ce = fmaf(A.h, x.h, -ch);
   ce = fmaf(A.h, x.l, fmaf(A.l, x.h, ce));
-  const float sh = __fadd_rn(__fmul_rn(ch, mu1.h), -mu2.h);
-  const float bb = sh + mu2.h;            // the part of the product in sh
-  const float d = -mu2.h - (sh - bb);
-  float v = fmaf(ch, mu1.h, -bb);
-  v = fmaf(ch, mu1.l, fmaf(ce, mu1.h, v));
-  const float e = d + (v - mu2.l);
+  const float qh = __fmul_rn(ch, mu1.h);
+  const float sh = __fadd_rn(qh, -mu2.h);
+  float e;
+  if (FINE) {
+    float qe = fmaf(ch, mu1.h, -qh);
+    qe = fmaf(ch, mu1.l, fmaf(ce, mu1.h, qe));
+    const float bb = sh - qh;
+    e = (qh - (sh - bb)) + (-mu2.h - bb);
+    e += qe - mu2.l;
+  } else {
+    const float bb = sh + mu2.h;          // the part of the product in sh
+    const float d = -mu2.h - (sh - bb);
+    float v = fmaf(ch, mu1.h, -bb);
+    v = fmaf(ch, mu1.l, fmaf(ce, mu1.h, v));
+    e = d + (v - mu2.l);
+  }
   const float rh = sh + e;
   return {rh, e - (rh - sh)};
 }

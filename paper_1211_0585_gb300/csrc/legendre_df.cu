@@ -69,14 +69,14 @@ constexpr int kDB = 8;   // l per block of the analysis
 
 // kDB recurrence steps of one ring pair from l0, accumulating mu * (E or O)
 // into the 2 kDB compensated sums; INJECT places the table start values.
-template <bool INJECT>
+template <bool INJECT, bool FINE>
 __device__ __forceinline__ void analysis_block(int l0, const float2 *sA, dfl x, dfl &p1, dfl &p2, int ls, float4 v,
                                                float4 e, float4 o, float (&S)[16], float (&C)[16]) {
 #pragma unroll
   for (int j = 0; j < kDB; ++j) {
     const int l = l0 + j;
     const float2 a2 = sA[j];
-    dfl mu = df_step(dfl{a2.x, a2.y}, x, p1, p2);
+    dfl mu = df_step<FINE>(dfl{a2.x, a2.y}, x, p1, p2);
     if (INJECT) {
       if (l == ls) mu = dfl{v.x, v.y};
       if (l == ls + 1) mu = dfl{v.z, v.w};
@@ -84,8 +84,8 @@ __device__ __forceinline__ void analysis_block(int l0, const float2 *sA, dfl x, 
     p2 = p1;
     p1 = mu;
     const float4 f = (j & 1) ? o : e;
-    dot2_acc(S[2 * j], C[2 * j], mu, dfl{f.x, f.y});
-    dot2_acc(S[2 * j + 1], C[2 * j + 1], mu, dfl{f.z, f.w});
+    dot2_acc<FINE>(S[2 * j], C[2 * j], mu, dfl{f.x, f.y});
+    dot2_acc<FINE>(S[2 * j + 1], C[2 * j + 1], mu, dfl{f.z, f.w});
   }
 }
 
@@ -190,7 +190,7 @@ __global__ void lam_table_kernel(const double *xk, const double2 *rec, const int
 // barrier each (16 l, two barriers and sums in double before) and one form of the
 // recurrence block a warp took the iteration to 78 ms. FP32 issue bounds both
 // (37 instructions a term: 25 ms a pass).
-template <int MODE, int NT>
+template <int MODE, int NT, bool FINE>
 __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) legendre_df_kernel(const LegArgs A, const LegDfArgs D) {
   extern __shared__ double2 dsm[];
   __shared__ float2 red[2][NT / 32][16];
@@ -302,10 +302,10 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) legendre_df_kernel(cons
           const float4 e4 = begun ? stE[kk] : z, o4 = begun ? stO[kk] : z, q4 = stP[kk];
           dfl p1 = dfl{q4.x, q4.y}, p2 = dfl{q4.z, q4.w};
           if (__any_sync(0xffffffffu, starts))
-            analysis_block<true>(l0, sA + (l0 - m), dfl{x2.x, x2.y}, p1, p2, ls,
+            analysis_block<true, FINE>(l0, sA + (l0 - m), dfl{x2.x, x2.y}, p1, p2, ls,
                                  starts ? D.sv[(size_t)m * RP + k0 + kk] : z, e4, o4, S, C);
           else
-            analysis_block<false>(l0, sA + (l0 - m), dfl{x2.x, x2.y}, p1, p2, ls, z, e4, o4, S, C);
+            analysis_block<false, FINE>(l0, sA + (l0 - m), dfl{x2.x, x2.y}, p1, p2, ls, z, e4, o4, S, C);
           if (begun) stP[kk] = make_float4(p1.h, p1.l, p2.h, p2.l);
         }
         warp_sums16(S, C);
@@ -401,41 +401,41 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) legendre_df_kernel(cons
       int l = ls;
       {
         const float4 c = ss[l - m];
-        if (((l - m) & 1) == 0) { dot2_acc(ERs, ERc, p2, dfl{c.x, c.y}); dot2_acc(EIs, EIc, p2, dfl{c.z, c.w}); }
-        else { dot2_acc(ORs, ORc, p2, dfl{c.x, c.y}); dot2_acc(OIs, OIc, p2, dfl{c.z, c.w}); }
+        if (((l - m) & 1) == 0) { dot2_acc<FINE>(ERs, ERc, p2, dfl{c.x, c.y}); dot2_acc<FINE>(EIs, EIc, p2, dfl{c.z, c.w}); }
+        else { dot2_acc<FINE>(ORs, ORc, p2, dfl{c.x, c.y}); dot2_acc<FINE>(OIs, OIc, p2, dfl{c.z, c.w}); }
       }
       if (l + 1 <= L) {
         const float4 c = ss[l + 1 - m];
-        if (((l + 1 - m) & 1) == 0) { dot2_acc(ERs, ERc, p1, dfl{c.x, c.y}); dot2_acc(EIs, EIc, p1, dfl{c.z, c.w}); }
-        else { dot2_acc(ORs, ORc, p1, dfl{c.x, c.y}); dot2_acc(OIs, OIc, p1, dfl{c.z, c.w}); }
+        if (((l + 1 - m) & 1) == 0) { dot2_acc<FINE>(ERs, ERc, p1, dfl{c.x, c.y}); dot2_acc<FINE>(EIs, EIc, p1, dfl{c.z, c.w}); }
+        else { dot2_acc<FINE>(ORs, ORc, p1, dfl{c.x, c.y}); dot2_acc<FINE>(OIs, OIc, p1, dfl{c.z, c.w}); }
       }
       l += 2;
       if (((l - m) & 1) == 1 && l <= L) {
         const float2 a2 = sA[l - m];
-        const dfl mu = df_step(dfl{a2.x, a2.y}, x, p1, p2);
+        const dfl mu = df_step<FINE>(dfl{a2.x, a2.y}, x, p1, p2);
         p2 = p1; p1 = mu;
         const float4 c = ss[l - m];
-        dot2_acc(ORs, ORc, mu, dfl{c.x, c.y});
-        dot2_acc(OIs, OIc, mu, dfl{c.z, c.w});
+        dot2_acc<FINE>(ORs, ORc, mu, dfl{c.x, c.y});
+        dot2_acc<FINE>(OIs, OIc, mu, dfl{c.z, c.w});
         ++l;
       }
       for (; l + 1 <= L; l += 2) {
         const float2 a0 = sA[l - m], a1 = sA[l + 1 - m];
-        const dfl me = df_step(dfl{a0.x, a0.y}, x, p1, p2);
-        const dfl mo = df_step(dfl{a1.x, a1.y}, x, me, p1);
+        const dfl me = df_step<FINE>(dfl{a0.x, a0.y}, x, p1, p2);
+        const dfl mo = df_step<FINE>(dfl{a1.x, a1.y}, x, me, p1);
         p2 = me; p1 = mo;
         const float4 ce = ss[l - m], co = ss[l + 1 - m];
-        dot2_acc(ERs, ERc, me, dfl{ce.x, ce.y});
-        dot2_acc(EIs, EIc, me, dfl{ce.z, ce.w});
-        dot2_acc(ORs, ORc, mo, dfl{co.x, co.y});
-        dot2_acc(OIs, OIc, mo, dfl{co.z, co.w});
+        dot2_acc<FINE>(ERs, ERc, me, dfl{ce.x, ce.y});
+        dot2_acc<FINE>(EIs, EIc, me, dfl{ce.z, ce.w});
+        dot2_acc<FINE>(ORs, ORc, mo, dfl{co.x, co.y});
+        dot2_acc<FINE>(OIs, OIc, mo, dfl{co.z, co.w});
       }
       if (l <= L) {
         const float2 a0 = sA[l - m];
-        const dfl me = df_step(dfl{a0.x, a0.y}, x, p1, p2);
+        const dfl me = df_step<FINE>(dfl{a0.x, a0.y}, x, p1, p2);
         const float4 ce = ss[l - m];
-        dot2_acc(ERs, ERc, me, dfl{ce.x, ce.y});
-        dot2_acc(EIs, EIc, me, dfl{ce.z, ce.w});
+        dot2_acc<FINE>(ERs, ERc, me, dfl{ce.x, ce.y});
+        dot2_acc<FINE>(EIs, EIc, me, dfl{ce.z, ce.w});
       }
     }
     A.FS[mk] = f_rings(df_norm(ERs, ERc), df_norm(EIs, EIc), df_norm(ORs, ORc), df_norm(OIs, OIc));
@@ -452,12 +452,12 @@ static size_t leg_df_smem(int lmax, int RP, int chunk) {
   return Lp * sizeof(double2) + (Lp + 1) * sizeof(float2) + q * sizeof(float4) + 16;
 }
 
-template <int MODE, int NT>
+template <int MODE, int NT, bool FINE = false>
 static void launch_df(const LegArgs &a, const LegDfArgs &d, cudaStream_t s) {
-  raise_smem_cap(reinterpret_cast<const void *>(legendre_df_kernel<MODE, NT>));
+  raise_smem_cap(reinterpret_cast<const void *>(legendre_df_kernel<MODE, NT, FINE>));
   // the synthesis alone holds no ring-pair state
   const size_t sm = leg_df_smem(a.lmax, a.RP, MODE == LEG_SYNTH ? 0 : kAnaChunk<NT>);
-  legendre_df_kernel<MODE, NT><<<a.lmax + 1, NT, sm, s>>>(a, d);
+  legendre_df_kernel<MODE, NT, FINE><<<a.lmax + 1, NT, sm, s>>>(a, d);
 }
 
 void launch_legendre_df(const LegArgs &a, const LegDfArgs &d, cudaStream_t s, int mode) {
@@ -478,17 +478,21 @@ void launch_legendre_df(const LegArgs &a, const LegDfArgs &d, cudaStream_t s, in
   }
   // four ring pairs a thread keep the larger CTAs' sums over lanes as cheap a term as the smaller ones'
   const bool wide = a.RP >= 2048;
+  const bool fine = a.RP <= 128;   // short sums in the finer steps, as over the table (legendre_tab.cu)
   switch (mode) {
     case LEG_SYNTH:
       if (wide) launch_df<LEG_SYNTH, 1024>(a, d, s);
+      else if (fine) launch_df<LEG_SYNTH, 256, true>(a, d, s);
       else launch_df<LEG_SYNTH, 256>(a, d, s);
       break;
     case LEG_ANALYSIS:
       if (wide) launch_df<LEG_ANALYSIS, 512>(a, d, s);
+      else if (fine) launch_df<LEG_ANALYSIS, 256, true>(a, d, s);
       else launch_df<LEG_ANALYSIS, 256>(a, d, s);
       break;
     default:
       if (wide) launch_df<LEG_ITER, 512>(a, d, s);
+      else if (fine) launch_df<LEG_ITER, 256, true>(a, d, s);
       else launch_df<LEG_ITER, 256>(a, d, s);
       break;
   }

@@ -45,3 +45,12 @@ def test_polarised_solve_at_high_signal_to_noise():
     5.92e-15 with quotients, times 1.2 (1.48 times with products with the determinant's reciprocal in their place)."""
     case = dict(kind="pol_solve", nside=8, lmax=16, tol=1e-4)
     assert mean_error(case, 8, lambda r: r["alm"][0], True) <= 1.2 * 5.92e-15
+
+
+@pytest.mark.parametrize("kind,base", [("analysis", 3.14e-14), ("iterate", 1.42e-14)])
+def test_recurrence_form(kind, base):
+    """16 seeds, times 1.06 (1.16 and 1.24 times with sums and steps whose errors round at the sum's ulp)."""
+    case = dict(kind=kind, nside=16, lmax=37, lsht=37)
+    if kind == "iterate":
+        case.update(lam=3.0, niter=3)
+    assert mean_error(case, 16, lambda r: r["alm"] if kind == "iterate" else r, False) <= 1.06 * base
