@@ -172,25 +172,6 @@ __device__ __forceinline__ void mma_chunk(uint32_t dmain, uint32_t dcorr, uint8_
 }  // namespace
 
 // ---------------------------------------------------------------- tables
-// The recurrence step the tables are built with, once per shape. df_step's sum
-// rounds its error term once less; here every operation stands alone, because
-// a table value next to a rounding boundary of its 22 bits would otherwise move
-// by 2^-22, and every mixed result with it.
-__device__ __forceinline__ dfl table_step(dfl A, dfl x, dfl mu1, dfl mu2) {
-  const float ch = A.h * x.h;
-  float ce = fmaf(A.h, x.h, -ch);
-  ce = fmaf(A.h, x.l, fmaf(A.l, x.h, ce));
-  const float qh = ch * mu1.h;
-  float qe = fmaf(ch, mu1.h, -qh);
-  qe = fmaf(ch, mu1.l, fmaf(ce, mu1.h, qe));
-  const float sh = qh - mu2.h;
-  const float bb = sh - qh;
-  float e = (qh - (sh - bb)) + (-mu2.h - bb);
-  e += qe - mu2.l;
-  const float rh = sh + e;
-  return {rh, e - (rh - sh)};
-}
-
 // One thread per (m, k): the double-float recurrence from the start values
 // writes lambda_lm(x_k) (rounded to 22 bits, 0 below l_start) into both table
 // layouts (only the analysis layout when lamT is nullptr: the synthesis rows are
@@ -234,7 +215,7 @@ __global__ void lam_tc_tables_kernel(const double *xk, const LegDfArgs D, int lm
       else if (l == ls + 1) mu = dfl{s4.z, s4.w};
       else {
         const float2 a2 = D.A[base + (l - m)];
-        mu = table_step(dfl{a2.x, a2.y}, x, p1, p2);
+        mu = df_step<true>(dfl{a2.x, a2.y}, x, p1, p2);
       }
       p2 = p1;
       p1 = mu;
