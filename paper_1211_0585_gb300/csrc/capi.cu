@@ -395,11 +395,14 @@ wf_status plan_rebind(Plan *P, const double *cl, const double *w, double tau, lo
   return WF_OK;
 }
 
+// the power of two in (Omega / 4, Omega / 2]
+double Plan::record_scale() const { return std::ldexp(1.0, std::ilogb(0.5 * omega)); }
+
 RingArgs Plan::ring_args() const {
   RingArgs a{};
   a.rings = d_rings; a.order = d_order; a.porder = d_porder; a.first = 0; a.scratch = d_ring_scratch; a.tw = d_tw; a.logMmax = logMmax; a.hs = d_hs; a.chirp = d_chirp; a.B = d_B;
   a.FS = d_FS; a.FT = d_FT; a.RP = RP; a.d = d_d; a.w = d_w; a.ring_part = d_ring_part; a.ctl = d_ctl;
-  a.lsht = lmax; a.omega = omega; a.tau = tau; a.gain = d_gain; a.gainlam = d_gainlam;
+  a.lsht = lmax; a.omega = omega; a.tau = tau; a.fscale = (float)record_scale(); a.gain = d_gain; a.gainlam = d_gainlam;
   return a;
 }
 
@@ -407,6 +410,7 @@ LegArgs Plan::leg_args() const {
   LegArgs a{};
   a.x = d_x; a.rec = d_rec; a.ls = d_ls; a.sv = d_sv; a.cl = d_cl; a.FT = d_FT; a.FS = d_FS; a.alm = d_s;
   a.m_part = d_m_part; a.part = d_part; a.coef = d_coef; a.ctl = d_ctl; a.lsht = lmax; a.lmax = lmax; a.RP = RP; a.omega = omega; a.tau = tau;
+  a.fomega = 0.5 * omega / record_scale();
   return a;
 }
 

@@ -45,14 +45,22 @@ __device__ __forceinline__ dfl df_add(dfl a, dfl b) {
 }
 
 // a + b with the low parts' sum error-free too (accurate double-word addition, Joldes, Muller and Popescu, ACM TOMS 44,
-// 2017): where a few sums stand between long chains of products, as the Fourier records' do
+// 2017): where a few sums stand between long chains of products, as the Fourier records' do. FINE: that of the errors
+// too, one rounding in all (24 instructions instead of 20)
+template <bool FINE>
 __device__ __forceinline__ dfl df_add2(dfl a, dfl b) {
   const float s = a.h + b.h, bb = s - a.h;
   const float e = (a.h - (s - bb)) + (b.h - bb);
   const float t = a.l + b.l, bt = t - a.l;
   const float f = (a.l - (t - bt)) + (b.l - bt);
   const float c = e + t;
-  const float v = s + c, w = f + (c - (v - s));
+  const float v = s + c;
+  float w = f;
+  if (FINE) {
+    const float bc = c - e;
+    w += (e - (c - bc)) + (t - bc);
+  }
+  w += c - (v - s);
   const float r = v + w;
   return {r, w - (r - v)};
 }
@@ -61,15 +69,6 @@ __device__ __forceinline__ dfl df_add2(dfl a, dfl b) {
 __device__ __forceinline__ dfl df_mul(dfl a, dfl b) {
   const float p = a.h * b.h;
   float e = fmaf(a.h, b.h, -p);
-  e = fmaf(a.h, b.l, fmaf(a.l, b.h, e));
-  const float r = p + e;
-  return {r, e - (r - p)};
-}
-
-// a * b with the product of the low parts
-__device__ __forceinline__ dfl df_mul2(dfl a, dfl b) {
-  const float p = a.h * b.h;
-  float e = fmaf(a.l, b.l, fmaf(a.h, b.h, -p));
   e = fmaf(a.h, b.l, fmaf(a.l, b.h, e));
   const float r = p + e;
   return {r, e - (r - p)};
@@ -84,8 +83,8 @@ __device__ __forceinline__ dfl df_mul2(dfl a, dfl b) {
 // and of p that the rounded sum lost, the part of p is formed from the exact
 // product (one fma instead of two_prod's error term and a subtraction) and the
 // cross terms are added to it. Those three round at the sum's own ulp, which
-// short sums feel (7 % more error over 16 terms, 1 % over 128); long ones are
-// bound by the rounding of C, which dot2_tidy keeps small.
+// short sums feel (7 % more error over 16 terms, 1 % over 128: fine_steps);
+// long ones are bound by the rounding of C, which dot2_tidy keeps small.
 template <bool FINE = false>
 __device__ __forceinline__ void dot2_acc(float &S, float &C, dfl a, dfl b) {
   const float p = __fmul_rn(a.h, b.h);
@@ -147,14 +146,16 @@ __device__ __forceinline__ dfl df_step(dfl A, dfl x, dfl mu1, dfl mu2) {
 
 // A Fourier record (north re, im, south re, im; df_pack'ed) as the sums of its two rings for even l - m, E = N + S,
 // and for odd, O = N - S, each (re hi, re lo, im hi, im lo); and the record of E and O.
+template <bool FINE>
 __device__ __forceinline__ void f_parities(const double4_32a &t, float4 &E, float4 &O) {
   const dfl nr = df_unpack(t.x), ni = df_unpack(t.y), sr = df_unpack(t.z), si = df_unpack(t.w);
-  E = df_pair(df_add2(nr, sr), df_add2(ni, si));
-  O = df_pair(df_add2(nr, df_neg(sr)), df_add2(ni, df_neg(si)));
+  E = df_pair(df_add2<FINE>(nr, sr), df_add2<FINE>(ni, si));
+  O = df_pair(df_add2<FINE>(nr, df_neg(sr)), df_add2<FINE>(ni, df_neg(si)));
 }
+template <bool FINE>
 __device__ __forceinline__ double4_32a f_rings(dfl er, dfl ei, dfl orr, dfl oi) {
-  return make_double4_32a(df_pack(df_add2(er, orr)), df_pack(df_add2(ei, oi)), df_pack(df_add2(er, df_neg(orr))),
-                          df_pack(df_add2(ei, df_neg(oi))));
+  return make_double4_32a(df_pack(df_add2<FINE>(er, orr)), df_pack(df_add2<FINE>(ei, oi)), df_pack(df_add2<FINE>(er, df_neg(orr))),
+                          df_pack(df_add2<FINE>(ei, df_neg(oi))));
 }
 
 }  // namespace wfk

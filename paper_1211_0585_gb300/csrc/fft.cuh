@@ -108,7 +108,10 @@ struct OpsF32 {  // float complex; twiddles from a float table
   }
 };
 
-struct OpsDF {  // double-float complex: float4 (re hi, re lo, im hi, im lo)
+// double-float complex: float4 (re hi, re lo, im hi, im lo). FINE, on short rings: products brought back to normal form
+// before they are summed, whose errors round at a lower ulp
+template <bool FINE>
+struct OpsDF {
   using T = float4;
   using W = float4;
   static constexpr int kSw = 3;
@@ -122,10 +125,10 @@ struct OpsDF {  // double-float complex: float4 (re hi, re lo, im hi, im lo)
     return make_float2(r, e - (r - s));
   }
   static __device__ __forceinline__ float2 dmul(float ah, float al, float bh, float bl) {
-    const float p = ah * bh;
-    float e = fmaf(ah, bh, -p);
+    const float p = __fmul_rn(ah, bh);
+    float e = fmaf(al, bl, fmaf(ah, bh, -p));
     e = fmaf(ah, bl, fmaf(al, bh, e));
-    const float r = p + e;
+    const float r = __fadd_rn(p, e);
     return make_float2(r, e - (r - p));
   }
   static __device__ __forceinline__ T add(T a, T b) {
@@ -138,9 +141,14 @@ struct OpsDF {  // double-float complex: float4 (re hi, re lo, im hi, im lo)
   }
   // p q - r s (real double-floats): two_prod of both, two_sum of the high
   // products, the error and cross terms added up and renormalised once; 19 FP32
-  // instructions against 25 of two products and a sum
+  // instructions against 27 of two products with those of the low parts and a
+  // sum, FINE
   static __device__ __forceinline__ float2 pqrs(float ph, float pl, float qh, float ql, float rh, float rl, float sh,
                                                 float sl) {
+    if (FINE) {
+      const float2 x = dmul(ph, pl, qh, ql), y = dmul(rh, rl, sh, sl);
+      return dadd(x.x, x.y, -y.x, -y.y);
+    }
     const float a = __fmul_rn(ph, qh), b = __fmul_rn(rh, sh);
     float u = fmaf(ph, qh, -a), v = fmaf(rh, sh, -b);
     const float s = __fadd_rn(a, -b);

@@ -44,9 +44,11 @@ __device__ __forceinline__ FoldPair fold_record(const double4_32a *FS, size_t at
   return {make_float4(sg * nr.h, sg * nr.l, ci * ni.h, ci * ni.l),
           make_float4(sg * sr.h, sg * sr.l, ci * si.h, ci * si.l)};
 }
+template <bool FINE>
 __device__ __forceinline__ float4 fold_add(float4 a, float4 b) {
-  return df_pair(df_add2(dfl{a.x, a.y}, dfl{b.x, b.y}), df_add2(dfl{a.z, a.w}, dfl{b.z, b.w}));
+  return df_pair(df_add2<FINE>(dfl{a.x, a.y}, dfl{b.x, b.y}), df_add2<FINE>(dfl{a.z, a.w}, dfl{b.z, b.w}));
 }
+template <bool FINE>
 __device__ __forceinline__ FoldPair fold_alias_sum2(const double4_32a *FS, int RP, int k, int shifted, int n, int q,
                                                     int L, int j0, int dj) {
   const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -54,7 +56,7 @@ __device__ __forceinline__ FoldPair fold_alias_sum2(const double4_32a *FS, int R
   bool first = true;
   auto take = [&](FoldPair r) {
     if (first) a = r;
-    else { a.n = fold_add(a.n, r.n); a.s = fold_add(a.s, r.s); }
+    else { a.n = fold_add<FINE>(a.n, r.n); a.s = fold_add<FINE>(a.s, r.s); }
     first = false;
   };
   for (int j = j0, m = q + n * j0; m <= L; j += dj, m += n * dj)
@@ -69,27 +71,27 @@ __device__ __forceinline__ FoldPair fold_alias_sum2(const double4_32a *FS, int R
 // of at most L / n + 1 aliases is split over as many threads as it has terms
 // and the block has room for (over blockDim.x / n threads whatever the series'
 // length, the sum over them walked up to 64 empty parts on the smallest rings).
-template <class Store>
+template <bool FINE, class Store>
 __device__ __forceinline__ void fold_ring2(const double4_32a *FS, int RP, int k, int shifted, int n, int L,
                                            FoldPair *part, Store store) {
   const int nt = blockDim.x;
   const int nj = min(nt / n, L / n + 1);
   if (nj <= 1) {
     for (int q = threadIdx.x; q < n; q += nt) {
-      const FoldPair g = fold_alias_sum2(FS, RP, k, shifted, n, q, L, 0, 1);
+      const FoldPair g = fold_alias_sum2<FINE>(FS, RP, k, shifted, n, q, L, 0, 1);
       store(q, g.n, g.s);
     }
     return;
   }
   const int t = threadIdx.x;
-  if (t < n * nj) part[t] = fold_alias_sum2(FS, RP, k, shifted, n, t % n, L, t / n, nj);
+  if (t < n * nj) part[t] = fold_alias_sum2<FINE>(FS, RP, k, shifted, n, t % n, L, t / n, nj);
   __syncthreads();
   if (t < n) {
     FoldPair g = part[t];
     for (int jg = 1; jg < nj; ++jg) {
       const FoldPair p = part[jg * n + t];
-      g.n = fold_add(g.n, p.n);
-      g.s = fold_add(g.s, p.s);
+      g.n = fold_add<FINE>(g.n, p.n);
+      g.s = fold_add<FINE>(g.s, p.s);
     }
     store(t, g.n, g.s);
   }

@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) legendre_df_kernel(cons
           t = A.FT[(size_t)m * RP + k0 + kk];
           xk = df_from(A.x[k0 + kk]);
         }
-        f_parities(t, stE[kk], stO[kk]);
+        f_parities<FINE>(t, stE[kk], stO[kk]);
         stP[kk] = make_float4(0.f, 0.f, 0.f, 0.f);
         stX[kk] = make_float2(xk.h, xk.l);
       }
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) legendre_df_kernel(cons
     }
     // undo the rescaling: lambda = g mu
     for (int l = m + threadIdx.x; l <= L; l += blockDim.x) {
-      const double gl = D.g[base + (l - m)];
+      const double gl = A.fomega * D.g[base + (l - m)];
       tl[l - m].x *= gl;
       tl[l - m].y *= gl;
     }
@@ -438,7 +438,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) legendre_df_kernel(cons
         dot2_acc<FINE>(EIs, EIc, me, dfl{ce.z, ce.w});
       }
     }
-    A.FS[mk] = f_rings(df_norm(ERs, ERc), df_norm(EIs, EIc), df_norm(ORs, ORc), df_norm(OIs, OIc));
+    A.FS[mk] = f_rings<FINE>(df_norm(ERs, ERc), df_norm(EIs, EIc), df_norm(ORs, ORc), df_norm(OIs, OIc));
   }
 }
 
@@ -478,7 +478,7 @@ void launch_legendre_df(const LegArgs &a, const LegDfArgs &d, cudaStream_t s, in
   }
   // four ring pairs a thread keep the larger CTAs' sums over lanes as cheap a term as the smaller ones'
   const bool wide = a.RP >= 2048;
-  const bool fine = a.RP <= 128;   // short sums in the finer steps, as over the table (legendre_tab.cu)
+  const bool fine = fine_steps(a.RP);
   switch (mode) {
     case LEG_SYNTH:
       if (wide) launch_df<LEG_SYNTH, 1024>(a, d, s);

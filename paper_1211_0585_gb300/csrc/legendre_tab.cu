@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kThreads, NB == 1 ? 3 : 2) tab_analysis_kernel
 #pragma unroll
       for (int b = 0; b < NB; ++b) {
         float4 e = make_float4(0.f, 0.f, 0.f, 0.f), o = e;
-        if (S.Lb[b] >= m) f_parities(Bm.FT[b][(size_t)m * RP + k0 + kk], e, o);
+        if (S.Lb[b] >= m) f_parities<FINE>(Bm.FT[b][(size_t)m * RP + k0 + kk], e, o);
         fsm[(size_t)(2 * b) * nkc + kk] = e;
         fsm[(size_t)(2 * b + 1) * nkc + kk] = o;
       }
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(kThreads, NB == 1 ? 3 : 2) tab_analysis_kernel
   __syncthreads();
 
   // the chunk's l: Eq. 4, or the t_l themselves
-  const double wgt = (m == 0) ? 1.0 : 2.0;
+  const double wgt = (m == 0) ? 1.0 : 2.0, h = A.fomega;
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
     if (!S.on[b]) continue;
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kThreads, NB == 1 ? 3 : 2) tab_analysis_kernel
       if (l > lmax) break;
       const double2 t = tl[b][i];
       if (!ITER) {
-        alm[l - m] = l <= S.Lb[b] ? t : make_double2(0.0, 0.0);
+        alm[l - m] = l <= S.Lb[b] ? make_double2(h * t.x, h * t.y) : make_double2(0.0, 0.0);
         continue;
       }
       const double2 so = alm[l - m];
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(kThreads, NB == 1 ? 3 : 2) tab_analysis_kernel
       double2 sn = make_double2(0.0, 0.0);
       if (l <= S.Lb[b] && c > 0.0) {
         const double f = c / (c + lto);
-        sn = make_double2(f * (so.x + t.x), f * (so.y + t.y));
+        sn = make_double2(f * fma(h, t.x, so.x), f * fma(h, t.y, so.y));
       }
       if (c > 0.0) c2 += wgt * (so.x * so.x + so.y * so.y) / c;
       const double dx = sn.x - so.x, dy = sn.y - so.y;
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(kThreads, 3) tab_synthesis_kernel(const LegArg
 #pragma unroll
     for (int b = 0; b < NB; ++b)
       if (S.on[b])
-        Bm.FS[b][(size_t)m * RP + k] = f_rings(df_norm(acc[b][0], acc[b][1]), df_norm(acc[b][2], acc[b][3]),
+        Bm.FS[b][(size_t)m * RP + k] = f_rings<FINE>(df_norm(acc[b][0], acc[b][1]), df_norm(acc[b][2], acc[b][3]),
                                                df_norm(acc[b][4], acc[b][5]), df_norm(acc[b][6], acc[b][7]));
   }
 }
@@ -409,12 +409,7 @@ size_t leg_tab_smem(int lmax, int RP) { return std::max(ana_smem(1, RP), syn_sme
 
 void launch_legendre_tab(const LegArgs &a, const LegDfArgs &d, const LegBatchMaps &bm, int nb, cudaStream_t s,
                          int mode) {
-  // Sums of few terms in the finer steps (dot2_acc). Up to Nside 64 latency bounds these kernels and the two more
-  // instructions cost little (an Nside 16 solve 1 to 2 %, the FFT's longer product included; error 4.9 instead
-  // of 5.5e-15); with the line at
-  // Nside 128 a T + P solve there, bound by FP32 issue in the same sums (pol.cu), takes 68 instead of 62 ms, and
-  // dot2_tidy does as much for its error (7.3e-15 against 9.9e-15)
-  const bool fine = a.RP <= 128;
+  const bool fine = fine_steps(a.RP);
   if (nb == 1) fine ? launch_tab<1, true>(a, d, bm, s, mode) : launch_tab<1, false>(a, d, bm, s, mode);
   else fine ? launch_tab<2, true>(a, d, bm, s, mode) : launch_tab<2, false>(a, d, bm, s, mode);
 }

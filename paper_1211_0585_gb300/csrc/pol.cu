@@ -194,9 +194,15 @@ __device__ __forceinline__ float4 cdf(double re, double im) {   // complex doubl
 }
 __device__ __forceinline__ float4 zero4() { return make_float4(0.f, 0.f, 0.f, 0.f); }
 
-// (S, C) += (S, C) of the lane `off` away (xor), error-free in S
-__device__ __forceinline__ void xor_sum_df(float &S, float &C, int off) {
-  const float rS = __shfl_xor_sync(0xffffffffu, S, off), rC = __shfl_xor_sync(0xffffffffu, C, off);
+// (S, C) += (rS, rC), another lane's: error-free in S; FINE, both renormalised and one rounding
+template <bool FINE>
+__device__ __forceinline__ void lane_add(float &S, float &C, float rS, float rC) {
+  if (FINE) {
+    const dfl v = df_add2<true>(df_norm(S, C), df_norm(rS, rC));
+    S = v.h;
+    C = v.l;
+    return;
+  }
   const float s = S + rS;
   const float bb = s - S;
   C = C + rC + ((S - (s - bb)) + (rS - bb));
@@ -206,6 +212,7 @@ __device__ __forceinline__ void xor_sum_df(float &S, float &C, int off) {
 // Eight compensated sums over the warp: lane q ends with sum q >> 2 of its 8 (lanes 4 q .. 4 q + 3 hold sum q).
 // Halves are exchanged on the way down (4 + 2 + 1 additions, then 2), all in double-float: in FP64, 40 additions
 // on a pipe of 1/63 the rate took longer than a short row's products.
+template <bool FINE>
 __device__ __forceinline__ dfl warp_sum8_df(float (&S)[8], float (&C)[8]) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
@@ -216,14 +223,14 @@ __device__ __forceinline__ dfl warp_sum8_df(float (&S)[8], float (&C)[8]) {
       const float oS = up ? S[j] : S[j + n], oC = up ? C[j] : C[j + n];   // sent
       const float kS = up ? S[j + n] : S[j], kC = up ? C[j + n] : C[j];   // kept
       const float rS = __shfl_xor_sync(0xffffffffu, oS, off), rC = __shfl_xor_sync(0xffffffffu, oC, off);
-      const float s = kS + rS;
-      const float bb = s - kS;
-      S[j] = s;
-      C[j] = kC + rC + ((kS - (s - bb)) + (rS - bb));
+      S[j] = kS;
+      C[j] = kC;
+      lane_add<FINE>(S[j], C[j], rS, rC);
     }
   }
-  xor_sum_df(S[0], C[0], 2);
-  xor_sum_df(S[0], C[0], 1);
+#pragma unroll
+  for (int off = 2; off >= 1; off >>= 1)
+    lane_add<FINE>(S[0], C[0], __shfl_xor_sync(0xffffffffu, S[0], off), __shfl_xor_sync(0xffffffffu, C[0], off));
   return df_norm(S[0], C[0]);
 }
 
@@ -242,8 +249,8 @@ template <bool FINE>
 __global__ void __launch_bounds__(kPolThreads, 3) spin2_analysis_df_kernel(const Ctl *gate, const float4 *tab,
                                                                             const int *ls, const double4_32a *FTQ,
                                                                             const double4_32a *FTU, int lmax, int RP,
-                                                                            int nk, int add, int lchunk, double2 *aE,
-                                                                            double2 *aB) {
+                                                                            int nk, int add, int lchunk, double h,
+                                                                            double2 *aE, double2 *aB) {
   if (gate && gate->done) return;
   extern __shared__ float4 pol_dsm[];   // [4][nk] combinations, then [nk / 32] first l of each tile
   const int m = blockIdx.x;
@@ -261,8 +268,8 @@ __global__ void __launch_bounds__(kPolThreads, 3) spin2_analysis_df_kernel(const
   int tf = 0;                           // the tiles any row of the chunk reads
   while (tf < ntile && tmin[tf] > lend + 1) ++tf;
   for (int k = 32 * tf + threadIdx.x; k < nk; k += blockDim.x) {
-    f_parities(FTQ[(size_t)m * RP + k], pol_dsm[k], pol_dsm[nk + k]);
-    f_parities(FTU[(size_t)m * RP + k], pol_dsm[2 * nk + k], pol_dsm[3 * nk + k]);
+    f_parities<FINE>(FTQ[(size_t)m * RP + k], pol_dsm[k], pol_dsm[nk + k]);
+    f_parities<FINE>(FTU[(size_t)m * RP + k], pol_dsm[2 * nk + k], pol_dsm[3 * nk + k]);
   }
   __syncthreads();
   const size_t base = idx_lm(lmax, m, m);
@@ -322,12 +329,12 @@ __global__ void __launch_bounds__(kPolThreads, 3) spin2_analysis_df_kernel(const
         for (int j = 0; j < 8; ++j) dot2_tidy(S[j], C[j]);
       }
     }
-    const dfl v = warp_sum8_df(S, C);
+    const dfl v = warp_sum8_df<FINE>(S, C);
     if ((lane & 3) == 0) {   // sum lane / 4: E re, im, B re, im of l, then of l + 1
       const int q = lane >> 2, lq = l + (q >> 2);
       if (lq <= lend) {
         double &dst = reinterpret_cast<double *>((((q >> 1) & 1) ? aB : aE) + base + (lq - m))[q & 1];
-        const double a = -df_to(v);
+        const double a = -h * df_to(v);   // h: LegArgs::fomega
         dst = lq >= 2 ? (add ? dst + a : a) : 0.0;
       }
     }
@@ -425,9 +432,9 @@ __global__ void __launch_bounds__(kPolThreads, 3) spin2_synthesis_df_kernel(cons
     o[j] = df_norm(S1[j], C1[j]);
   }
   // sums over both parities (p) and their difference (d)
-  auto p = [&](int j) { return df_add2(e[j], o[j]); };
-  auto d = [&](int j) { return df_add2(e[j], df_neg(o[j])); };
-  auto put = [](dfl x, dfl y) { return df_pack(df_neg(df_add2(x, y))); };
+  auto p = [&](int j) { return df_add2<FINE>(e[j], o[j]); };
+  auto d = [&](int j) { return df_add2<FINE>(e[j], df_neg(o[j])); };
+  auto put = [](dfl x, dfl y) { return df_pack(df_neg(df_add2<FINE>(x, y))); };
   // north: Q = -(F+ E + i F- B), U = -(F+ B - i F- E); south: F+ -> p F+, F- -> -p F-
   FSQ[(size_t)m * RP + k] = make_double4_32a(put(p(0), df_neg(p(1))), put(p(2), p(3)), put(d(0), d(1)),
                                              put(d(2), df_neg(d(3))));
@@ -616,7 +623,7 @@ void Pol::synth(cudaStream_t s, const double2 *alm, double *map, const Ctl *gate
   la.gate = gate;
   P->launch_leg(la, s, LEG_SYNTH);                                    // T -> the plan's FS
   if (df) {
-    auto kernel = RP <= 128 ? spin2_synthesis_df_kernel<true> : spin2_synthesis_df_kernel<false>;   // short sums in the finer steps
+    auto kernel = fine_steps(RP) ? spin2_synthesis_df_kernel<true> : spin2_synthesis_df_kernel<false>;
     raise_smem_cap(reinterpret_cast<const void *>(kernel));
     // half of the ring pairs a CTA up to 256 of them: enough CTAs where few values of m do not fill the chip,
     // and the coefficients (whose conversion is FP64 work) read by few
@@ -664,14 +671,14 @@ void Pol::analysis(cudaStream_t s, const double *map, double2 *alm, const Ctl *g
   for (int k0 = 0; k0 < RP; k0 += kSpin2Pairs) {
     const int nk = std::min(kSpin2Pairs, RP - k0), add = k0 > 0;
     if (df) {
-      auto kernel = RP <= 128 ? spin2_analysis_df_kernel<true> : spin2_analysis_df_kernel<false>;   // short sums in the finer steps
+      auto kernel = fine_steps(RP) ? spin2_analysis_df_kernel<true> : spin2_analysis_df_kernel<false>;
       raise_smem_cap(reinterpret_cast<const void *>(kernel));
       // 64 values of l a CTA (four row pairs a warp), 16 where lmax leaves few chunks
       const int lchunk = lmax >= 256 ? 64 : 16;
       const dim3 grid(lmax + 1, (lmax + lchunk) / lchunk);
       kernel<<<grid, kPolThreads, sizeof(float4) * 4 * nk + sizeof(int) * ((nk + 31) / 32), s>>>(
           gate, reinterpret_cast<const float4 *>(d_tab) + k0, P->d_ls + k0, d_FTQ + k0, d_FTU + k0, lmax, RP, nk, add,
-          lchunk, alm + nalm, alm + 2 * nalm);
+          lchunk, la.fomega, alm + nalm, alm + 2 * nalm);
     } else {
       raise_smem_cap(reinterpret_cast<const void *>(spin2_analysis_kernel));
       spin2_analysis_kernel<<<lmax + 1, kPolThreads, sizeof(double4_32a) * 2 * nk, s>>>(

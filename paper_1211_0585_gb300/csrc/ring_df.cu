@@ -25,7 +25,6 @@ namespace {
 // complex double-float held as float4 (re.h, re.l, im.h, im.l)
 __device__ __forceinline__ dfl RE(float4 v) { return {v.x, v.y}; }
 __device__ __forceinline__ dfl IM(float4 v) { return {v.z, v.w}; }
-__device__ __forceinline__ float4 cmul(float4 a, float4 b) { return OpsDF::mul(a, b); }
 __device__ __forceinline__ float4 cconj(float4 a) { return make_float4(a.x, a.y, -a.z, -a.w); }
 __device__ __forceinline__ float4 cneg(float4 a) { return make_float4(-a.x, -a.y, -a.z, -a.w); }
 
@@ -62,9 +61,10 @@ __device__ __forceinline__ void warp_sum_df(float &S, float &C) {
 // in double-float throughout 203 and 52 us, with the twiddles by stage
 // (fft.cuh) 184 us at Nside 512.
 constexpr int kRingDfThreads = 256;
-template <int MODE>
+template <int MODE, bool FINE>
 __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingArgs A, const RingDfArgs T,
                                                                      const __grid_constant__ RingMaps Maps) {
+  using O = OpsDF<FINE>;
   extern __shared__ float4 rsm[];
   const RingMap &Q = Maps.m[blockIdx.y];
   const int2 pr = A.porder[A.first + blockIdx.x];  // (north ring, south ring or -1)
@@ -110,23 +110,23 @@ __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingAr
 
   if (MODE == RING_SYNTH || MODE == RING_ITER) {
     // Z = G_N + i G_S
-    fold_ring2(Q.FS, A.RP, k, rg.shifted, n, L, fold_part, [&](int q, float4 gN, float4 gS) {
-      float4 acc = df_pair(df_add2(RE(gN), df_neg(IM(gS))), df_add2(IM(gN), RE(gS)));
-      if (rg.shifted) acc = cmul(acc, hs[q]);
-      buf[px<OpsDF>(q)] = rg.blue ? cmul(cconj(acc), ch[q]) : acc;
+    fold_ring2<FINE>(Q.FS, A.RP, k, rg.shifted, n, L, fold_part, [&](int q, float4 gN, float4 gS) {
+      float4 acc = df_pair(df_add2<FINE>(RE(gN), df_neg(IM(gS))), df_add2<FINE>(IM(gN), RE(gS)));
+      if (rg.shifted) acc = O::mul(acc, hs[q]);
+      buf[px<O>(q)] = rg.blue ? O::mul(cconj(acc), ch[q]) : acc;
     });
     if (rg.blue) {
-      for (int q = n + threadIdx.x; q < M; q += blockDim.x) buf[px<OpsDF>(q)] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int q = n + threadIdx.x; q < M; q += blockDim.x) buf[px<O>(q)] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncthreads();
-    if (rg.blue) bluestein4<OpsDF, 1>(buf, Mp, M, rg.logM, Bf, T.tw, A.logMmax);
-    else fft_dif4<OpsDF, 1>(buf, Mp, M, rg.logM, +1, T.tw, A.logMmax);
+    if (rg.blue) bluestein4<O, 1>(buf, Mp, M, rg.logM, Bf, T.tw, A.logMmax);
+    else fft_dif4<O, 1>(buf, Mp, M, rg.logM, +1, T.tw, A.logMmax);
   }
   // pixel p of both rings: z = f_N + i f_S at buf[loc(p)] (Bluestein: conj of ch[p] buf[p])
-  auto loc = [&](int p) { return rg.blue ? px<OpsDF>(p) : px<OpsDF>(digitrev(p, rg.logM)); };
+  auto loc = [&](int p) { return rg.blue ? px<O>(p) : px<O>(digitrev(p, rg.logM)); };
   auto pixel = [&](int p) {
     const float4 v = buf[loc(p)];
-    return rg.blue ? cconj(cmul(ch[p], v)) : v;
+    return rg.blue ? cconj(O::mul(ch[p], v)) : v;
   };
   if (MODE == RING_SYNTH) {
     for (int p = threadIdx.x; p < n; p += blockDim.x) {
@@ -166,10 +166,10 @@ __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingAr
       const dfl uN = update(rg.off + p, RE(z), 0);
       const dfl uS = two ? update(offS + p, IM(z), 1) : dfl{0.f, 0.f};
       const float4 u = df_pair(uN, uS);
-      buf[loc(p)] = rg.blue ? cmul(u, ch[p]) : u;
+      buf[loc(p)] = rg.blue ? O::mul(u, ch[p]) : u;
     }
     if (rg.blue) {
-      for (int q = n + threadIdx.x; q < M; q += blockDim.x) buf[px<OpsDF>(q)] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int q = n + threadIdx.x; q < M; q += blockDim.x) buf[px<O>(q)] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     {
       const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -196,32 +196,33 @@ __global__ void __launch_bounds__(kRingDfThreads, 3) ring_df_kernel(const RingAr
     for (int p = threadIdx.x; p < M; p += blockDim.x) {
       if (p < n) {
         const float4 u = df_pair(df_from(Q.map_in[rg.off + p]), df_from(two ? Q.map_in[offS + p] : 0.0));
-        buf[loc(p)] = rg.blue ? cmul(u, ch[p]) : u;
+        buf[loc(p)] = rg.blue ? O::mul(u, ch[p]) : u;
       } else if (rg.blue) {
-        buf[px<OpsDF>(p)] = make_float4(0.f, 0.f, 0.f, 0.f);
+        buf[px<O>(p)] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
     }
     __syncthreads();
   }
 
-  if (rg.blue) bluestein4<OpsDF, 1>(buf, Mp, M, rg.logM, Bf, T.tw, A.logMmax);
-  else fft_dit4<OpsDF, 1>(buf, Mp, M, rg.logM, -1, T.tw, A.logMmax);
-  const dfl om = df_from(0.5 * A.omega);
+  if (rg.blue) bluestein4<O, 1>(buf, Mp, M, rg.logM, Bf, T.tw, A.logMmax);
+  else fft_dit4<O, 1>(buf, Mp, M, rg.logM, -1, T.tw, A.logMmax);
   for (int m = threadIdx.x; m <= L; m += blockDim.x) {
     const int q = m % n, j = m / n, qn = q ? n - q : 0;
-    const float4 Zq = rg.blue ? cmul(ch[q], buf[px<OpsDF>(q)]) : buf[px<OpsDF>(q)];
-    const float4 Zn = rg.blue ? cmul(ch[qn], buf[px<OpsDF>(qn)]) : buf[px<OpsDF>(qn)];
-    // U_N = (Z_q + conj Z_{n-q}) / 2, U_S = (Z_q - conj Z_{n-q}) / (2 i); the halves are in omega
-    float4 UN = df_pair(df_add(RE(Zq), RE(Zn)), df_add(IM(Zq), df_neg(IM(Zn))));
-    float4 US = df_pair(df_add(IM(Zq), IM(Zn)), df_add(RE(Zn), df_neg(RE(Zq))));
+    const float4 Zq = rg.blue ? O::mul(ch[q], buf[px<O>(q)]) : buf[px<O>(q)];
+    const float4 Zn = rg.blue ? O::mul(ch[qn], buf[px<O>(qn)]) : buf[px<O>(qn)];
+    // U_N = (Z_q + conj Z_{n-q}) / 2, U_S = (Z_q - conj Z_{n-q}) / (2 i); the records hold 2 U times a power of two
+    // next to Omega / 2, and the analysis' sums are multiplied by the rest in double: a rounding less than here
+    auto add = [](dfl x, dfl y) { return FINE ? df_add2<true>(x, y) : df_add(x, y); };
+    float4 UN = df_pair(add(RE(Zq), RE(Zn)), add(IM(Zq), df_neg(IM(Zn))));
+    float4 US = df_pair(add(IM(Zq), IM(Zn)), add(RE(Zn), df_neg(RE(Zq))));
     if (rg.shifted) {
-      UN = cmul(UN, cconj(hs[q]));
-      US = cmul(US, cconj(hs[q]));
+      UN = O::mul(UN, cconj(hs[q]));
+      US = O::mul(US, cconj(hs[q]));
       if (j & 1) { UN = cneg(UN); US = cneg(US); }
     }
-    Q.FT[(size_t)m * A.RP + k] = make_double4_32a(
-        df_pack(df_mul2(RE(UN), om)), df_pack(df_mul2(IM(UN), om)), two ? df_pack(df_mul2(RE(US), om)) : 0.0,
-        two ? df_pack(df_mul2(IM(US), om)) : 0.0);
+    auto put = [&](dfl v) { return df_pack(dfl{A.fscale * v.h, A.fscale * v.l}); };
+    Q.FT[(size_t)m * A.RP + k] =
+        make_double4_32a(put(RE(UN)), put(IM(UN)), two ? put(RE(US)) : 0.0, two ? put(IM(US)) : 0.0);
   }
 }
 
@@ -280,11 +281,11 @@ void launch_pack_twiddles(const double2 *tw, int logMmax, float4 *df, float2 *f3
   pack_twiddles_kernel<<<(n + 255) / 256, 256, 0, s>>>(tw, logMmax, df, f32);
 }
 
-template <int MODE>
-static void launch_ring_df_mode(const RingArgs *a, const RingDfArgs *t, int nmaps, const RingClass *cls, int ncls,
+template <int MODE, bool FINE>
+static void launch_ring_df_form(const RingArgs *a, const RingDfArgs *t, int nmaps, const RingClass *cls, int ncls,
                                 cudaStream_t s) {
   auto smem = [](const RingClass &c) { return c.global ? (size_t)16 : ((size_t)1 << c.logM) * sizeof(float4); };
-  raise_smem_cap(reinterpret_cast<const void *>(ring_df_kernel<MODE>));
+  raise_smem_cap(reinterpret_cast<const void *>(ring_df_kernel<MODE, FINE>));
   for (int c = 0; c < ncls; ++c) {
     if (cls[c].count <= 0) continue;
     const size_t sm = smem(cls[c]);
@@ -301,9 +302,16 @@ static void launch_ring_df_mode(const RingArgs *a, const RingDfArgs *t, int nmap
         q.m[i] = RingMap{x.FS, x.FT, x.map_in, x.map_out, y.d, y.w, x.w, y.gain, y.gainlam, x.ring_part, x.ctl,
                          x.gate, x.tau};
       }
-      launch_pdl(ring_df_kernel<MODE>, dim3(cls[c].count, n), kRingDfThreads, sm, s, ac, t[0], q);
+      launch_pdl(ring_df_kernel<MODE, FINE>, dim3(cls[c].count, n), kRingDfThreads, sm, s, ac, t[0], q);
     }
   }
+}
+
+template <int MODE>
+static void launch_ring_df_mode(const RingArgs *a, const RingDfArgs *t, int nmaps, const RingClass *cls, int ncls,
+                                cudaStream_t s) {
+  if (fine_steps(a[0].RP)) launch_ring_df_form<MODE, true>(a, t, nmaps, cls, ncls, s);
+  else launch_ring_df_form<MODE, false>(a, t, nmaps, cls, ncls, s);
 }
 
 void launch_ring_df(const RingArgs *a, const RingDfArgs *t, int nmaps, const RingClass *cls, int ncls,

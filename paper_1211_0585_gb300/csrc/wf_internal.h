@@ -8,7 +8,8 @@
 //              FS: synthesis side (from a_lm), FT: analysis side (to a_lm).
 //              Native FP64 stages hold doubles; the double-float stages (ring_df,
 //              legendre_df, legendre_tab, spin-2) hold each value as its (hi, lo)
-//              floats in the same 8 bytes (df_pack).
+//              floats in the same 8 bytes (df_pack), and FT without the last factor
+//              of Omega (LegArgs::fomega), which the analysis multiplies its sums by.
 //   a_lm       m-major complex doubles, index(l, m) = m (2 lmax + 1 - m) / 2 + l.
 //   maps       RING order doubles.
 #pragma once
@@ -108,6 +109,7 @@ struct RingArgs {
   const Ctl *ctl;         // RING_ITER: lambda, lsht, done
   int lsht;               // standalone modes
   double omega, tau;
+  float fscale;           // double-float records FT: the power of two in (Omega / 4, Omega / 2]
   double *gain;           // [npix] cached w / (1 + (lambda - 1) tau w) (double-float ring kernel)
   double *gainlam;        // [R] lambda the cached gains of each ring belong to (-1: none)
   const Ctl *gate;        // RING_SYNTH / RING_ANALYSIS inside a controlled iteration: skip once gate->done
@@ -131,6 +133,7 @@ struct LegArgs {
                           // (nullptr for the standalone transforms)
   int lsht, lmax, RP;
   double omega, tau;
+  double fomega;          // double-float stages: Omega / 2 over RingArgs::fscale
 };
 
 // Tables of the double-float Legendre kernel (legendre_df.cu).
@@ -288,6 +291,13 @@ void launch_posterior_norms(const double2 *a, const double2 *ta, const double2 *
 // rows of the precomputed double-float lambda table: of one m (two l each), and of all
 __host__ __device__ inline int tab_rows(int lmax, int m) { return (lmax - m + 2) / 2; }
 size_t lam_table_rows(int lmax);
+// Whether the double-float stages of a shape take the finer forms (FINE: df.cuh, fft.cuh) of their sums and products.
+// Their roundings show in short sums and short FFTs: without them the transforms' errors at Nside 8 to 32 are up to
+// 1.07 (E and B: 1.25, recurrence form: 1.2) times what they are with records and sums over lanes in double, with them
+// 0.96 to 1.01 times. From Nside 128 on folding long sums back (dot2_tidy) does more for the error (0.5 to 0.99 times).
+// Latency bounds the kernels up to Nside 64, so they cost little: Nside 16 solve 12.97 ms, 12.47 without the FFT's; a
+// T + P solve at Nside 128, bound by FP32 issue in these sums, took 68 instead of 62 ms with them.
+inline bool fine_steps(int RP) { return RP <= 128; }
 // largest dynamic shared memory of the table form's kernels
 size_t leg_tab_smem(int lmax, int RP);
 void launch_lam_table(const double *x, const double2 *rec, const int *ls64, const double2 *sv64, const int *ls_df,

@@ -89,6 +89,7 @@ struct Plan : wf_plan_s {
   wf_status alloc_tab_work();           // d_coef, d_part
   wf_status ensure_hist(int cap);
   cudaStream_t run_stream() const;
+  double record_scale() const;
   RingArgs ring_args() const;
   LegArgs leg_args() const;
   LegDfArgs legdf_args() const { return LegDfArgs{d_dfA, d_dfg, d_dfls, d_dfsv, d_tab, d_poff}; }

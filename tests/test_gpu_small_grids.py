@@ -54,3 +54,12 @@ def test_recurrence_form(kind, base):
     if kind == "iterate":
         case.update(lam=3.0, niter=3)
     assert mean_error(case, 16, lambda r: r["alm"] if kind == "iterate" else r, False) <= 1.06 * base
+
+
+@pytest.mark.parametrize("kind,lmax,nside,part,seeds,base,margin", [
+    ("analysis", 37, 16, None, 16, 5.745e-15, 1.03),       # 1.067 times with a rounding for Omega in every record
+    ("synthesis", 16, 16, None, 16, 6.347e-15, 1.03),      # 1.047 times with the products of long rings in the FFTs
+    ("pol_pair", 16, 8, 1, 16, 3.892e-15, 1.12)])          # E: 1.208 times with the shorter sums over lanes
+def test_table_form(kind, lmax, nside, part, seeds, base, margin):
+    case = dict(kind=kind, nside=nside, lmax=lmax, lsht=lmax)
+    assert mean_error(case, seeds, lambda r: r if part is None else r["alm"][part], True) <= margin * base
