@@ -93,7 +93,7 @@ BatchArgs Engine::args() const {
   a.rings = geo->d_rings;
   a.porder = geo->d_porder;
   a.first = 0;
-  a.twf = geo->d_twf; a.hsf = geo->d_hsf; a.chf = geo->d_chf; a.Bf = geo->d_Bf;
+  a.hsf = geo->d_hsf; a.chf = geo->d_chf;
   a.tw2 = tw2; a.Bf2 = Bf2;
   a.logMmax = geo->logMmax;
   a.lmax = geo->lmax; a.RP = geo->RP; a.R = geo->R; a.B = B;

@@ -28,6 +28,14 @@ __device__ __forceinline__ dfl df_unpack(double v) {
 __device__ __forceinline__ dfl df_neg(dfl a) { return {-a.h, -a.l}; }
 __device__ __forceinline__ float4 df_pair(dfl a, dfl b) { return make_float4(a.h, a.l, b.h, b.l); }
 
+// (S, C) += (rS, rC), another thread's compensated sum: error-free in S
+__device__ __forceinline__ void comp_add(float &S, float &C, float rS, float rC) {
+  const float s = S + rS;
+  const float bb = s - S;
+  C = C + rC + ((S - (s - bb)) + (rS - bb));
+  S = s;
+}
+
 // S + C of a compensated sum as a double-float
 __device__ __forceinline__ dfl df_norm(float S, float C) {
   const float s = S + C, bb = s - S;

@@ -45,12 +45,6 @@ __device__ __forceinline__ size_t alm_idx_d(int lmax, int l, int m) {
 // Sixteen compensated sums over the warp's lanes by exchanging halves: lanes 2 q and 2 q + 1 end with sum q
 __device__ __forceinline__ void warp_sums16(float (&S)[16], float (&C)[16]) {
   const int lane = threadIdx.x & 31;
-  auto add = [](float &s0, float &c0, float s1, float c1) {
-    const float s = s0 + s1;
-    const float bb = s - s0;
-    c0 = c0 + c1 + ((s0 - (s - bb)) + (s1 - bb));
-    s0 = s;
-  };
 #pragma unroll
   for (int off = 16, n = 8; n >= 1; off >>= 1, n >>= 1) {
     const bool up = (lane & off) != 0;
@@ -59,10 +53,10 @@ __device__ __forceinline__ void warp_sums16(float (&S)[16], float (&C)[16]) {
       const float oS = up ? S[j] : S[j + n], oC = up ? C[j] : C[j + n];
       S[j] = up ? S[j + n] : S[j];
       C[j] = up ? C[j + n] : C[j];
-      add(S[j], C[j], __shfl_xor_sync(0xffffffffu, oS, off), __shfl_xor_sync(0xffffffffu, oC, off));
+      comp_add(S[j], C[j], __shfl_xor_sync(0xffffffffu, oS, off), __shfl_xor_sync(0xffffffffu, oC, off));
     }
   }
-  add(S[0], C[0], __shfl_xor_sync(0xffffffffu, S[0], 1), __shfl_xor_sync(0xffffffffu, C[0], 1));
+  comp_add(S[0], C[0], __shfl_xor_sync(0xffffffffu, S[0], 1), __shfl_xor_sync(0xffffffffu, C[0], 1));
 }
 
 constexpr int kDB = 8;   // l per block of the analysis

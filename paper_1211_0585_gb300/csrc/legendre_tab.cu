@@ -43,14 +43,6 @@ constexpr int kNoStartT = 1 << 30;
 
 __device__ __forceinline__ size_t aidx_t(int lmax, int l, int m) { return (size_t)m * (2 * lmax + 1 - m) / 2 + l; }
 
-// (s0, c0) += (s1, c1), error-free in s
-__device__ __forceinline__ void comp_add(float &s0, float &c0, float s1, float c1) {
-  const float s = s0 + s1;
-  const float bb = s - s0;
-  c0 = c0 + c1 + ((s0 - (s - bb)) + (s1 - bb));
-  s0 = s;
-}
-
 // the maps of a launch: which run, and their band limits
 template <int NB, bool ITER>
 struct MapSet {

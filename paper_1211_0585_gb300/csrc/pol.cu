@@ -201,12 +201,9 @@ __device__ __forceinline__ void lane_add(float &S, float &C, float rS, float rC)
     const dfl v = df_add2<true>(df_norm(S, C), df_norm(rS, rC));
     S = v.h;
     C = v.l;
-    return;
+  } else {
+    comp_add(S, C, rS, rC);
   }
-  const float s = S + rS;
-  const float bb = s - S;
-  C = C + rC + ((S - (s - bb)) + (rS - bb));
-  S = s;
 }
 
 // Eight compensated sums over the warp: lane q ends with sum q >> 2 of its 8 (lanes 4 q .. 4 q + 3 hold sum q).

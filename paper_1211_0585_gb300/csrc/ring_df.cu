@@ -31,13 +31,8 @@ __device__ __forceinline__ float4 cneg(float4 a) { return make_float4(-a.x, -a.y
 // the compensated sum (S, C) over the warp's lanes, on every lane
 __device__ __forceinline__ void warp_sum_df(float &S, float &C) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float rS = __shfl_xor_sync(0xffffffffu, S, o), rC = __shfl_xor_sync(0xffffffffu, C, o);
-    const float s = S + rS;
-    const float bb = s - S;
-    C = C + rC + ((S - (s - bb)) + (rS - bb));
-    S = s;
-  }
+  for (int o = 16; o > 0; o >>= 1)
+    comp_add(S, C, __shfl_xor_sync(0xffffffffu, S, o), __shfl_xor_sync(0xffffffffu, C, o));
 }
 
 }  // namespace

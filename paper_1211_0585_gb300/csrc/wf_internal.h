@@ -208,7 +208,7 @@ struct BatchArgs {
   const RingDev *rings;
   const int2 *porder;        // ring pair of ring-stage CTA i: porder[first + i] = (north ring, south ring or -1)
   int first;
-  const float4 *twf, *hsf, *chf, *Bf;
+  const float4 *hsf, *chf;
   const float2 *tw2, *Bf2;   // FP32 twiddles by stage and Bluestein filter tables (hi parts)
   int logMmax;
   int lmax, RP, R, B;
