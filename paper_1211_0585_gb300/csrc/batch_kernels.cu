@@ -47,7 +47,7 @@ __device__ __forceinline__ void prefetch_l2(const void *p) {
 // CTA takes both: each record is read and written whole. (A CTA per ring read
 // every record twice and wrote it in 8-byte halves: 3.65 ms an iteration at
 // Nside 512 / 64 slots, now 2.83 with the twiddles laid out by stage, fft.cuh;
-// the load and store pipe, 77 % busy at Nside 256, bounds the long rings.) The arrays share every twiddle load, the pixel
+// the L1 / shared-memory data pipe, 71 to 74 % busy at Nside 256, bounds the long rings.) The arrays share every twiddle load, the pixel
 // pass updates them in place (the inverse transform's output order is the
 // forward transform's input order), and the G slots read their Fourier
 // coefficients as one contiguous run of G float4. Four CTAs of 256 threads per

@@ -67,8 +67,8 @@ struct MapSet {
 // more than the SM's FP32 issue slots). The sigma lanes combine by exchanging
 // halves. Bound by HBM at Nside 512 (540 us a launch at lmax 1024, 0.87 of the
 // copy rate; 595 us with one tile in flight, 643 us with groups of 8 rows, whose
-// registers leave two CTAs per SM), by FP32 issue with two maps (833 us for
-// both) and below Nside 512. 96 rows a CTA: 91 us at Nside 256 / lmax 512 and 816
+// registers leave two CTAs per SM), by latency at the two CTAs an SM that two maps'
+// registers leave (833 us for both) and by FP32 issue and HBM below Nside 512 (0.54 of the issue slots at Nside 256). 96 rows a CTA: 91 us at Nside 256 / lmax 512 and 816
 // at Nside 512 for two maps, against 97 and 855 with 64 and 98 and 968 with 32.
 template <int NB, bool ITER, bool FINE>
 __global__ void __launch_bounds__(kThreads, NB == 1 ? 3 : 2) tab_analysis_kernel(const LegArgs A, const LegDfArgs D,
